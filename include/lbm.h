@@ -223,6 +223,21 @@ long long lbm_kernels_per_step(const lbm_handle *h);
  * LBM_ERR_ARG for other values, with the previous configuration kept. */
 int lbm_set_launch(lbm_handle *h, int warps, int rows, int grid, int proj_rows);
 
+/* Advances up to `steps` (1..4) time steps per launch, in blocks of about
+ * `rows` (>= 8) rows: intermediate steps stay on chip, so a launch reads and
+ * writes the populations once.  Ensembles of 2^20 cells and more get the
+ * fastest setting at create (lbm_set_launch goes back to one step).  The
+ * steps of a call that do not fill a launch, and the steps that record a
+ * snapshot, run as shorter launches.  Results do not depend on it.
+ * LBM_ERR_ARG for steps > 1 unless every member is FP32 with nx % 4 == 0,
+ * ny >= 4, collision 0, force kind 0 or 1 and rho0 in [1e-30, 1e30], in
+ * double-buffer storage (storage 2, or 0 where the tuner chose it); the
+ * previous setting is then kept. */
+int lbm_set_steps_per_launch(lbm_handle *h, int steps, int rows);
+
+/* Steps one launch advances at most (host-only; -1 for a NULL handle). */
+int lbm_steps_per_launch(const lbm_handle *h);
+
 /* Records the moment snapshot (rho, j) of every member at the current time
  * into the 3-slot history used by the eq. (17) time derivative. */
 int lbm_record_snapshot(lbm_handle *h);

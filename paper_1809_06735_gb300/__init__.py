@@ -91,6 +91,8 @@ def load_library(path: str = LIB_PATH):
         "lbm_launch_count": ([P], ctypes.c_longlong),
         "lbm_kernels_per_step": ([P], ctypes.c_longlong),
         "lbm_set_launch": ([P, I, I, I, I], I),
+        "lbm_set_steps_per_launch": ([P, I, I], I),
+        "lbm_steps_per_launch": ([P], I),
         "lbm_tuning": ([P, P, P, P, P, P, P], I),
         "lbm_record_snapshot": ([P], I),
         "lbm_moments": ([P, I, P, P, P, P], I),
@@ -300,6 +302,16 @@ class Lattice:
         """Replace the autotuned launch configuration (see lbm_set_launch);
         proj_rows 0 keeps the projection's rows per thread."""
         self._check(self.lib.lbm_set_launch(self.h, warps, rows, grid, proj_rows))
+
+    def set_steps_per_launch(self, steps: int, rows: int = 64):
+        """Advance up to ``steps`` (1..4) time steps per launch in blocks of
+        about ``rows`` rows (see lbm_set_steps_per_launch)."""
+        self._check(self.lib.lbm_set_steps_per_launch(self.h, int(steps), int(rows)))
+
+    @property
+    def steps_per_launch(self) -> int:
+        """Time steps one launch advances at most (tuned at create)."""
+        return int(self.lib.lbm_steps_per_launch(self.h))
 
     def record_snapshot(self):
         self._check(self.lib.lbm_record_snapshot(self.h))

@@ -17,6 +17,7 @@
 
 
 using lbm::Member;
+using lbm::MultiWarp;
 using lbm::Tile;
 
 namespace {
@@ -31,7 +32,8 @@ size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 thread_local std::string g_last_error = "no error";
 
 struct Layout {
-  size_t members, tiles, status, sync;
+  size_t members, tiles, multi, status, sync;
+  size_t multi_cap;  // entries of the several-steps table
   std::vector<size_t> pop0, pop1, fx, fy, fx64, fy64, snap;
   std::vector<size_t> ft, ft64, trig, trig64, damp, damp_f, damp_ring, proj, drows, pcount;
   std::vector<size_t> nu_ring;  // variable viscosity: local viscosity per snapshot slot
@@ -162,12 +164,17 @@ Layout make_layout(const lbm_config *cfg) {
   L.members = take(sizeof(Member) * n);
   // tile table sized for the smallest tile height (1 row)
   size_t max_tiles = 0;
+  L.multi_cap = 0;
   for (int m = 0; m < n; ++m) {
     const lbm_member_cfg &c = cfg->members[m];
     if (vector_eligible(c, cfg->precision)) {
       max_tiles += (size_t)((c.nx + kTileW - 1) / kTileW) * c.ny;
+      L.multi_cap += lbm::multi_capacity(c.nx, c.ny);
     }
   }
+  // the several-steps kernel needs the two arrays of a double buffer
+  if (cfg->storage == 1) L.multi_cap = 0;
+  L.multi = take(sizeof(MultiWarp) * std::max<size_t>(L.multi_cap, 1));
   L.tiles = take(sizeof(Tile) * std::max<size_t>(max_tiles, 1));
   L.status = take(sizeof(int) * n);
   L.sync = take(4 * sizeof(unsigned));  // persistent small-grid step: count, gen, err
@@ -256,8 +263,14 @@ struct lbm_handle {
   long long ring_time[3] = {-1, -1, -1};
   lbm::DiagScratch sc{};
   lbm::LaunchCfg lc{8, 1, 0, 0, 8};
+  MultiWarp *d_multi = nullptr;
+  int multi_T = 1;      // steps per launch (1: the single-step kernel only)
+  int multi_rows = 0;   // rows of a block
+  int multi_ctas = 0;
+  bool multi_forced = false;  // some member has a force or drag
   int graph_k = 0;
   cudaGraphExec_t graph[4] = {nullptr, nullptr, nullptr, nullptr};  // by storage state
+  int graph_launches[4] = {0, 0, 0, 0};  // step launches of each (state flips)
   int persist_ctas = 0;  // > 0: one small general-kernel member, steps in one cooperative launch
   lbm::GridSync gsync{};
   float tuned_ms = 0.f;  // autotuned time of one step, ms (0: not tuned)
@@ -309,6 +322,36 @@ int build_tiles(lbm_handle *h) {
   return LBM_OK;
 }
 
+// The warp table of the several-steps kernel: blocks of `rows` rows, whole rows
+// as one group where that takes at most gmax warps.
+int build_multi(lbm_handle *h, int T, int rows, int gmax) {
+  std::vector<MultiWarp> tab;
+  for (int m = 0; m < (int)h->mcfg.size(); ++m)
+    lbm::multi_member(m, h->mcfg[m].nx, h->mcfg[m].ny, rows, gmax, &tab);
+  while (tab.size() % lbm::kMultiWarps) tab.push_back(MultiWarp{-1});
+  if (tab.size() > h->lay.multi_cap)
+    return fail(h, LBM_ERR_WORKSPACE, "several-steps table larger than its workspace");
+  CK(cudaMemcpyAsync(h->d_multi, tab.data(), sizeof(MultiWarp) * tab.size(),
+                     cudaMemcpyHostToDevice, h->stream));
+  CK(cudaStreamSynchronize(h->stream));
+  h->multi_T = T;
+  h->multi_rows = rows;
+  h->multi_ctas = (int)(tab.size() / lbm::kMultiWarps);
+  return LBM_OK;
+}
+
+// Members the several-steps kernel can advance: double-buffer storage, every
+// member on the vectorised kernel with BGK, no force that needs the whole
+// state of each step (the damping of force kind 2).
+bool multi_eligible(const lbm_handle *h) {
+  if (h->precision != 32 || h->cfg.storage == 1 || h->has_kind2 || h->has_vv ||
+      !h->scalar_members.empty())
+    return false;
+  for (const lbm_member_cfg &c : h->mcfg)  // densities whose reciprocal is a normal number
+    if (c.ny < lbm::kMultiMinNy || c.rho0 < 1e-30 || c.rho0 > 1e30) return false;
+  return true;
+}
+
 // Largest grid of the handle (batched per-member launches).
 void max_grid(const lbm_handle *h, int *nx, int *ny) {
   *nx = 1;
@@ -358,6 +401,30 @@ int launch_one_step(lbm_handle *h, cudaStream_t s, int cur) {
   return LBM_OK;
 }
 
+// k steps of every member on stream s from storage state *cur: launches of up
+// to multi_T steps, as even as k allows.  Returns the state in *cur and the
+// step launches in *n.
+int launch_steps(lbm_handle *h, cudaStream_t s, int *cur, long long k, int *n) {
+  *n = 0;
+  while (k > 0) {
+    int t = 1;
+    if (h->multi_T > 1 && *cur < 2) {
+      const long long left = (k + h->multi_T - 1) / h->multi_T;
+      t = (int)((k + left - 1) / left);
+    }
+    if (t > 1) {
+      CK(lbm::launch_multi(t, h->multi_forced, h->d_members, h->d_multi, h->multi_ctas, *cur,
+                           *cur & 1, s));
+    } else {
+      if (int rc = launch_one_step(h, s, *cur)) return rc;
+    }
+    *cur ^= 1;
+    k -= t;
+    *n += 1;
+  }
+  return LBM_OK;
+}
+
 long long kernels_per_step(const lbm_handle *h) {
   const long long ns = (long long)h->scalar_members.size();
   return (h->ntiles > 0 ? 1 : 0) + (ns + 255) / 256 + (h->has_kind2 ? 1 : 0);
@@ -371,11 +438,8 @@ void drop_graphs(lbm_handle *h) {
 int get_graph(lbm_handle *h, int cur, cudaGraphExec_t *out) {
   if (!h->graph[cur]) {
     CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-    int c = cur, rc = LBM_OK;
-    for (int i = 0; i < h->graph_k && rc == LBM_OK; ++i) {
-      rc = launch_one_step(h, h->cap_stream, c);
-      c ^= 1;
-    }
+    int c = cur;
+    const int rc = launch_steps(h, h->cap_stream, &c, h->graph_k, &h->graph_launches[cur]);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(h->cap_stream, &g);
     if (rc != LBM_OK) { if (g) cudaGraphDestroy(g); return rc; }
@@ -407,16 +471,17 @@ int run_steps(lbm_handle *h, long long k) {
       int rc = get_graph(h, h->cur, &g);
       if (rc) return rc;
       CK(cudaGraphLaunch(g, h->stream));
-      h->launches += (long long)h->graph_k * kernels_per_step(h);
+      h->launches += (long long)h->graph_launches[h->cur] * kernels_per_step(h);
+      h->cur ^= h->graph_launches[h->cur] & 1;
       k -= h->graph_k;
-      h->t += h->graph_k;  // graph_k is even: buffer parity unchanged
+      h->t += h->graph_k;
     } else {
-      int rc = launch_one_step(h, h->stream, h->cur);
-      if (rc) return rc;
-      h->launches += kernels_per_step(h);
-      h->cur ^= 1;
-      k -= 1;
-      h->t += 1;
+      const long long part = h->graph_k > 0 ? std::min<long long>(k, h->graph_k) : k;
+      int n = 0;
+      if (int rc = launch_steps(h, h->stream, &h->cur, part, &n)) return rc;
+      h->launches += n * kernels_per_step(h);
+      k -= part;
+      h->t += part;
     }
   }
   return LBM_OK;
@@ -485,7 +550,7 @@ int autotune(lbm_handle *h) {
   int dev = 0, nsm = 0;
   CK(cudaGetDevice(&dev));
   CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  struct Cand { lbm::LaunchCfg lc; int state; float ms; };
+  struct Cand { lbm::LaunchCfg lc; int state, per; float ms; };
   std::vector<int> states;
   if (h->cfg.storage == 0) states = {0, 2};
   else states = {h->cfg.storage == 1 ? 2 : 0};
@@ -494,7 +559,7 @@ int autotune(lbm_handle *h) {
     for (int wy : {4, 8})
       for (int rows : {1, 2, 4})
         for (int per : {0, 4, 8})
-          cands.push_back({{wy, rows, per * nsm, h->lc.paper_force, h->lc.proj_rows}, st, 0.f});
+          cands.push_back({{wy, rows, per * nsm, h->lc.paper_force, h->lc.proj_rows}, st, per, 0.f});
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   // 2 warm-up and `steps` timed steps of candidate i: ms per step
   auto time_candidate = [&](size_t i, int steps, float *ms) -> int {
@@ -522,16 +587,91 @@ int autotune(lbm_handle *h) {
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
   if (e != cudaSuccess)
     rc = fail(h, LBM_ERR_CUDA, std::string("autotune events: ") + cudaGetErrorString(e));
+  // several steps per launch on double-buffer storage: three steps on the
+  // tallest blocks that fill 1 .. 4 waves of two CTAs per SM (taller blocks
+  // recompute fewer rows), whole rows as groups of up to 8, 4 or 1 warps; then
+  // two and four steps on the fastest of these shapes
+  struct Multi { int T, rows, gmax; float ms; };
+  Multi multi{1, 0, 0, 1e30f};
+  if (rc == LBM_OK && multi_eligible(h)) {
+    // one warm-up launch and 2 to 6 timed ones, about 2 ms where that is enough
+    auto time_multi = [&](Multi &c) -> int {
+      if (int rc2 = build_multi(h, c.T, c.rows, c.gmax)) return rc2;
+      int st = 0, n = 0;
+      if (int rc2 = launch_steps(h, h->stream, &st, c.T, &n)) return rc2;
+      const float est = multi.ms < 1e30f ? multi.ms : 1e-8f * (float)cells;
+      const int launches = std::max(2, std::min(6, (int)(2.f / (c.T * est))));
+      CK(cudaEventRecord(e0, h->stream));
+      if (int rc2 = launch_steps(h, h->stream, &st, (long long)launches * c.T, &n)) return rc2;
+      CK(cudaEventRecord(e1, h->stream));
+      CK(cudaEventSynchronize(e1));
+      CK(cudaEventElapsedTime(&c.ms, e0, e1));
+      c.ms /= (float)(launches * c.T);
+      if (c.ms < multi.ms) multi = c;
+      return LBM_OK;
+    };
+    std::vector<Multi> tries;
+    auto faster = [](const Multi &a, const Multi &b) { return a.ms < b.ms; };
+    for (int gmax : {8, 4, 1}) {
+      int last = 0;
+      for (int w = 1; w <= 4; ++w) {
+        int lo = lbm::kMultiMinRows, hi = 256;  // CTAs fall as rows grow
+        while (lo < hi) {
+          const int mid = (lo + hi) / 2;
+          double ctas = 0.0;
+          for (const lbm_member_cfg &c : h->mcfg) ctas += lbm::multi_ctas(c.nx, c.ny, mid, gmax);
+          if (ctas <= 2.0 * w * nsm) hi = mid;
+          else lo = mid + 1;
+        }
+        if (lo != last) tries.push_back({3, lo, gmax, 0.f});
+        last = lo;
+      }
+    }
+    for (size_t k = 0; k < tries.size() && rc == LBM_OK; ++k) rc = time_multi(tries[k]);
+    std::sort(tries.begin(), tries.end(), faster);
+    const Multi top = tries[0];
+    for (int T : {2, 4}) {
+      tries.push_back({T, top.rows, top.gmax, 0.f});
+      if (rc == LBM_OK) rc = time_multi(tries.back());
+    }
+    // the two fastest again, three times each: the median decides
+    std::sort(tries.begin(), tries.end(), faster);
+    multi.ms = 1e30f;
+    Multi pick = multi;
+    for (size_t k = 0; k < 2 && rc == LBM_OK; ++k) {
+      Multi t[3] = {tries[k], tries[k], tries[k]};
+      for (int r = 0; r < 3 && rc == LBM_OK; ++r) rc = time_multi(t[r]);
+      std::sort(t, t + 3, faster);
+      if (rc == LBM_OK && t[1].ms < pick.ms) pick = t[1];
+    }
+    multi = pick;
+    h->multi_T = 1;  // the single-step shapes are timed next
+  }
+  // single-step shapes.  Where several steps per launch can be taken, first
+  // those that were ever chosen (4 warps, 0 or 4 CTAs per SM) and the others
+  // only if one of them beats it
+  if (multi.T > 1) {
+    auto common = [](const Cand &c) { return c.lc.block_warps_y == 4 && c.per <= 4; };
+    std::stable_partition(cands.begin(), cands.end(), common);
+    const size_t n = std::count_if(cands.begin(), cands.end(), common);
+    float fastest = 1e30f;
+    for (size_t i = 0; i < n && rc == LBM_OK; ++i) {
+      rc = time_candidate(i, 6, &cands[i].ms);
+      fastest = std::min(fastest, cands[i].ms);
+    }
+    if (multi.ms < fastest) cands.resize(n);
+  }
   // every candidate once (6 steps), then the three fastest again, three runs
   // of 12 steps each: the median decides (single short runs are noisy)
   for (size_t i = 0; i < cands.size() && rc == LBM_OK; ++i)
-    rc = time_candidate(i, 6, &cands[i].ms);
+    if (cands[i].ms == 0.f) rc = time_candidate(i, 6, &cands[i].ms);
   std::vector<int> order(cands.size());
   for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
   std::sort(order.begin(), order.end(), [&](int a, int b) { return cands[a].ms < cands[b].ms; });
   int best = order.empty() ? 0 : order[0];
   float best_ms = 1e30f;
-  for (size_t k = 0; k < order.size() && k < 3 && rc == LBM_OK; ++k) {
+  const bool keep_multi = multi.T > 1 && multi.ms < cands[order[0]].ms;
+  for (size_t k = 0; k < order.size() && k < 3 && rc == LBM_OK && !keep_multi; ++k) {
     float t[3];
     for (int r = 0; r < 3 && rc == LBM_OK; ++r) rc = time_candidate(order[k], 12, &t[r]);
     if (rc != LBM_OK) break;
@@ -567,6 +707,17 @@ int autotune(lbm_handle *h) {
   h->lc = cands[best].lc;
   h->cur = cands[best].state;
   h->tuned_ms = best_ms;
+  h->multi_T = 1;
+  if (keep_multi) {  // single steps (remainders) in the same storage
+    for (size_t i = 0; i < order.size(); ++i)
+      if (cands[order[i]].state == 0) {
+        h->lc = cands[order[i]].lc;
+        break;
+      }
+    h->cur = 0;
+    h->tuned_ms = multi.ms;
+    if ((rc = build_multi(h, multi.T, multi.rows, multi.gmax))) return rc;
+  }
   return build_tiles(h);
 }
 
@@ -607,6 +758,7 @@ int lbm_create(const lbm_config *cfg, void *workspace, size_t bytes, lbm_handle 
   h->graph_k = cfg->graph_steps > 0 ? (cfg->graph_steps + 1) / 2 * 2 : 0;
   h->d_members = reinterpret_cast<Member *>(ws_at(h, lay.members));
   h->d_tiles = reinterpret_cast<Tile *>(ws_at(h, lay.tiles));
+  h->d_multi = reinterpret_cast<MultiWarp *>(ws_at(h, lay.multi));
   h->sc.f = reinterpret_cast<double *>(ws_at(h, lay.scratch));
   h->sc.N = lay.Nmax;
   h->sc.partials = reinterpret_cast<double *>(ws_at(h, lay.partials));
@@ -733,6 +885,8 @@ int lbm_create(const lbm_config *cfg, void *workspace, size_t bytes, lbm_handle 
     return cleanup(fail(nullptr, LBM_ERR_CUDA, std::string("create: ") + cudaGetErrorString(e)));
   h->cur = cfg->storage == 1 ? 2 : 0;
   h->lc.paper_force = h->has_elbm ? 3 : (h->has_vv ? 2 : (h->has_kind2 ? 1 : 0));
+  for (const lbm_member_cfg &c : h->mcfg)
+    h->multi_forced |= c.alpha != 0.0 || (c.force_kind != 0 && c.F0 != 0.0);
   {
     unsigned *w = reinterpret_cast<unsigned *>(ws_at(h, lay.sync));
     h->gsync = lbm::GridSync{w, w + 1, reinterpret_cast<int *>(w + 2)};
@@ -902,9 +1056,29 @@ int lbm_set_launch(lbm_handle *h, int warps, int rows, int grid, int proj_rows) 
   drop_graphs(h);
   h->lc = lbm::LaunchCfg{warps, rows, grid, h->lc.paper_force,
                          proj_rows > 0 ? proj_rows : h->lc.proj_rows};
+  h->multi_T = 1;  // the single-step kernel in the given shape
   h->tuned_ms = 0.f;
   return build_tiles(h);
 }
+
+int lbm_set_steps_per_launch(lbm_handle *h, int steps, int rows) {
+  if (!h) return fail(nullptr, LBM_ERR_ARG, "handle is NULL");
+  if (steps < 1 || steps > lbm::kMultiMaxSteps) return fail(h, LBM_ERR_ARG, "steps must be 1..4");
+  if (rows < lbm::kMultiMinRows) return fail(h, LBM_ERR_ARG, "rows must be >= 8");
+  if (steps > 1 && (!multi_eligible(h) || h->cur >= 2))
+    return fail(h, LBM_ERR_ARG, "several steps per launch need FP32 members with nx % 4 == 0 and "
+                                "ny >= 4 in double-buffer storage, with BGK and without force kind 2");
+  if (int rc = wait_diag(h)) return rc;
+  drop_graphs(h);
+  h->tuned_ms = 0.f;
+  if (steps == 1) {
+    h->multi_T = 1;
+    return LBM_OK;
+  }
+  return build_multi(h, steps, rows, lbm::kMultiWarps);
+}
+
+int lbm_steps_per_launch(const lbm_handle *h) { return h ? h->multi_T : -1; }
 
 int lbm_tuning(const lbm_handle *h, int *storage, int *warps, int *rows, int *grid,
                float *step_ms, int *proj_rows) {

@@ -13,6 +13,7 @@
 #include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
+#include <vector>
 
 namespace lbm {
 
@@ -212,6 +213,27 @@ struct LaunchCfg {
   int proj_rows;      // rows per thread of the FP32 four-cell projection (force
                       // kind 2): a block covers 128 x 8 proj_rows cells
 };
+
+// One warp of the several-steps kernel (lbm_multi.cu): the columns [x0, xend)
+// it advances (unwrapped; 4 per lane) and stores ([out0, out1)), its block of
+// rows, and its place w among the g warps of its group (consecutive warps of
+// one CTA).  member < 0: no work.
+struct MultiWarp {
+  int member, x0, xend, out0, out1, y0, rows, g, w, pad;
+};
+constexpr int kMultiWarps = 8;     // warps per CTA
+constexpr int kMultiMaxSteps = 4;  // steps per launch at most
+constexpr int kMultiMinRows = 8;  // smallest block of rows
+constexpr int kMultiMinNy = 4;    // smallest member
+// Appends the warps of one member: blocks of about `rows` rows, whole rows as
+// one group where that takes at most gmax warps.
+void multi_member(int member, int nx, int ny, int rows, int gmax, std::vector<MultiWarp> *tab);
+double multi_ctas(int nx, int ny, int rows, int gmax);  // CTAs of it
+size_t multi_capacity(int nx, int ny);  // table entries of a member at most
+// T = 2..4 steps of every member in the table from double-buffer storage
+// `state` into the other buffer (forced: some member has a force or drag).
+cudaError_t launch_multi(int T, bool forced, const Member *d_members, const MultiWarp *tab, int ctas,
+                         int state, int flip, cudaStream_t s);
 
 // One step of every vector-kernel member (flip: tiles in reverse order).
 cudaError_t launch_step_f32_vec(const Member *d_members, const Tile *d_tiles, int ntiles,

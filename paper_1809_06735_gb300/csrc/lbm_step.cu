@@ -23,459 +23,9 @@
 // its source row, and the +-1 shift of the x-moving populations is a warp
 // shuffle with one scalar load at each warp edge (the AA odd phase does the
 // same for its shifted stores), so DRAM sees coalesced 16-byte accesses.
-#include "lbm_internal.cuh"
+#include "lbm_collide.cuh"
 
 namespace lbm {
-
-// ---------------------------------------------------------------------------
-// Collision of one cell.
-// ---------------------------------------------------------------------------
-
-// FP32 deviation form: g_l = f_l - t_l rho0.  rho = rho0 + sum g,
-// j = sum c g.  g_eq_l = t_l [drho + rho (3 c.u + 4.5 (c.u)^2 - 1.5 u.u)];
-// EDM term F_l = f_eq_l(rho, u + du) - f_eq_l(rho, u) written as
-// t_l rho [3 c.du + 4.5 c.du (2 c.u + c.du) - 1.5 du.(2u + du)], du = F/rho,
-// F = F_ext - alpha j.  Post-collision g_l - omega (g_l - g_eq_l) + F_l.
-// Local relaxation time of the variable-viscosity collisions in deviation
-// form: Pi^neq = sum c c g - drho cs^2 I - rho u u (moments as collide_f32
-// forms them, so the snapshot's viscosity is the one the step used).
-__device__ __forceinline__ float local_tau_f32(const float g[kQ], float drho, float rho, float ux,
-                                               float uy, float tau0, int coll, float Cs) {
-  const float d4 = (g[5] + g[6]) + (g[7] + g[8]);
-  const float pxx = (g[1] + g[3]) + d4 - drho * (1.0f / 3.0f) - rho * ux * ux;
-  const float pyy = (g[2] + g[4]) + d4 - drho * (1.0f / 3.0f) - rho * uy * uy;
-  const float pxy = (g[5] - g[6]) + (g[7] - g[8]) - rho * ux * uy;
-  return tau_from_stress<float>(pxx, pxy, pyy, rho, tau0, coll, Cs);
-}
-__device__ __forceinline__ void moments_f32(const float g[kQ], float rho0, float &drho,
-                                            float &rho, float &jx, float &jy, float &ir,
-                                            float &ux, float &uy) {
-  drho = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
-  jx = (g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]);
-  jy = (g[2] - g[4]) + (g[5] + g[6]) - (g[7] + g[8]);
-  rho = rho0 + drho;
-  ir = 1.0f / rho;
-  ux = jx * ir;
-  uy = jy * ir;
-}
-// FP64: Pi^neq = sum c c f - rho cs^2 I - rho u u.
-__device__ __forceinline__ double local_tau_f64(const double f[kQ], double rho, double ux,
-                                                double uy, double tau0, int coll, double Cs) {
-  double sxx = 0.0, sxy = 0.0, syy = 0.0;
-#pragma unroll
-  for (int l = 0; l < kQ; ++l) {
-    if (cx_of(l) != 0) sxx += f[l];
-    if (cx_of(l) * cy_of(l) != 0) sxy += cx_of(l) * cy_of(l) * f[l];
-    if (cy_of(l) != 0) syy += f[l];
-  }
-  return tau_from_stress<double>(sxx - rho / 3.0 - rho * ux * ux, sxy - rho * ux * uy,
-                                 syy - rho / 3.0 - rho * uy * uy, rho, tau0, coll, Cs);
-}
-__device__ __forceinline__ void moments_f64(const double f[kQ], double &rho, double &ux,
-                                            double &uy) {
-  double r = 0.0, jx = 0.0, jy = 0.0;
-#pragma unroll
-  for (int l = 0; l < kQ; ++l) {  // terms with c = 0 skipped (a product by 0 is not
-    r += f[l];                       // dropped by IEEE arithmetic: it costs an FMA)
-    if (cx_of(l) != 0) jx += cx_of(l) * f[l];
-    if (cy_of(l) != 0) jy += cy_of(l) * f[l];
-  }
-  rho = r;
-  const double ir = 1.0 / r;
-  ux = jx * ir;
-  uy = jy * ir;
-}
-
-// ---------------------------------------------------------------------------
-// Entropic LBM (collision 3): the equilibrium minimising H = sum f ln(f/t),
-// the non-trivial root alpha of H(f + alpha Delta) = H(f), Delta = f_eq - f,
-// f' = f + alpha Delta / (2 tau0) + F_l (EDM on the same equilibrium).
-// ---------------------------------------------------------------------------
-
-// phi(z) = (1 + z) ln(1 + z) - z: series where the terms cancel.
-// ln(1 + z) for the FP32 entropic collision, whose arguments are mostly
-// small (relative populations' departures): its Taylor series in Horner
-// form where |z| < 1/8 (the terms after z^9 / 9 are below 1e-10 of |z|,
-// under the FP32 rounding), the library function elsewhere.  FP64 keeps the
-// library functions.
-__device__ __forceinline__ float ln1p_series(float z) {
-  float p = 1.0f / 9.0f;
-  p = fmaf(-z, p, 1.0f / 8.0f);
-  p = fmaf(-z, p, 1.0f / 7.0f);
-  p = fmaf(-z, p, 1.0f / 6.0f);
-  p = fmaf(-z, p, 1.0f / 5.0f);
-  p = fmaf(-z, p, 1.0f / 4.0f);
-  p = fmaf(-z, p, 1.0f / 3.0f);
-  p = fmaf(-z, p, 1.0f / 2.0f);
-  p = fmaf(-z, p, 1.0f);
-  return z * p;
-}
-template <typename T>
-__device__ __forceinline__ T ln1p_e(T z) {
-  if constexpr (sizeof(T) == 4)
-    return fabsf(z) < 0.125f ? ln1p_series(z) : log1pf(z);
-  else
-    return log1p(z);
-}
-
-// a / b for the entropic collision: FP32 with the fast division intrinsic
-// (at most 2 ulp; every denominator here is a population, a density or a
-// sum of order one), FP64 exact.
-template <typename T>
-__device__ __forceinline__ T div_e(T a, T b) {
-  if constexpr (sizeof(T) == 4)
-    return __fdividef(a, b);
-  else
-    return a / b;
-}
-
-template <typename T>
-__device__ __forceinline__ T phi_entropy(T z) {
-  const T lim = sizeof(T) == 4 ? T(0.1) : T(0.1);
-  if (fabs(z) < lim) {
-    const int K = sizeof(T) == 4 ? 10 : 24;
-    T s = T(0), p = z * z;
-#pragma unroll
-    for (int k = 2; k < K; ++k) {
-      s += ((k & 1) ? -p : p) * T(1.0 / (k * (k - 1)));
-      p *= z;
-    }
-    return s;
-  }
-  return (T(1) + z) * ln1p_e<T>(z) - z;
-}
-
-// g(a) = sum f phi(a y) - a S2, y = Delta / f, S2 = sum Delta ln(1 + y);
-// *scale (if given) receives the magnitude of the terms, the size of g's
-// rounding noise.
-template <typename T>
-__device__ __forceinline__ T entropy_gap(const T f[kQ], const T y[kQ], T S2, T a,
-                                         T *scale = nullptr) {
-  T s = T(0);
-#pragma unroll
-  for (int l = 0; l < kQ; ++l) s += f[l] * phi_entropy<T>(a * y[l]);
-  if (scale) *scale = s + a * fabs(S2);
-  return s - a * S2;
-}
-
-// The root alpha > 1 (alpha = 2 at equilibrium, for non-positive populations
-// or without a root below min(a_max, 64)).  FP64: bisection to 1e-15 (the
-// oracle's procedure); FP32: the third-order series of the root in the
-// populations' relative departures y when every |y| < 0.02 (error below
-// 1e-7), otherwise Newton from that series, g'(a) = sum Delta ln(1 + a y) -
-// S2, kept inside a bisection bracket, until |g| is at the level of its
-// rounding (1e-6 of the terms; then one last Newton step if it stays in the
-// bracket) or a step below 1e-3 a (error of order 1e-6 a after it).
-template <typename T>
-__device__ T elbm_alpha(const T f[kQ], const T d[kQ]) {
-  T y[kQ], ymax = T(0), S2 = T(0);
-#pragma unroll
-  for (int l = 0; l < kQ; ++l) {
-    if (!(f[l] > T(0))) return T(2);
-    y[l] = div_e<T>(d[l], f[l]);
-    ymax = fmax(ymax, fabs(y[l]));
-  }
-  if (ymax < (sizeof(T) == 4 ? T(1e-7) : T(1e-12))) return T(2);
-  // the bracket (1, a_max): f + a Delta stays positive below a_max
-  auto upper = [&]() {
-    T amax = T(64);
-#pragma unroll
-    for (int l = 0; l < kQ; ++l)
-      if (y[l] < T(0)) amax = fmin(amax, div_e<T>(-T(1), y[l]));
-    return amax * (sizeof(T) == 4 ? T(1 - 1e-6) : T(1 - 1e-12));
-  };
-  T lo = T(1), hi;
-  if constexpr (sizeof(T) == 8) {
-    hi = upper();
-#pragma unroll
-    for (int l = 0; l < kQ; ++l) S2 += d[l] * ln1p_e<T>(y[l]);
-    if (entropy_gap<T>(f, y, S2, hi) < T(0)) return T(2);
-    for (int it = 0; it < 200 && hi - lo > 1e-15 * hi; ++it) {
-      const T mid = T(0.5) * (lo + hi);
-      if (entropy_gap<T>(f, y, S2, mid) < T(0))
-        lo = mid;
-      else
-        hi = mid;
-    }
-    return T(0.5) * (lo + hi);
-  } else {
-    // The root as a series in y = Delta / f about the BGK value a = 2: with
-    // T_k = sum_l f_l y_l^k (of order y^k), the entropy condition g(a) / a
-    // = sum_{k>=2} (-1)^k T_k (a^(k-1) - k) / (k (k - 1)) = 0 solved order
-    // by order in y gives a = 2 + c1 + c2 + c3 + O(y^4),
-    //   c1 = u / 3, c2 = 4 u^2 / 9 - 2 q4 / 3,
-    //   c3 = 11 q5 / 10 - 14 u q4 / 9 + 17 u^3 / 27,
-    // u = T3 / T2, q4 = T4 / T2, q5 = T5 / T2.  Against the root of the
-    // entropy condition to 40 digits its error is below 1e-7 (under the FP32
-    // rounding of a) while max |y| < 0.02: the series is then the root.
-    // Otherwise it starts Newton's iteration on g.
-    T T2 = T(0), T3 = T(0), T4 = T(0), T5 = T(0);
-#pragma unroll
-    for (int l = 0; l < kQ; ++l) {  // f y^k = Delta y^(k-1)
-      const T y2 = y[l] * y[l], dy2 = d[l] * y2;
-      T2 = fma(d[l], y[l], T2);
-      T3 = fma(d[l], y2, T3);
-      T4 = fma(dy2, y[l], T4);
-      T5 = fma(dy2, y2, T5);
-    }
-    const T r2 = div_e<T>(T(1), T2), u = T3 * r2, q4 = T4 * r2, q5 = T5 * r2;
-    T a = T(2) + (u * T(1.0 / 3.0) + (T(4.0 / 9.0) * u * u - T(2.0 / 3.0) * q4 +
-                                      T(1.1) * q5 - T(14.0 / 9.0) * u * q4 +
-                                      T(17.0 / 27.0) * u * u * u));
-    if (ymax < T(0.02)) return a;
-    hi = upper();
-#pragma unroll
-    for (int l = 0; l < kQ; ++l) S2 += d[l] * ln1p_e<T>(y[l]);
-    if (!(a > lo && a < hi)) a = fmin(T(2), T(0.5) * (lo + hi));
-    bool bracketed = false;
-    for (int it = 0; it < 30; ++it) {
-      // g(a) and g'(a) = sum Delta ln(1 + a y) - S2 share ln(1 + a y): one
-      // log1p per population (phi as entropy_gap evaluates it)
-      T s = T(0), dg = -S2;
-#pragma unroll
-      for (int l = 0; l < kQ; ++l) {
-        const T z = a * y[l], lz = ln1p_e<T>(z);
-        T ph;
-        if (fabs(z) < T(0.1)) {
-          // phi(z) = sum_{k>=2} (-1)^k z^k / (k (k - 1)), terms to z^9, in
-          // Horner form
-          T p = T(1.0 / 72.0);
-#pragma unroll
-          for (int k = 8; k >= 2; --k) p = fma(-z, p, T(1.0 / (k * (k - 1))));
-          ph = z * z * p;
-        } else {
-          ph = (T(1) + z) * lz - z;
-        }
-        s += f[l] * ph;
-        dg += d[l] * lz;
-      }
-      const T scale = s + a * fabs(S2);
-      const T g = s - a * S2;
-      const bool conv = fabs(g) <= T(1e-6) * scale;
-      if (g < T(0))
-        lo = a;
-      else
-        hi = a;
-      T an = a - div_e<T>(g, dg);
-      const bool inside = an > lo && an < hi;
-      if (conv) return inside ? an : a;
-      // Newton on the convex g converges quadratically: a step below 1e-3 a
-      // leaves an error of order 1e-6 a, the FP32 rounding level of the root
-      if (inside && fabs(an - a) < T(1e-3) * a) return an;
-      if (!bracketed) {  // no root below the positivity limit: the BGK value
-        bracketed = true;
-        if (entropy_gap<T>(f, y, S2, hi) < T(0)) return T(2);
-      }
-      if (!inside) an = T(0.5) * (lo + hi);  // left the bracket: bisect
-      const bool done = fabs(an - a) < T(1e-6) * a;
-      a = an;
-      if (done) break;
-    }
-    return a;
-  }
-}
-
-// ln of the entropic equilibrium's velocity factor, per population (FP64):
-// ln P_l(u) = sum_a [ln(2 - s_a) + c_la ln((2 u_a + s_a) / (1 - u_a))],
-// s_a = sqrt(1 + 3 u_a^2), each logarithm as log1p of a cancellation-free
-// argument (s - 1 = 3 u^2 / (1 + s)).
-template <typename T>
-__device__ __forceinline__ void entropic_logp(T ux, T uy, T lp[kQ]) {
-  const T sx = sqrt(T(1) + T(3) * ux * ux), sy = sqrt(T(1) + T(3) * uy * uy);
-  const T qx = div_e<T>(T(3) * ux * ux, T(1) + sx), qy = div_e<T>(T(3) * uy * uy, T(1) + sy);
-  const T a0x = ln1p_e<T>(-qx), a0y = ln1p_e<T>(-qy);
-  const T a1x = ln1p_e<T>(div_e<T>(T(3) * ux + qx, T(1) - ux));
-  const T a1y = ln1p_e<T>(div_e<T>(T(3) * uy + qy, T(1) - uy));
-#pragma unroll
-  for (int l = 0; l < kQ; ++l)
-    lp[l] = a0x + a0y + (T)cx_of(l) * a1x + (T)cy_of(l) * a1y;
-}
-
-// P_l(u) - 1 for FP32 from the product form of the same factor,
-// P_l = prod_a (2 - s_a) ((2 u_a + s_a) / (1 - u_a))^(c_la): with
-// q = s - 1 = 3 u^2 / (1 + s), the factor of an axis is 1 + Z_c for
-// c = 0, +1, -1: Z_0 = -q, Z_(+1) = b - q - q b with b = (3 u + q) / (1 - u),
-// Z_(-1) = b' - q - q b' with b' = -(3 u + q) / (1 + 2 u + q), and
-// P - 1 = X + Y + X Y: no logarithm or exponential, no cancellation.
-__device__ __forceinline__ void entropic_em_f32(float ux, float uy, float em[kQ]) {
-  float X[3], Y[3];  // indexed by c + 1
-  auto axis = [](float u, float (&Z)[3]) {
-    const float s = sqrtf(1.0f + 3.0f * u * u);
-    const float q = __fdividef(3.0f * u * u, 1.0f + s);
-    const float n = 3.0f * u + q;
-    const float b = __fdividef(n, 1.0f - u), bm = -__fdividef(n, 1.0f + 2.0f * u + q);
-    Z[0] = fmaf(-q, bm, bm - q);
-    Z[1] = -q;
-    Z[2] = fmaf(-q, b, b - q);
-  };
-  axis(ux, X);
-  axis(uy, Y);
-#pragma unroll
-  for (int l = 0; l < kQ; ++l) {
-    const float x = X[cx_of(l) + 1], y = Y[cy_of(l) + 1];
-    em[l] = fmaf(x, y, x + y);
-  }
-}
-
-// One ELBM collision in storage form (FP32: deviations g = f - t rho0, FP64:
-// f); returns alpha.
-template <typename T>
-__device__ T collide_elbm(T v[kQ], T rho0, T tau0, T Fex, T Fey, T alpha_drag) {
-  T rho, jx, jy, drho, ux, uy;
-  if constexpr (sizeof(T) == 4) {
-    float ir;
-    moments_f32(v, rho0, drho, rho, jx, jy, ir, ux, uy);
-  } else {
-    rho = T(0);
-    jx = T(0);
-    jy = T(0);
-#pragma unroll
-    for (int l = 0; l < kQ; ++l) {
-      rho += v[l];
-      if (cx_of(l) != 0) jx += cx_of(l) * v[l];
-      if (cy_of(l) != 0) jy += cy_of(l) * v[l];
-    }
-    drho = T(0);
-    ux = jx / rho;
-    uy = jy / rho;
-  }
-  const T Fx = Fex - alpha_drag * jx, Fy = Fey - alpha_drag * jy;
-  // without force the shifted velocity is u itself and the EDM term is
-  // exactly zero: its second equilibrium is skipped
-  const bool forced = Fx != T(0) || Fy != T(0);
-  T f[kQ], d[kQ], Fl[kQ];
-  if constexpr (sizeof(T) == 4) {
-    float em[kQ], ems[kQ];  // P_l - 1 at u and at the shifted velocity
-    entropic_em_f32(ux, uy, em);
-    if (forced) entropic_em_f32(ux + div_e<T>(Fx, rho), uy + div_e<T>(Fy, rho), ems);
-#pragma unroll
-    for (int l = 0; l < kQ; ++l) {
-      const float t = w_of(l);
-      f[l] = fmaf(t, rho0, v[l]);
-      // f_eq - f = t rho (1 + em) - t rho0 - v = t (drho + rho em) - v
-      d[l] = fmaf(t, fmaf(rho, em[l], drho), -v[l]);
-      Fl[l] = forced ? t * rho * (ems[l] - em[l]) : 0.0f;
-    }
-  } else {
-    T lp[kQ], lps[kQ];
-    entropic_logp<T>(ux, uy, lp);
-    if (forced) entropic_logp<T>(ux + div_e<T>(Fx, rho), uy + div_e<T>(Fy, rho), lps);
-#pragma unroll
-    for (int l = 0; l < kQ; ++l) {
-      const T t = (T)w_of(l);
-      const T em = expm1(lp[l]);  // P_l - 1
-      f[l] = v[l];
-      d[l] = t * rho * (T(1) + em) - v[l];
-      Fl[l] = forced ? t * rho * (T(1) + em) * expm1(lps[l] - lp[l]) : T(0);
-    }
-  }
-  const T a = elbm_alpha<T>(f, d);
-  const T ab = div_e<T>(a, T(2) * tau0);
-  if (forced) {
-#pragma unroll
-    for (int l = 0; l < kQ; ++l) v[l] = v[l] + ab * d[l] + Fl[l];
-  } else {
-#pragma unroll
-    for (int l = 0; l < kQ; ++l) v[l] = v[l] + ab * d[l];
-  }
-  return a;
-}
-
-// Relaxation time 2 tau0 / alpha of the ELBM state v (storage form).
-template <typename T>
-__device__ T elbm_tau(const T v[kQ], T rho0, T tau0) {
-  T w[kQ];
-#pragma unroll
-  for (int l = 0; l < kQ; ++l) w[l] = v[l];
-  const T a = collide_elbm<T>(w, rho0, tau0, T(0), T(0), T(0));
-  return T(2) * tau0 / a;
-}
-
-// With VV (variable viscosity, collision != 0) omega = 1 / local_tau_f32.
-template <bool VV = false>
-__device__ __forceinline__ void collide_f32(float g[kQ], float rho0, float om, float Fex,
-                                            float Fey, float alpha, int coll = 0,
-                                            float tau0 = 0.f, float Cs = 0.f) {
-  float drho, rho, jx, jy, ir, ux, uy;
-  moments_f32(g, rho0, drho, rho, jx, jy, ir, ux, uy);
-  if constexpr (VV) {
-    if (coll != 0) om = 1.0f / local_tau_f32(g, drho, rho, ux, uy, tau0, coll, Cs);
-  }
-  const float Fx = Fex - alpha * jx, Fy = Fey - alpha * jy;
-  const float dux = Fx * ir, duy = Fy * ir;
-  const float usq = ux * ux + uy * uy;
-  const float dsq = dux * (2.0f * ux + dux) + duy * (2.0f * uy + duy);
-  const float base_eq = drho - 1.5f * rho * usq;  // t-scaled later
-  const float base_F = -1.5f * rho * dsq;
-#pragma unroll
-  for (int l = 0; l < kQ; ++l) {
-    const float t = (float)w_of(l);
-    const float cu = (float)cx_of(l) * ux + (float)cy_of(l) * uy;
-    const float cd = (float)cx_of(l) * dux + (float)cy_of(l) * duy;
-    const float geq = t * (base_eq + rho * cu * (3.0f + 4.5f * cu));
-    const float Fl = t * (base_F + rho * cd * (3.0f + 4.5f * (2.0f * cu + cd)));
-    g[l] = g[l] - om * (g[l] - geq) + Fl;
-  }
-}
-
-// FP64 plain form on the full populations f_l; coll != 0: omega from the
-// local relaxation time (Pi^neq = sum c c f - rho cs^2 I - rho u u).
-// The populations go in opposite pairs (l, opp(l)), c_opp = -c_l: the
-// equilibrium and the exact-difference term split into a part even in c
-// (the same for both) and an odd part (opposite signs), each formed once:
-//   feq = t rho [1 - 1.5 |u|^2 + 4.5 (c.u)^2] +- 3 t rho |c.u|,
-//   F_l = t rho [9 (c.u)(c.du) + 4.5 (c.du)^2 - 1.5 (2 u.du + |du|^2)] +- 3 t rho |c.du|,
-// (du = F / rho), which halves the FP64 work (FP64 is this part's slow pipe).
-// The relaxed sums om feq + F are formed before the common factor t rho:
-//   e = t rho [om (base + 4.5 (c.u)^2) + (c.du) (4.5 c.du + 9 c.u) + mdsq],
-//   o = 3 t rho (om c.u + c.du),  mdsq = -1.5 (2 u.du + |du|^2),
-// 13 FP64 operations per pair.
-__device__ __forceinline__ void collide_pair_f64(double &fp, double &fm, double cu, double cd,
-                                                 double trho, double trho3, double base,
-                                                 double mdsq, double om, double keep) {
-  const double e = trho * fma(om, fma(4.5 * cu, cu, base), fma(cd, fma(4.5, cd, 9.0 * cu), mdsq));
-  const double o = trho3 * fma(om, cu, cd);
-  fp = fma(keep, fp, e + o);
-  fm = fma(keep, fm, e - o);
-}
-
-__device__ __forceinline__ void collide_f64(double f[kQ], double om, double Fex, double Fey,
-                                            double alpha, int coll = 0, double tau0 = 0.0,
-                                            double Cs = 0.0) {
-  const double rho = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])) + f[8];
-  const double jx = (f[1] + f[5] + f[8]) - (f[3] + f[6] + f[7]);
-  const double jy = (f[2] + f[5] + f[6]) - (f[4] + f[7] + f[8]);
-  const double ir = 1.0 / rho;
-  const double ux = jx * ir, uy = jy * ir;
-  if (coll != 0) om = 1.0 / local_tau_f64(f, rho, ux, uy, tau0, coll, Cs);
-  const double Fx = Fex - alpha * jx, Fy = Fey - alpha * jy;
-  const double dux = Fx * ir, duy = Fy * ir;
-  const double usq = ux * ux + uy * uy;
-  const double dsq = dux * (2.0 * ux + dux) + duy * (2.0 * uy + duy);
-  const double base = 1.0 - 1.5 * usq, keep = 1.0 - om, mdsq = -1.5 * dsq;
-  const double r0 = (4.0 / 9.0) * rho, r1 = (1.0 / 9.0) * rho, r2 = (1.0 / 36.0) * rho;
-  const double r13 = (1.0 / 3.0) * rho, r23 = (1.0 / 12.0) * rho;  // 3 t rho
-  // rest population: no odd part
-  f[0] = fma(keep, f[0], r0 * fma(om, base, mdsq));
-  collide_pair_f64(f[1], f[3], ux, dux, r1, r13, base, mdsq, om, keep);
-  collide_pair_f64(f[2], f[4], uy, duy, r1, r13, base, mdsq, om, keep);
-  collide_pair_f64(f[5], f[7], ux + uy, dux + duy, r2, r23, base, mdsq, om, keep);
-  collide_pair_f64(f[6], f[8], uy - ux, duy - dux, r2, r23, base, mdsq, om, keep);
-}
-
-// Compensated FP32 sum of FP32 values as the unevaluated pair (s, c): the
-// FP64 sum is (double)s + (double)c (the csum value) and differences of
-// nearby sums can be formed in FP32 as (s - s') + (c - c').
-__device__ __forceinline__ void csum_pair(const float *v, const int *sign, int n, float &s,
-                                          float &c) {
-  s = sign[0] * v[0];
-  c = 0.f;
-  for (int k = 1; k < n; ++k) {
-    float e;
-    two_sum(s, sign[k] * v[k], s, e);
-    c += e;
-  }
-}
 
 // ---------------------------------------------------------------------------
 // Hot kernel: batched FP32 stream-collide, 4 cells per lane, nx % 4 == 0.
