@@ -835,6 +835,15 @@ int lbm_create(const lbm_config *cfg, void *workspace, size_t bytes, lbm_handle 
       h->has_kind2 = true;
       if (h->precision != 32 || c.nx % 4 != 0) h->proj_quad = false;
     }
+    if (h->precision == 64 && c.collision == 0) {  // see collide_fixed
+      lbm::FixedBgk &B = M.fixed;
+      B.k = std::ilogb(c.rho0) + 2;
+      B.om = std::llrint(std::ldexp(M.omega, 62));
+      B.ok = B.k > -900 && B.k < 900 && std::fabs(c.alpha) < 0.25 && M.omega < 2.0 - 1e-9;
+      B.om9 = (long long)(((unsigned __int128)B.om * 8 + 4) / 9);
+      B.alpha = B.ok ? std::llrint(std::ldexp(c.alpha, 64)) : 0;
+      B.forced = c.force_kind != 0 || c.alpha != 0.0;
+    }
     h->hm.push_back(M);
     // Kolmogorov tables: F_ext,x(y) = F0 sin(2 pi kf y / ny), F_ext,y(x) likewise.
     std::vector<double> fx(c.ny, 0.0), fy(c.nx, 0.0);

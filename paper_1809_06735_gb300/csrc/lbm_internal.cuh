@@ -32,6 +32,15 @@ __host__ __device__ constexpr int opposite(int l) {
   return l == 0 ? 0 : (l <= 4 ? ((l + 1) % 4) + 1 : ((l - 5 + 2) % 4) + 5);
 }
 
+// Constants of the fixed-point form of the FP64 collision (collide_fixed):
+// k = exponent of rho0 plus two, so that rho0 lies in [1/4, 1/2) 2^k.
+struct FixedBgk {
+  int k, ok;           // ok: the member can take it (BGK, moderate parameters)
+  long long om, om9;   // omega 2^62, omega / 9 2^65
+  long long alpha;     // drag 2^64
+  int forced, pad;     // forced: a force or drag
+};
+
 // Per-member parameters, uploaded once into the workspace.
 struct Member {
   int nx, ny, pitch;     // grid and row pitch (elements)
@@ -71,6 +80,7 @@ struct Member {
   double Cs;
   void *nu_ring;         // local viscosity at each snapshot slot [3][N]
                          // (storage precision), collision != 0
+  FixedBgk fixed;        // FP64 storage
 };
 
 // Local relaxation time of a cell from its non-equilibrium stress

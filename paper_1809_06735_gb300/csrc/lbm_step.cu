@@ -360,15 +360,22 @@ __device__ __forceinline__ void step_cell(const Member &M, int state, int x, int
       rec[(size_t)l * N + (size_t)y * M.nx + x] = v;
     }
   }
-  if (M.collision == 3) {
-    if constexpr (sizeof(T) == 4)
-      collide_elbm<float>(f, M.rho0_f, M.tau_f, fx, fy, M.alpha_f);
-    else
-      collide_elbm<double>(f, 0.0, M.tau, fx, fy, M.alpha);
-  } else if constexpr (sizeof(T) == 4) {
-    collide_f32<true>(f, M.rho0_f, M.omega_f, fx, fy, M.alpha_f, M.collision, M.tau_f, M.Cs_f);
+  if constexpr (sizeof(T) == 8) {
+    if (!M.fixed.ok || !collide_fixed(f, M.fixed, fx, fy)) {
+      double g[kQ];  // read again: the fixed-point form keeps no copy
+#pragma unroll
+      for (int l = 0; l < kQ; ++l) {
+        const double *a = reinterpret_cast<const double *>(src) + pub_index(M, state, l, x, y);
+        g[l] = L2ONLY ? __ldcg(a) : *a;
+      }
+      collide_f64_call(g, M, fx, fy);
+#pragma unroll
+      for (int l = 0; l < kQ; ++l) f[l] = g[l];
+    }
+  } else if (M.collision == 3) {
+    collide_elbm<float>(f, M.rho0_f, M.tau_f, fx, fy, M.alpha_f);
   } else {
-    collide_f64(f, M.omega, fx, fy, M.alpha, M.collision, M.tau, M.Cs);
+    collide_f32<true>(f, M.rho0_f, M.omega_f, fx, fy, M.alpha_f, M.collision, M.tau_f, M.Cs_f);
   }
 #pragma unroll
   for (int l = 0; l < kQ; ++l) {
@@ -385,8 +392,12 @@ __device__ __forceinline__ void step_cell(const Member &M, int state, int x, int
   }
 }
 
-template <typename T>
-__global__ void k_step_scalar(const Member *__restrict__ members, int member, int state,
+// NT threads per CTA, at least MB CTAs per SM: FP64 grids from 2^17 cells up
+// take 3 x 256 threads (80 registers; 512^2 unforced 12.3 us against 13.7
+// with 116), smaller ones as many registers as the compiler likes (256^2:
+// 5.95 against 6.20 us).
+template <typename T, int NT, int MB>
+__global__ void __launch_bounds__(NT, MB) k_step_scalar(const Member *__restrict__ members, int member, int state,
                               double *rec) {
   const Member &M = members[member];
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -459,8 +470,8 @@ __global__ void __launch_bounds__(kPersistThreads)
 // CTAs return at once), so a step of many general-kernel members (the
 // entropic collision, FP64 ensembles, nx % 4 != 0) fills the GPU without a
 // partial wave per member.
-template <typename T>
-__global__ void k_step_scalar_multi(const Member *__restrict__ members, InitList list,
+template <typename T, int NT, int MB>
+__global__ void __launch_bounds__(NT, MB) k_step_scalar_multi(const Member *__restrict__ members, InitList list,
                                     int state) {
   const Member &M = members[list.m[blockIdx.z]];
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -546,9 +557,11 @@ cudaError_t launch_step_scalar_batch(int precision, const Member *d_members, con
     dim3 g = grid2d(nx_max, ny_max, b);
     g.z = list.n;
     if (precision == 32)
-      k_step_scalar_multi<float><<<g, b, 0, s>>>(d_members, list, state);
+      k_step_scalar_multi<float, 256, 1><<<g, b, 0, s>>>(d_members, list, state);
+    else if (b.x == 32)
+      k_step_scalar_multi<double, 64, 1><<<g, b, 0, s>>>(d_members, list, state);
     else
-      k_step_scalar_multi<double><<<g, b, 0, s>>>(d_members, list, state);
+      k_step_scalar_multi<double, 256, 3><<<g, b, 0, s>>>(d_members, list, state);
   }
   return cudaGetLastError();
 }
@@ -559,11 +572,14 @@ cudaError_t launch_step_scalar(int precision, const Member *d_members, int membe
   // their FP64 arithmetic (slow on this part) spreads evenly over the SMs
   // (256^2 FP64: 16.9 against 18.2 us per step with 256-thread CTAs in 1.7
   // waves; no difference from 384^2 up)
-  const dim3 b = (long long)nx * ny < (1LL << 17) ? dim3(32, 2) : dim3(64, 4);
+  const bool small = (long long)nx * ny < (1LL << 17);
+  const dim3 b = small ? dim3(32, 2) : dim3(64, 4), g = grid2d(nx, ny, b);
   if (precision == 32)
-    k_step_scalar<float><<<grid2d(nx, ny, b), b, 0, s>>>(d_members, member, state, rec);
+    k_step_scalar<float, 256, 1><<<g, b, 0, s>>>(d_members, member, state, rec);
+  else if (small)
+    k_step_scalar<double, 64, 1><<<g, b, 0, s>>>(d_members, member, state, rec);
   else
-    k_step_scalar<double><<<grid2d(nx, ny, b), b, 0, s>>>(d_members, member, state, rec);
+    k_step_scalar<double, 256, 3><<<g, b, 0, s>>>(d_members, member, state, rec);
   return cudaGetLastError();
 }
 
