@@ -209,7 +209,7 @@ Layout make_layout(const lbm_config *cfg) {
   L.scratch_fields = lbm::kDiagFields;
   size_t pad = 0;  // the 12 prefix tables carry one extra row and column
   for (int m = 0; m < n; ++m)
-    pad = std::max(pad, (size_t)cfg->members[m].nx + cfg->members[m].ny + 1);
+    pad = std::max(pad, (size_t)cfg->members[m].nx + 7 * (size_t)cfg->members[m].ny + 7);
   // slot 0 doubles as general staging (three snapshots, adjoint fields)
   L.slot_doubles = std::max(lbm::diag_slot_doubles(L.Nmax, pad),
                             ((size_t)L.scratch_fields * L.Nmax + 31) / 32 * 32);
@@ -841,6 +841,7 @@ int lbm_create(const lbm_config *cfg, void *workspace, size_t bytes, lbm_handle 
       B.om = std::llrint(std::ldexp(M.omega, 62));
       B.ok = B.k > -900 && B.k < 900 && std::fabs(c.alpha) < 0.25 && M.omega < 2.0 - 1e-9;
       B.om9 = (long long)(((unsigned __int128)B.om * 8 + 4) / 9);
+      B.om9h = (long long)(((unsigned __int128)B.om * 4 + 4) / 9);
       B.alpha = B.ok ? std::llrint(std::ldexp(c.alpha, 64)) : 0;
       B.forced = c.force_kind != 0 || c.alpha != 0.0;
     }
@@ -1327,6 +1328,7 @@ int balance_members(lbm_handle *h, const int *members, int nm, const int *L, int
     CK(cudaMemcpyAsync(orig_dev, origins, 8 * total_boxes, cudaMemcpyHostToDevice, s));
   // one job per member with at least one fitting size; batches of up to
   // sc.slots jobs, each batch one set of ten launches
+  const int batch_jobs = std::min(nm, h->sc.slots);
   std::vector<lbm::DiagJob> jobs;
   for (int i = 0; i < nm; ++i) {
     if (where[i].empty()) continue;
@@ -1354,8 +1356,9 @@ int balance_members(lbm_handle *h, const int *members, int nm, const int *L, int
     J.meta = meta_dev + (size_t)i * kMaxL * 8;
     J.nL = (int)where[i].size();
     J.max_boxes = maxb[i];
-    J.qblocks = lbm::diag_query_blocks(maxb[i], origins != nullptr,
-                                       std::min(nm, h->sc.slots));
+    J.qblocks = lbm::diag_query_blocks(hm.nx, hm.ny, maxb[i], origins != nullptr, batch_jobs);
+    J.qwhole = lbm::diag_whole_blocks(hm.nx * hm.ny, batch_jobs);
+    for (int q : where[i]) J.any_whole |= !origins && lbm::diag_whole_box(L[q], hm.nx, hm.ny);
     J.force_kind = hm.force_kind;
     if (hm.collision != 0) {  // local viscosity recorded with the snapshot at n
       const size_t N = (size_t)hm.nx * hm.ny;
@@ -1380,7 +1383,7 @@ int balance_members(lbm_handle *h, const int *members, int nm, const int *L, int
       const int G = (int)std::min(jobs.size() - j0, (size_t)h->sc.slots);
       CK(lbm::diag_balance(jobs.data() + j0, jobs_dev + j0, G, h->diag_precision,
                            h->precision == 32, orig_dev, stats_dev, per_box_out,
-                           dist ? &dd : nullptr, s));
+                           dist ? &dd : nullptr, batch_jobs, s));
       h->launches += 10;  // 4 term passes, scales, strip sums, table builder, constants, query, statistics
     }
   }

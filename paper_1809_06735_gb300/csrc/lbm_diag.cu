@@ -96,6 +96,23 @@ __host__ __device__ inline size_t sat_stride(int nx, int ny) {
   return (size_t)(nx + 1) * (size_t)(ny + 1);
 }
 
+// For every periodic origin at once (no origin list) the tables are planar
+// instead: P_f(x, y) at f planar_stride + y planar_pitch + 3 + x, so that
+// neighbouring origins read neighbouring words, and the four prefixes that a
+// lane of the table builder holds (x = 4 i + 1 on) start on a 32-byte boundary.
+__host__ __device__ inline size_t planar_pitch(int nx) { return ((size_t)nx + 7) / 4 * 4; }
+__host__ __device__ inline size_t planar_stride(int nx, int ny) {
+  return planar_pitch(nx) * ((size_t)ny + 1);
+}
+
+// Sizes of nearly the whole grid in both directions: their boxes are almost
+// equal, so their standard deviation is what the sums' rounding leaves of a
+// difference of two equal numbers.  k_query takes them for every origin too,
+// whose order of summation that value then stays that of an origin list.
+__host__ __device__ inline bool whole_grid_box(int L, int nx, int ny) {
+  return 20LL * L > 19LL * nx && 20LL * L > 19LL * ny;
+}
+
 __device__ __forceinline__ int wr(int i, int n) {
   if (n >= 4) return i < 0 ? i + n : (i >= n ? i - n : i);
   return wrapi(i, n);
@@ -1250,12 +1267,15 @@ __global__ void __launch_bounds__(NF * 32) k_col_sums(const DiagJob *__restrict_
 // two shared tiles [field][129] (column c at (c % 4) 32 + c / 4: conflict-free
 // writes) and copied out as the consecutive words of its records, so one
 // barrier per row suffices.
-template <typename T, int NF>
+// PLANAR: the tables of one plane per field; each lane stores its four
+// prefixes as 32 aligned bytes, without staging and barriers (8192^2: 2.2 ms
+// against 3.04 for the records).
+template <typename T, int NF, bool PLANAR>
 __global__ void __launch_bounds__(NF * 32) k_sat_tile(const DiagJob *__restrict__ jobs,
                                                       int rb_rows) {
   constexpr int R = sizeof(T) == 4 ? 8 : 4;  // rows of loads in flight per warp
   constexpr int NT = NF * 32, TS = kStrip + 1;
-  __shared__ long long tile[2][NF][TS];
+  __shared__ long long tile[PLANAR ? 1 : 2][PLANAR ? 1 : NF][TS];
   const int f = threadIdx.x >> 5, lane = threadIdx.x & 31, s = blockIdx.x, rb = blockIdx.y;
   const int nrb = gridDim.y;
   const DiagJob &J = jobs[blockIdx.z];
@@ -1272,10 +1292,29 @@ __global__ void __launch_bounds__(NF * 32) k_sat_tile(const DiagJob *__restrict_
   long long *tab = sat_base(J.base, N);
   const int e = reinterpret_cast<const int *>(J.part + exps_at())[f];
   long long col[4] = {0, 0, 0, 0}, lf = 0;
-  if (rb == 0) {
+  const size_t pp = planar_pitch(nx);
+  long long *plane = tab + (size_t)f * planar_stride(nx, ny) + 3;  // P_f(0, 0)
+  // stores P(x + 1 .. x + 4, row) where those columns exist
+  auto put = [&](int row, const long long (&v)[4]) {
+    long long *o = plane + (size_t)row * pp + x + 1;
+    if (x + 3 < nx) {
+      *reinterpret_cast<longlong2 *>(o) = make_longlong2(v[0], v[1]);
+      *reinterpret_cast<longlong2 *>(o + 2) = make_longlong2(v[2], v[3]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (x + j < nx) o[j] = v[j];
+    }
+    if (s == 0 && lane == 0) o[-1] = 0;  // column 0
+  };
+  if (PLANAR && rb == 0) {
+    const long long zero[4] = {0, 0, 0, 0};
+    put(0, zero);
+  }
+  if (!PLANAR && rb == 0) {
     for (int w = threadIdx.x; w < nw; w += NT) tab[(size_t)(x0 + 1) * NF + w] = 0;  // row 0
     if (s == 0 && threadIdx.x < NF) tab[threadIdx.x] = 0;
-  } else {  // the rows above this block: left parts plus the strip's column prefix
+  } else if (rb > 0) {  // the rows above this block: left parts plus the strip's column prefix
     const long long *cs = colsum_base(J.base, N, NF, ns, ny) + ((size_t)f * ns + s) * nrb * kStrip;
     const long long *lsum =
         colsum_base(J.base, N, NF, ns, ny) + (size_t)NF * ns * nrb * kStrip + ((size_t)f * ns + s) * nrb;
@@ -1310,17 +1349,20 @@ __global__ void __launch_bounds__(NF * 32) k_sat_tile(const DiagJob *__restrict_
       v[2] += v[1];
       v[3] += v[2];
       const long long off = l + warp_incl_scan(v[3], lane) - v[3];
-      long long *t = tile[y & 1][f];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        col[j] += off + v[j];
-        t[j * 32 + lane] = col[j];
+      for (int j = 0; j < 4; ++j) col[j] += off + v[j];
+      if constexpr (PLANAR) {
+        put(y + 1, col);
+        continue;
       }
+      long long *t = tile[PLANAR ? 0 : y & 1][PLANAR ? 0 : f];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) t[j * 32 + lane] = col[j];
       __syncthreads();
       long long *out = tab + ((size_t)(y + 1) * rs + x0 + 1) * NF;
       for (int w = threadIdx.x; w < nw; w += NT) {
         const int c = w / NF, g = w - c * NF;
-        out[w] = tile[y & 1][g][(c & 3) * 32 + (c >> 2)];
+        out[w] = tile[PLANAR ? 0 : y & 1][PLANAR ? 0 : g][(c & 3) * 32 + (c >> 2)];
       }
       if (s == 0 && threadIdx.x < NF) tab[(size_t)(y + 1) * rs * NF + threadIdx.x] = 0;
     }
@@ -1345,6 +1387,28 @@ __device__ __forceinline__ unsigned long long Pext(const long long *S, int nx, i
   return v;
 }
 
+// The same from a planar table.
+__device__ __forceinline__ unsigned long long Pplane(const long long *S, int nx, int ny, int x,
+                                                     int y) {
+  const int qx = x >= nx, qy = y >= ny;
+  const int xm = x - qx * nx, ym = y - qy * ny;
+  const size_t pp = planar_pitch(nx);
+  auto at = [&](int a, int b) { return (unsigned long long)S[(size_t)b * pp + 3 + a]; };
+  unsigned long long v = at(xm, ym);
+  if (qx) v += at(nx, ym);
+  if (qy) v += at(xm, ny);
+  if (qx && qy) v += at(nx, ny);
+  return v;
+}
+
+// max(m, |v|) for m >= 0; NaN in v is ignored, as fmax does.  FP64 by the bits
+// (non-negative doubles order like their bits), off the FP64 pipe.
+__device__ __forceinline__ float abs_max(float m, float v) { return fmax(m, fabs(v)); }
+__device__ __forceinline__ double abs_max(double m, double v) {
+  const long long b = __double_as_longlong(v) & 0x7fffffffffffffffll, a = __double_as_longlong(m);
+  return b > a && b <= 0x7ff0000000000000ll ? __longlong_as_double(b) : m;
+}
+
 template <typename MT>
 __device__ __forceinline__ MT delta_of(MT lhs, MT sum, MT mx) {
   const MT num = fabs(sum - lhs);
@@ -1353,7 +1417,7 @@ __device__ __forceinline__ MT delta_of(MT lhs, MT sum, MT mx) {
 }
 
 // One CTA per job, one thread per (size, field); constants at [size][kNT].
-__global__ void k_query_consts(const DiagJob *__restrict__ jobs, int nF) {
+__global__ void k_query_consts(const DiagJob *__restrict__ jobs, int nF, int planar) {
   const DiagJob &J = jobs[blockIdx.x];
   const int t = threadIdx.x;
   const int iL = t / kNT, k = t % kNT;
@@ -1361,7 +1425,9 @@ __global__ void k_query_consts(const DiagJob *__restrict__ jobs, int nF) {
   const int nx = J.nx, ny = J.ny;
   const size_t N = (size_t)nx * ny;
   const double area = (double)J.meta[8 * iL] * (double)J.meta[8 * iL];
-  const long long total = sat_base(J.base, N)[(sat_stride(nx, ny) - 1) * nF + k];
+  const size_t last = planar ? (size_t)k * planar_stride(nx, ny) + ny * planar_pitch(nx) + 3 + nx
+                             : (sat_stride(nx, ny) - 1) * nF + k;
+  const long long total = sat_base(J.base, N)[last];
   const double inv = J.part[inv_scale(k)];
   QConst q;
   q.mean_d = (double)total * inv / (double)N;
@@ -1452,19 +1518,22 @@ __device__ void block_sum_store_pairs(MT (&v)[NQ], double *out0, double *out1) {
 // d_k, d_k^2 and of the error's (or Ma_V's) deviation and its square; with
 // EXT also a CTA histogram in shared memory, added to the global one with
 // integer atomics (order-free, so deterministic).
+// planar: every origin of the whole_grid_box sizes, from planar tables (other
+// sizes are k_query_all's).
 template <typename MT, bool PER_BOX, bool EXT>
 __global__ void __launch_bounds__(256, 3) k_query(const DiagJob *__restrict__ jobs, int nF,
                                                const int *__restrict__ origins,
-                                               double *per_box, DiagDist ext) {
+                                               double *per_box, DiagDist ext, int planar) {
   constexpr int NZ = EXT ? 2 : 1;
   const DiagJob &J = jobs[blockIdx.z / NZ];
   const bool mpart = EXT && blockIdx.z % NZ == 1;
   const int iL = blockIdx.y;
-  if (iL >= J.nL || (int)blockIdx.x >= J.qblocks) return;
+  const int qb = planar ? J.qwhole : J.qblocks;
+  if (iL >= J.nL || (int)blockIdx.x >= qb) return;
+  if (planar && !whole_grid_box(J.meta[8 * iL], J.nx, J.ny)) return;
   const int grp = mpart ? 2 : (int)(threadIdx.x & 1), k0 = 6 * grp;
   const int slot = mpart ? (int)threadIdx.x : (int)(threadIdx.x >> 1);
   const int per_pass = mpart ? 256 : 128;
-  const int qb = J.qblocks;
   const int nx = J.nx, ny = J.ny;
   const int *meta = J.meta;
   const int L = meta[8 * iL], nb = meta[8 * iL + 1], ooff = meta[8 * iL + 2];
@@ -1499,38 +1568,26 @@ __global__ void __launch_bounds__(256, 3) k_query(const DiagJob *__restrict__ jo
   const int stride = qb * per_pass;
   int b = blockIdx.x * per_pass + slot;
   auto origin = [&](int i, int &x, int &y) {
-    if (ooff >= 0) {
-      x = origins[2 * (ooff + i)];
-      y = origins[2 * (ooff + i) + 1];
-    } else {
+    if (planar) {
       x = i % nx;
       y = i / nx;
+    } else {
+      x = origins[2 * (ooff + i)];
+      y = origins[2 * (ooff + i) + 1];
     }
   };
   int x0 = 0, y0 = 0;
   if (b < nb) origin(b, x0, y0);
-  // all periodic origins in row-major order: the next origin is this one
-  // advanced by the stride (no division per box)
-  const int sdx = ooff < 0 ? stride % nx : 0, sdy = ooff < 0 ? stride / nx : 0;
   for (; b < nb; b += stride) {
     int xn = 0, yn = 0;  // the next box's origin, loaded ahead
-    if (ooff < 0) {
-      xn = x0 + sdx;
-      yn = y0 + sdy;
-      if (xn >= nx) {
-        xn -= nx;
-        ++yn;
-      }
-    } else if (b + stride < nb) {
-      origin(b + stride, xn, yn);
-    }
+    if (b + stride < nb) origin(b + stride, xn, yn);
     const bool inside = x0 + L <= nx && y0 + L <= ny;
     MT lhs = 0, sum = 0, mx = 0;
     double *o = PER_BOX ? per_box + ((size_t)meta[8 * iL + 3] + b) * 15 : nullptr;
     // a non-wrapping box of a 12-field table: the six values of a corner are
     // 48 bytes at a 16-byte boundary, three vector loads per corner
     unsigned long long vs[6];
-    const bool vec = nF == 12 && nfield == 6;
+    const bool vec = nF == 12 && nfield == 6 && !planar;
     if (vec && !inside) {
       // a box across the periodic edge: the prefix sum extended periodically
       // is a signed sum of at most 3 x 3 table corners, columns
@@ -1582,6 +1639,10 @@ __global__ void __launch_bounds__(256, 3) k_query(const DiagJob *__restrict__ jo
       unsigned long long bs;
       if (vec) {
         bs = vs[j];
+      } else if (planar) {
+        const long long *Sp = sat_base(J.base, N) + (size_t)(k0 + j) * planar_stride(nx, ny);
+        bs = Pplane(Sp, nx, ny, x0 + L, y0 + L) - Pplane(Sp, nx, ny, x0, y0 + L) -
+             Pplane(Sp, nx, ny, x0 + L, y0) + Pplane(Sp, nx, ny, x0, y0);
       } else if (inside) {  // no periodic wrap: four direct corner loads
         const long long *lo = Sk + ((size_t)y0 * rs + x0) * nF, *hi = lo + (size_t)L * rs * nF;
         const size_t dx = (size_t)L * nF;
@@ -1651,15 +1712,221 @@ __global__ void __launch_bounds__(256, 3) k_query(const DiagJob *__restrict__ jo
   }
 }
 
+// ---------------------------------------------------------------------------
+// Every periodic origin of every size, from planar tables.  A thread owns one
+// column x of origins and one balance (or Ma_V) and walks chains of origins
+// y, y + L, y + 2 L, ...: with D(y) = P(x + L, y) - P(x, y) a box is
+// D(y + L) - D(y), and the upper row of one box is the lower row of the next,
+// so a box reads one new row of two neighbouring-lane-contiguous words per
+// field instead of four scattered records, and subtracts half as often.
+// k_query, which it replaces here, was bound by the L1 wavefronts of 48-byte
+// records and by issue; 8192^2, 12 sizes: 22.1 against 49.3 ms (issue
+// slots 66% busy at 20 warp instructions per box).
+// ---------------------------------------------------------------------------
+
+// (k_query, which it replaces here, keeps the sizes of nearly the whole grid.)
+
+// How the origins of a grid are shared out: CTAs of 256 threads, xt columns
+// by 256 / xt chains, nxb CTAs along x times `parts` along the chains.
+struct AllGrid {
+  int xt, nxb, parts;
+};
+__host__ __device__ inline AllGrid all_grid(int nx, int ny, int batch_jobs) {
+  AllGrid g;
+  g.xt = nx > 128 ? 256 : (nx > 64 ? 128 : (nx > 32 ? 64 : 32));
+  if (nx > 256 && (nx + 255) / 256 * 256 * 7 > nx * 8 && (nx + 127) / 128 * 128 < (nx + 255) / 256 * 256)
+    g.xt = 128;  // a ragged last CTA column
+  const int yt = 256 / g.xt, xb = (nx + g.xt - 1) / g.xt;
+  g.nxb = xb < kMaxQueryBlocks ? xb : kMaxQueryBlocks;
+  // about 32 boxes per thread, down to 4 where the batch has few CTAs
+  int parts = (ny + yt * 32 - 1) / (yt * 32);
+  const int jobs = batch_jobs < 1 ? 1 : batch_jobs;
+  const int want = (256 / jobs + g.nxb - 1) / g.nxb, cap = (ny + yt * 4 - 1) / (yt * 4);
+  if (parts < want) parts = want < cap ? want : cap;
+  if (parts > kMaxQueryBlocks / g.nxb) parts = kMaxQueryBlocks / g.nxb;
+  g.parts = parts < 1 ? 1 : parts;
+  return g;
+}
+
+// 64-bit integer to double, to nearest (ties away from zero), by integer
+// instructions: the conversion instruction runs on the narrow FP64 pipe.
+__device__ __forceinline__ double i64_to_f64(long long v) {
+  const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  const int n = __clzll((long long)a);
+  unsigned long long x = a << (n & 63);
+  const unsigned long long r = x + 0x400ull;
+  const unsigned carry = r < x;  // all ones rounded up: the next power of two
+  const unsigned e = n == 64 ? 0u : (unsigned)(1023 + 63 - 1 - n) << 20;
+  const unsigned hi = (unsigned)(r >> 43) + e + (carry << 21);
+  return __hiloint2double((int)(hi | (v < 0 ? 0x80000000u : 0u)), (int)(unsigned)(r >> 11));
+}
+
+// The statistics of one column's boxes of NFLD fields from plane k0 on.
+template <typename MT, bool PER_BOX, bool EXT, int NFLD>
+__device__ __forceinline__ void query_column(const DiagJob &J, int iL, int grp, int blk, int nblk_x,
+                                             const AllGrid &ag, const MT *sedge, unsigned *shist,
+                                             int ne, double *per_box, MT (&acc)[kQStats]) {
+  const int nx = J.nx, ny = J.ny, k0 = 6 * grp;
+  const int *meta = J.meta;
+  const int L = meta[8 * iL];
+  const size_t N = (size_t)nx * ny, pp = planar_pitch(nx), ps = planar_stride(nx, ny);
+  const long long *S = sat_base(J.base, N) + (size_t)k0 * ps + 3;
+  const QConst *qc = reinterpret_cast<const QConst *>(J.part + kPartConsts) + (size_t)iL * kNT + k0;
+  const int tx = threadIdx.x & (ag.xt - 1), ty = threadIdx.x / ag.xt, yt = 256 / ag.xt;
+  const int xb = blk % ag.nxb, nw = ag.parts * yt, w = (blk / ag.nxb) * yt + ty;
+  const MT ma_ref = NFLD == 1 ? sqrt(fmax(qc[0].mean<MT>(), MT(0))) * MT(1.7320508075688772) : MT(0);
+  long long mq[NFLD];
+  MT coef[NFLD], mean[NFLD], s1[NFLD], s2[NFLD], d1 = 0, d2 = 0;
+#pragma unroll
+  for (int j = 0; j < NFLD; ++j) {
+    mq[j] = qc[j].mq;
+    coef[j] = qc[j].coef<MT>();
+    mean[j] = qc[j].mean<MT>();
+    s1[j] = MT(0);
+    s2[j] = MT(0);
+  }
+  // a chain of up to kSeg boxes per unit of work
+  constexpr int kSeg = 16;
+  const int seg = min(kSeg, (ny + L - 1) / L), nseg = ((ny + L - 1) / L + seg - 1) / seg;
+  for (int xc = xb; xc < nblk_x; xc += ag.nxb) {
+    const int x = xc * ag.xt + tx;
+    if (x >= nx) break;
+    // columns of D: + P(xa), - P(x), and + P(xw) where the box crosses the edge
+    const bool wx = x + L > nx;
+    const int da = (wx ? nx : x + L) - x, dw = x + L - nx - x;
+    auto row = [&](int y, unsigned long long (&d)[NFLD]) {
+      const long long *p = S + (size_t)y * pp + x;
+#pragma unroll
+      for (int j = 0; j < NFLD; ++j) {
+        const long long *q = p + j * ps;
+        d[j] = (unsigned long long)__ldg(q + da) - (unsigned long long)__ldg(q);
+        if (wx) d[j] += (unsigned long long)__ldg(q + dw);
+      }
+    };
+    for (int u = w; u < L * nseg; u += nw) {
+      int y = u % L + (u / L) * seg * L;
+      if (y >= ny) continue;
+      unsigned long long dp[NFLD];
+      row(y, dp);
+      for (int i = 0; i < seg && y < ny; ++i) {
+        const int yn = y + L;
+        unsigned long long dn[NFLD];
+        row(yn <= ny ? yn : ny, dn);
+        if (yn > ny) {  // across the periodic edge in y
+          unsigned long long dv[NFLD];
+          row(yn - ny, dv);
+#pragma unroll
+          for (int j = 0; j < NFLD; ++j) dn[j] += dv[j];
+        }
+        MT lhs = 0, sum = 0, mx = 0;
+        double *o = PER_BOX ? per_box + ((size_t)meta[8 * iL + 3] + (size_t)y * nx + x) * 15 : nullptr;
+#pragma unroll
+        for (int j = 0; j < NFLD; ++j) {
+          const long long dq = (long long)(dn[j] - dp[j] - (unsigned long long)mq[j]);
+          dp[j] = dn[j];
+          MT v;
+          if constexpr (sizeof(MT) == 4) {
+            const MT d = to_mt<MT>(dq) * coef[j];
+            v = d + mean[j];
+            s1[j] += d;
+            s2[j] += d * d;
+          } else {  // sums of the integers, scaled once at the end
+            const double c = i64_to_f64(dq);
+            v = fma(c, coef[j], mean[j]);
+            s1[j] += c;
+            s2[j] = fma(c, c, s2[j]);
+          }
+          if (j == 0) {
+            lhs = v;
+          } else {
+            sum += v;
+            mx = abs_max(mx, v);
+          }
+          if (PER_BOX) o[2 + k0 + j] = (double)v;
+        }
+        MT val;  // delta of the balance, or Ma_V
+        if constexpr (NFLD == 1) {
+          val = sqrt(fmax(lhs, MT(0))) * MT(1.7320508075688772);
+          const MT dm = val - ma_ref;
+          d1 += dm;
+          d2 += dm * dm;
+        } else {
+          val = delta_of(lhs, sum, mx);
+          d1 += val;
+          d2 += val * val;
+        }
+        if constexpr (EXT) {
+          if (val == val) atomicAdd(&shist[bin_of(val, sedge, ne)], 1u);
+        }
+        if (PER_BOX) {
+          o[grp] = (double)val;
+          if (grp == 1) o[14] = 0.0;
+        }
+        y = yn;
+      }
+    }
+  }
+  acc[0] = d1;
+  acc[1] = d2;
+#pragma unroll
+  for (int j = 0; j < NFLD; ++j) {
+    acc[2 + 2 * j] = sizeof(MT) == 8 ? s1[j] * coef[j] : s1[j];
+    acc[3 + 2 * j] = sizeof(MT) == 8 ? s2[j] * coef[j] * coef[j] : s2[j];
+  }
+}
+
+// Grid (sizes, query CTAs, groups x jobs), groups = 2 (energy, enstrophy), or
+// 3 with the distributions (EXT: Ma_V); blockIdx.z = groups * job + group.
+template <typename MT, bool PER_BOX, bool EXT>
+__global__ void __launch_bounds__(256, 2)
+    k_query_all(const DiagJob *__restrict__ jobs, double *per_box, DiagDist ext, int batch_jobs) {
+  constexpr int NG = EXT ? 3 : 2;
+  const DiagJob &J = jobs[blockIdx.z / NG];
+  const int grp = blockIdx.z % NG, iL = blockIdx.x, blk = blockIdx.y, qb = J.qblocks;
+  if (iL >= J.nL || blk >= qb || whole_grid_box(J.meta[8 * iL], J.nx, J.ny)) return;
+  __shared__ MT sedge[EXT ? kDiagMaxEdges : 1];
+  __shared__ unsigned shist[EXT ? kDiagMaxEdges + 1 : 1];
+  int ne = 0;
+  if constexpr (EXT) {
+    ne = grp == 2 ? ext.n_mach : ext.n_delta;
+    const double *e = grp == 2 ? ext.mach_edges : ext.delta_edges;
+    for (int i = threadIdx.x; i <= ne; i += 256) {
+      if (i < ne) sedge[i] = (MT)e[i];
+      shist[i] = 0u;
+    }
+    __syncthreads();
+  }
+  const AllGrid ag = all_grid(J.nx, J.ny, batch_jobs);
+  const int nblk_x = (J.nx + ag.xt - 1) / ag.xt;
+  MT acc[kQStats];
+#pragma unroll
+  for (int q = 0; q < kQStats; ++q) acc[q] = MT(0);
+  if (EXT && grp == 2)
+    query_column<MT, PER_BOX, EXT, 1>(J, iL, grp, blk, nblk_x, ag, sedge, shist, ne, per_box, acc);
+  else
+    query_column<MT, PER_BOX, EXT, 6>(J, iL, grp, blk, nblk_x, ag, sedge, shist, ne, per_box, acc);
+  double *pq = J.part + kPartQuery;
+  block_sum_store_mt<kQStats, MT>(acc, pq + (((size_t)iL * 3 + grp) * qb + blk) * kQStats);
+  if constexpr (EXT) {
+    __syncthreads();
+    unsigned long long *h =
+        ext.hist + ((size_t)J.meta[8 * iL + 4] * 3 + grp) * (kDiagMaxEdges + 1);
+    for (int i = threadIdx.x; i <= ne; i += 256)
+      if (shist[i]) atomicAdd(&h[i], (unsigned long long)shist[i]);
+  }
+}
+
 // Mean and population standard deviation of the 15 quantities per size,
 // and with `mach` those of Ma_V.  Grid (sizes, jobs), 384 threads: 8 per
 // (group, slot) sum interleaved block partials in a fixed order.
 template <typename MT>
-__global__ void k_stats_final(const DiagJob *__restrict__ jobs, double *stats, double *mach) {
+__global__ void k_stats_final(const DiagJob *__restrict__ jobs, double *stats, double *mach,
+                              int planar) {
   const DiagJob &J = jobs[blockIdx.y];
   const int iL = blockIdx.x;
   if (iL >= J.nL) return;
-  const int nblocks = J.qblocks;
+  const int nblocks =
+      planar && whole_grid_box(J.meta[8 * iL], J.nx, J.ny) ? J.qwhole : J.qblocks;
   const double *partials = J.part + kPartQuery;
   const QConst *consts = reinterpret_cast<const QConst *>(J.part + kPartConsts);
   const int q = threadIdx.x >> 3, j = threadIdx.x & 7;  // q = grp * 14 + slot
@@ -1739,13 +2006,17 @@ dim3 cells_grid(const Grid &g, dim3 b) {
 template <typename T, typename MT>
 cudaError_t balance_launches(const DiagJob *jobs_host, const DiagJob *jobs, int G, bool pairs,
                              const int *origins, double *stats, double *per_box,
-                             const DiagDist *dist, cudaStream_t s) {
-  int nx = 1, ny = 1, nL = 1, qblocks = 1;
+                             const DiagDist *dist, int batch_jobs, cudaStream_t s) {
+  const bool planar = origins == nullptr;  // every periodic origin
+  int nx = 1, ny = 1, nL = 1, qblocks = 1, qwhole = 1;
+  bool any_whole = false;
   for (int j = 0; j < G; ++j) {
     nx = std::max(nx, jobs_host[j].nx);
     ny = std::max(ny, jobs_host[j].ny);
     nL = std::max(nL, jobs_host[j].nL);
     qblocks = std::max(qblocks, jobs_host[j].qblocks);
+    qwhole = std::max(qwhole, jobs_host[j].qwhole);
+    any_whole |= jobs_host[j].any_whole != 0;
   }
   const int nF = dist ? kNT : 12;  // |u|^2 gets a table only for Ma_V
   const dim3 cb(32, 8), cg((nx + 31) / 32, (ny + 7) / 8, G);
@@ -1797,23 +2068,39 @@ cudaError_t balance_launches(const DiagJob *jobs_host, const DiagJob *jobs, int 
     else
       k_col_sums<T, 12><<<dim3(ns, nrb, G), 12 * 32, 0, s>>>(jobs, rb_rows);
   }
-  if (nF == kNT)
-    k_sat_tile<T, kNT><<<dim3(ns, nrb, G), kNT * 32, 0, s>>>(jobs, rb_rows);
-  else
-    k_sat_tile<T, 12><<<dim3(ns, nrb, G), 12 * 32, 0, s>>>(jobs, rb_rows);
-  k_query_consts<<<G, kDiagMaxL * kNT, 0, s>>>(jobs, nF);
-  const DiagDist none{};
-  if (dist) {
-    k_query<MT, false, true><<<dim3(qblocks, nL, 2 * G), 256, 0, s>>>(jobs, nF, origins, nullptr,
-                                                                       *dist);
-  } else {
-    const dim3 qg(qblocks, nL, G);
-    if (per_box)
-      k_query<MT, true, false><<<qg, 256, 0, s>>>(jobs, nF, origins, per_box, none);
+  const dim3 sg(ns, nrb, G);
+  if (planar) {
+    if (nF == kNT)
+      k_sat_tile<T, kNT, true><<<sg, kNT * 32, 0, s>>>(jobs, rb_rows);
     else
-      k_query<MT, false, false><<<qg, 256, 0, s>>>(jobs, nF, origins, nullptr, none);
+      k_sat_tile<T, 12, true><<<sg, 12 * 32, 0, s>>>(jobs, rb_rows);
+  } else if (nF == kNT) {
+    k_sat_tile<T, kNT, false><<<sg, kNT * 32, 0, s>>>(jobs, rb_rows);
+  } else {
+    k_sat_tile<T, 12, false><<<sg, 12 * 32, 0, s>>>(jobs, rb_rows);
   }
-  k_stats_final<MT><<<dim3(nL, G), 384, 0, s>>>(jobs, stats, dist ? dist->mach : nullptr);
+  k_query_consts<<<G, kDiagMaxL * kNT, 0, s>>>(jobs, nF, planar);
+  const DiagDist none{};
+  if (planar) {
+    const dim3 qg(nL, qblocks, (dist ? 3 : 2) * G);
+    if (dist)
+      k_query_all<MT, false, true><<<qg, 256, 0, s>>>(jobs, nullptr, *dist, batch_jobs);
+    else if (per_box)
+      k_query_all<MT, true, false><<<qg, 256, 0, s>>>(jobs, per_box, none, batch_jobs);
+    else
+      k_query_all<MT, false, false><<<qg, 256, 0, s>>>(jobs, nullptr, none, batch_jobs);
+  }
+  if (!planar || any_whole) {
+    const dim3 qg(planar ? qwhole : qblocks, nL, (dist ? 2 : 1) * G);
+    if (dist)
+      k_query<MT, false, true><<<qg, 256, 0, s>>>(jobs, nF, origins, nullptr, *dist, planar);
+    else if (per_box)
+      k_query<MT, true, false><<<qg, 256, 0, s>>>(jobs, nF, origins, per_box, none, planar);
+    else
+      k_query<MT, false, false><<<qg, 256, 0, s>>>(jobs, nF, origins, nullptr, none, planar);
+  }
+  k_stats_final<MT><<<dim3(nL, G), 384, 0, s>>>(jobs, stats, dist ? dist->mach : nullptr,
+                                                  planar);
   return cudaGetLastError();
 }
 
@@ -1849,23 +2136,33 @@ cudaError_t diag_global(const Member &hm, const double *snap3, const DiagScratch
   return cudaGetLastError();
 }
 
-// Box lists: about 8 boxes per thread pair; every periodic origin: about 32
-// per thread pair; at most kMaxQueryBlocks CTAs per (job, size, part).  A
-// batch of few jobs with few boxes (a small grid) gets smaller CTAs, down to
-// one pass of 128 boxes, about 256 per size over the batch: its FP64
-// statistics then spread over the SMs instead of queueing on a few (GB300
-// issues about 1.7 FP64 FMAs per clock per SM).
-int diag_query_blocks(int max_boxes, bool origin_list, int batch_jobs) {
-  const int per_cta = origin_list ? 1024 : 4096;
+static int diag_list_blocks(int max_boxes, int per_cta, int batch_jobs) {
   int qb = (max_boxes + per_cta - 1) / per_cta;
   const int want = (256 + std::max(1, batch_jobs) - 1) / std::max(1, batch_jobs);
   qb = std::max(qb, std::min(want, (max_boxes + 127) / 128));
   return std::min(kMaxQueryBlocks, std::max(1, qb));
 }
 
+// Every periodic origin: all_grid.  Box lists: about 8 boxes per thread pair;
+// at most kMaxQueryBlocks CTAs per (job, size, part).  A
+// batch of few jobs with few boxes (a small grid) gets smaller CTAs, down to
+// one pass of 128 boxes, about 256 per size over the batch: its FP64
+// statistics then spread over the SMs instead of queueing on a few (GB300
+// issues about 1.7 FP64 FMAs per clock per SM).
+int diag_query_blocks(int nx, int ny, int max_boxes, bool origin_list, int batch_jobs) {
+  if (!origin_list) {
+    const AllGrid g = all_grid(nx, ny, batch_jobs);
+    return g.nxb * g.parts;
+  }
+  return diag_list_blocks(max_boxes, 1024, batch_jobs);
+}
+int diag_whole_blocks(int boxes, int batch_jobs) { return diag_list_blocks(boxes, 4096, batch_jobs); }
+bool diag_whole_box(int L, int nx, int ny) { return whole_grid_box(L, nx, ny); }
+
 size_t diag_slot_doubles(size_t Nmax, size_t pad) {
   // snapshot slots + term-stage fields + kNT padded tables, in whole 256-byte
-  // units (so field rows keep the 16-byte alignment of vector loads)
+  // units (so field rows keep the 16-byte alignment of vector loads); the
+  // planar tables start on 32 bytes like the slot
   const size_t d = (size_t)(kSnapSlots + NF) * Nmax + kNT * (Nmax + pad);
   return (d + 31) / 32 * 32;
 }
@@ -1879,16 +2176,16 @@ size_t diag_job_partials(size_t Nmax, size_t pad) {
 cudaError_t diag_balance(const DiagJob *jobs_host, const DiagJob *jobs_dev, int G,
                          int precision, bool pairs, const int *origins_dev,
                          double *stats_dev, double *per_box_dev, const DiagDist *dist,
-                         cudaStream_t s) {
+                         int batch_jobs, cudaStream_t s) {
   if (G < 1 || (per_box_dev && G != 1) || (per_box_dev && dist)) return cudaErrorInvalidValue;
   if (dist && (dist->n_delta < 1 || dist->n_delta > kDiagMaxEdges || dist->n_mach < 1 ||
                dist->n_mach > kDiagMaxEdges))
     return cudaErrorInvalidValue;
   if (precision == 32)
     return balance_launches<float, float>(jobs_host, jobs_dev, G, pairs, origins_dev,
-                                          stats_dev, per_box_dev, dist, s);
+                                          stats_dev, per_box_dev, dist, batch_jobs, s);
   return balance_launches<double, double>(jobs_host, jobs_dev, G, pairs, origins_dev,
-                                          stats_dev, per_box_dev, dist, s);
+                                          stats_dev, per_box_dev, dist, batch_jobs, s);
 }
 
 }  // namespace lbm

@@ -36,7 +36,7 @@ __host__ __device__ constexpr int opposite(int l) {
 // k = exponent of rho0 plus two, so that rho0 lies in [1/4, 1/2) 2^k.
 struct FixedBgk {
   int k, ok;           // ok: the member can take it (BGK, moderate parameters)
-  long long om, om9;   // omega 2^62, omega / 9 2^65
+  long long om, om9, om9h;  // omega 2^62, omega / 9 2^65 and 2^64
   long long alpha;     // drag 2^64
   int forced, pad;     // forced: a force or drag
 };
@@ -352,13 +352,17 @@ struct DiagJob {
   const float *nu_cell_f;      // variable viscosity: local viscosity at n (FP32
   const double *nu_cell_d;     // or FP64 storage), else both NULL
   int qblocks;                 // query CTAs per (size, balance):
-                               // diag_query_blocks(max_boxes, origin list?)
+                               // diag_query_blocks(...)
+  int qwhole, any_whole;       // every origin: the CTAs of the sizes of nearly the
+                               // whole grid, and whether there are any
 };
 // Query CTAs for a job: a fixed function of its own box count, so that the
 // statistics do not depend on which members share a batch.
-int diag_query_blocks(int max_boxes, bool origin_list, int batch_jobs);
+int diag_query_blocks(int nx, int ny, int max_boxes, bool origin_list, int batch_jobs);
+int diag_whole_blocks(int boxes, int batch_jobs);
+bool diag_whole_box(int L, int nx, int ny);
 // Doubles of one field slot and of one partials slot for members of at most
-// Nmax cells and nx + ny + 1 <= pad.
+// Nmax cells and nx + 7 ny + 7 <= pad.
 size_t diag_slot_doubles(size_t Nmax, size_t pad);
 size_t diag_job_partials(size_t Nmax, size_t pad);
 // The balance diagnostic of G jobs (precision 32: FP32 term arithmetic, 64:
@@ -379,7 +383,7 @@ struct DiagDist {
 cudaError_t diag_balance(const DiagJob *jobs_host, const DiagJob *jobs_dev, int G,
                          int precision, bool pairs, const int *origins_dev,
                          double *stats_dev, double *per_box_dev, const DiagDist *dist,
-                         cudaStream_t s);
+                         int batch_jobs, cudaStream_t s);
 
 // Adjoint (lbm_adjoint.cu).
 cudaError_t adjoint_step(const Member &hm, const double *f_n, const double *lam_in,

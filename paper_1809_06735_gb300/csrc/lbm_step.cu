@@ -557,7 +557,7 @@ cudaError_t launch_step_scalar_batch(int precision, const Member *d_members, con
     dim3 g = grid2d(nx_max, ny_max, b);
     g.z = list.n;
     if (precision == 32)
-      k_step_scalar_multi<float, 256, 1><<<g, b, 0, s>>>(d_members, list, state);
+      k_step_scalar_multi<float, 256, 4><<<g, b, 0, s>>>(d_members, list, state);
     else if (b.x == 32)
       k_step_scalar_multi<double, 64, 1><<<g, b, 0, s>>>(d_members, list, state);
     else
@@ -575,7 +575,7 @@ cudaError_t launch_step_scalar(int precision, const Member *d_members, int membe
   const bool small = (long long)nx * ny < (1LL << 17);
   const dim3 b = small ? dim3(32, 2) : dim3(64, 4), g = grid2d(nx, ny, b);
   if (precision == 32)
-    k_step_scalar<float, 256, 1><<<g, b, 0, s>>>(d_members, member, state, rec);
+    k_step_scalar<float, 256, 4><<<g, b, 0, s>>>(d_members, member, state, rec);
   else if (small)
     k_step_scalar<double, 64, 1><<<g, b, 0, s>>>(d_members, member, state, rec);
   else
