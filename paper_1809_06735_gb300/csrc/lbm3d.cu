@@ -381,26 +381,34 @@ __device__ __forceinline__ int wrap4(int i, int n) {
   return ((i % n) + n) % n;
 }
 
-// Eq. (18) along axis a (0 x, 1 y, 2 z), periodic, in the arithmetic type T.
+// Wrapped offsets of one cell's stencil points, computed once and shared by
+// every derivative of the cell (the 30 derivatives of pass 1 spent most of
+// their instructions on them): o[a][k + 4] the offset of the point k cells
+// along axis a (0 x, 1 y, 2 z), c the cell itself.
+struct Nb3 {
+  int c, o[3][9];
+};
+__device__ __forceinline__ Nb3 make_nb3(const M3 &M, int x, int y, int z) {
+  Nb3 nb;
+  const int sy = M.nx, sz = M.nx * M.ny;
+  nb.c = z * sz + y * sy + x;
+#pragma unroll
+  for (int k = -4; k <= 4; ++k) {
+    nb.o[0][k + 4] = wrap4(x + k, M.nx) - x;
+    nb.o[1][k + 4] = (wrap4(y + k, M.ny) - y) * sy;
+    nb.o[2][k + 4] = (wrap4(z + k, M.nz) - z) * sz;
+  }
+  return nb;
+}
+
+// Eq. (18) along axis a, periodic, in the arithmetic type T.
 template <typename T>
-__device__ __forceinline__ T D3(const M3 &M, const T *A, int x, int y, int z, int a) {
+__device__ __forceinline__ T D3(const Nb3 &nb, const T *A, int a) {
   const T cf[4] = {T(0.8), T(-0.2), T(4.0 / 105.0), T(-1.0 / 280.0)};
+  const T *c = A + nb.c;
   T s = T(0);
 #pragma unroll
-  for (int k = 1; k <= 4; ++k) {
-    size_t p, q;
-    if (a == 0) {
-      p = cell(M, wrap4(x + k, M.nx), y, z);
-      q = cell(M, wrap4(x - k, M.nx), y, z);
-    } else if (a == 1) {
-      p = cell(M, x, wrap4(y + k, M.ny), z);
-      q = cell(M, x, wrap4(y - k, M.ny), z);
-    } else {
-      p = cell(M, x, y, wrap4(z + k, M.nz));
-      q = cell(M, x, y, wrap4(z - k, M.nz));
-    }
-    s += cf[k - 1] * (A[p] - A[q]);
-  }
+  for (int k = 1; k <= 4; ++k) s += cf[k - 1] * (__ldg(c + nb.o[a][4 + k]) - __ldg(c + nb.o[a][4 - k]));
   return s;
 }
 
@@ -479,27 +487,33 @@ __global__ void k3_prep(Diag3 J) {
 // O^n - O^{n-1} = dw01 . (2 w^n - dw01)/2), S, RHS^{E,2}, RHS^{E,4},
 // RHS^{O,2}, RHS^{O,3}, RHS^{O,6}, and the fluxes of pass 2.
 template <typename T>
-__global__ void k3_grad(Diag3 J) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) k3_grad(Diag3 J) {
   D3CELL;
+  const Nb3 nb = make_nb3(M, x, y, z);
   T G[3][3];
+#pragma unroll
   for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j) G[i][j] = D3<T>(M, F(UX0 + i), x, y, z, j);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) G[i][j] = D3<T>(nb, F(UX0 + i), j);
   T w0[3];
   w0[0] = G[2][1] - G[1][2];
   w0[1] = G[0][2] - G[2][0];
   w0[2] = G[1][0] - G[0][1];
   T dO[2];
   T w1[3];
+#pragma unroll
   for (int m = 0; m < 2; ++m) {
     const T *U = F((m ? DU12X : DU01X)), *V = F((m ? DU12Y : DU01Y)), *W = F((m ? DU12Z : DU01Z));
-    const T dw[3] = {D3<T>(M, W, x, y, z, 1) - D3<T>(M, V, x, y, z, 2),
-                     D3<T>(M, U, x, y, z, 2) - D3<T>(M, W, x, y, z, 0),
-                     D3<T>(M, V, x, y, z, 0) - D3<T>(M, U, x, y, z, 1)};
+    const T dw[3] = {D3<T>(nb, W, 1) - D3<T>(nb, V, 2),
+                     D3<T>(nb, U, 2) - D3<T>(nb, W, 0),
+                     D3<T>(nb, V, 0) - D3<T>(nb, U, 1)};
     const T *wl = m ? w1 : w0;  // the later level of the pair
     T p = T(0);
+#pragma unroll
     for (int i = 0; i < 3; ++i) p += dw[i] * (T(2) * wl[i] - dw[i]);
     dO[m] = T(0.5) * p;
     if (m == 0)
+#pragma unroll
       for (int i = 0; i < 3; ++i) w1[i] = w0[i] - dw[i];
   }
   F(T3 + 6)[c] = T(0.5) * (T(3) * dO[0] - dO[1]);
@@ -507,20 +521,26 @@ __global__ void k3_grad(Diag3 J) {
   const T u[3] = {F(UX0)[c], F(UY0)[c], F(UZ0)[c]}, r = F(R0)[c];
   const T nr = (T)M.nu * r;
   T S[3][3];
+#pragma unroll
   for (int i = 0; i < 3; ++i)
+#pragma unroll
     for (int j = 0; j < 3; ++j) S[i][j] = G[i][j] + G[j][i];
   T gp = T(0), sd = T(0), st = T(0);
-  for (int i = 0; i < 3; ++i) gp += u[i] * D3<T>(M, F(DR), x, y, z, i) / T(3);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) gp += u[i] * D3<T>(nb, F(DR), i) / T(3);
+#pragma unroll
   for (int i = 0; i < 3; ++i)
+#pragma unroll
     for (int j = 0; j < 3; ++j) {
       sd += S[i][j] * G[i][j];
       st += w0[i] * w0[j] * G[i][j];
     }
   const T div = G[0][0] + G[1][1] + G[2][2];
   T cf = T(0);  // omega . curl(F / rho)
+#pragma unroll
   for (int i = 0; i < 3; ++i) {
     const int j = (i + 1) % 3, k = (i + 2) % 3;
-    cf += w0[i] * (D3<T>(M, F(FRX + k), x, y, z, j) - D3<T>(M, F(FRX + j), x, y, z, k));
+    cf += w0[i] * (D3<T>(nb, F(FRX + k), j) - D3<T>(nb, F(FRX + j), k));
   }
   F(T3 + 2)[c] = -gp;
   F(T3 + 4)[c] = -nr * sd;
@@ -528,6 +548,7 @@ __global__ void k3_grad(Diag3 J) {
   F(T3 + 9)[c] = cf;
   F(T3 + 12)[c] = st;
   const T E0 = T(0.5) * r * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+#pragma unroll
   for (int j = 0; j < 3; ++j) {
     F(EUX + j)[c] = E0 * u[j];
     F(OUX + j)[c] = Om0 * u[j];
@@ -545,32 +566,38 @@ __global__ void k3_grad(Diag3 J) {
 // Pass 2: RHS^{E,1}, RHS^{E,5}, RHS^{O,1}; H_i = d_j(nu rho S_ij)/rho;
 // RHS^{O,4} = H . curl(omega); H x omega for pass 3.
 template <typename T>
-__global__ void k3_flux(Diag3 J) {
+__global__ void __launch_bounds__(256) k3_flux(Diag3 J) {
   D3CELL;
+  const Nb3 nb = make_nb3(M, x, y, z);
   T e1 = T(0), e5 = T(0), o1 = T(0);
+#pragma unroll
   for (int j = 0; j < 3; ++j) {
-    e1 -= D3<T>(M, F(EUX + j), x, y, z, j);
-    e5 += D3<T>(M, F(CUX + j), x, y, z, j);
-    o1 -= D3<T>(M, F(OUX + j), x, y, z, j);
+    e1 -= D3<T>(nb, F(EUX + j), j);
+    e5 += D3<T>(nb, F(CUX + j), j);
+    o1 -= D3<T>(nb, F(OUX + j), j);
   }
   const int sidx[3][3] = {{SXX, SXY, SXZ}, {SXY, SYY, SYZ}, {SXZ, SYZ, SZZ}};
   const T r = F(R0)[c];
   T H[3];
+#pragma unroll
   for (int i = 0; i < 3; ++i) {
     T h = T(0);
-    for (int j = 0; j < 3; ++j) h += D3<T>(M, F(sidx[i][j]), x, y, z, j);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) h += D3<T>(nb, F(sidx[i][j]), j);
     H[i] = h / r;
   }
   T o4 = T(0);
+#pragma unroll
   for (int i = 0; i < 3; ++i) {
     const int j = (i + 1) % 3, k = (i + 2) % 3;
-    o4 += H[i] * (D3<T>(M, F(WX + k), x, y, z, j) - D3<T>(M, F(WX + j), x, y, z, k));
+    o4 += H[i] * (D3<T>(nb, F(WX + k), j) - D3<T>(nb, F(WX + j), k));
   }
   const T w[3] = {F(WX)[c], F(WY)[c], F(WZ)[c]};
   F(T3 + 1)[c] = e1;
   F(T3 + 5)[c] = e5;
   F(T3 + 7)[c] = o1;
   F(T3 + 10)[c] = o4;
+#pragma unroll
   for (int j = 0; j < 3; ++j) {
     const int a = (j + 1) % 3, b = (j + 2) % 3;
     F(HWX + j)[c] = H[a] * w[b] - H[b] * w[a];
@@ -579,10 +606,12 @@ __global__ void k3_flux(Diag3 J) {
 
 // Pass 3: RHS^{O,5} = div(H x omega).
 template <typename T>
-__global__ void k3_curl(Diag3 J) {
+__global__ void __launch_bounds__(256) k3_curl(Diag3 J) {
   D3CELL;
+  const Nb3 nb = make_nb3(M, x, y, z);
   T s = T(0);
-  for (int j = 0; j < 3; ++j) s += D3<T>(M, F(HWX + j), x, y, z, j);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) s += D3<T>(nb, F(HWX + j), j);
   F(T3 + 11)[c] = s;
 }
 
@@ -650,58 +679,136 @@ __global__ void k3_scales(Diag3 J, const unsigned long long *maxbits, double *ma
   maxes[80 + k] = ldexp(1.0, -e);
 }
 
-// Quantised values scanned along x: one thread per (y, z, field) row.
+// round(v 2^e) to nearest even for |v| 2^e < 2^62.  FP32 by integer
+// instructions where 2^e is a float (see the 2D tables), FP64 and the rest by
+// the conversion.
+__device__ __forceinline__ long long quantize3(float v, int e, double sc) {
+  if (e > 120) return __double2ll_rn((double)v * sc);
+  const float w = v * __int_as_float((e + 127) << 23), aw = fabsf(w);
+  long long q;
+  if (aw < 8388608.0f) {
+    q = __float_as_int(aw + 8388608.0f) - 0x4B000000;
+  } else {
+    const unsigned bits = __float_as_uint(aw);
+    const int sh = (int)(bits >> 23) - 150;
+    q = sh < 40 ? (long long)((bits & 0x7fffffu) | 0x800000u) << sh : 0ll;
+  }
+  return w < 0.0f ? -q : q;
+}
+__device__ __forceinline__ long long quantize3(double v, int, double sc) {
+  return __double2ll_rn(v * sc);
+}
+
+// The tables' prefixes along x and y: a warp per (z plane, field) walks the
+// rows of each 128-column strip, four cells per lane and kR rows of loads in
+// flight: the row's prefix by a warp scan, the strip's part left of it from
+// the table's own previous column, and running column sums in registers.
+// (One thread per row along x and one per column along y took 358 + 146 us on
+// 128^3, uncoalesced and latency-bound.)
 template <typename T>
-__global__ void k3_scan_x(Diag3 J, const double *scales, long long *tab) {
+__global__ void __launch_bounds__(128) k3_scan_xy(Diag3 J, const double *scales, long long *tab) {
+  constexpr int kR = sizeof(T) == 4 ? 8 : 4;
   const M3 &M = *J.m;
-  const int y = blockIdx.x * blockDim.x + threadIdx.x, z = blockIdx.y, k = blockIdx.z;
-  if (y > M.ny || z > M.nz) return;
-  const size_t ts = (size_t)(M.nx + 1) * (M.ny + 1) * (M.nz + 1);
-  long long *t = tab + (size_t)k * ts;
-  if (y == 0 || z == 0) {  // zero planes
-    for (int x = 0; x <= M.nx; ++x) t[tidx(M, x, y, z)] = 0;
+  const int nx = M.nx, ny = M.ny, lane = threadIdx.x & 31;
+  const int z = blockIdx.x * 4 + (threadIdx.x >> 5), k = blockIdx.y;
+  if (z > M.nz) return;  // whole warps
+  const size_t rs = (size_t)nx + 1;
+  long long *t = tab + (size_t)k * rs * (ny + 1) * (M.nz + 1) + (size_t)z * rs * (ny + 1);
+  if (z == 0) {  // the zero plane
+    for (size_t i = lane; i < rs * (ny + 1); i += 32) t[i] = 0;
     return;
   }
-  const T *A = reinterpret_cast<const T *>(J.f + (size_t)(T3 + k) * M.N);
+  for (size_t i = lane; i < rs; i += 32) t[i] = 0;
+  const T *A = reinterpret_cast<const T *>(J.f + (size_t)(T3 + k) * M.N) + (size_t)(z - 1) * nx * ny;
   const double sc = scales[k];
-  long long acc = 0;
-  t[tidx(M, 0, y, z)] = 0;
-  for (int x = 0; x < M.nx; ++x) {
-    acc += __double2ll_rn((double)A[cell(M, x, y - 1, z - 1)] * sc);
-    t[tidx(M, x + 1, y, z)] = acc;
+  const int e = (int)scales[16 + k];
+  const bool vec = nx % 4 == 0;
+  for (int x0 = 0; x0 < nx; x0 += 128) {
+    __syncwarp();  // the previous strip's last column, written by another lane
+    const int x = x0 + 4 * lane;
+    long long col[4] = {0, 0, 0, 0};
+    for (int y0 = 0; y0 < ny; y0 += kR) {
+      T a[kR][4];
+      long long left[kR];
+#pragma unroll
+      for (int r = 0; r < kR; ++r) {
+        const int y = y0 + r;
+        const T *row = A + (size_t)y * nx + x;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) a[r][j] = T(0);
+        left[r] = 0;
+        if (y >= ny) continue;
+        if (vec && x < nx) {
+          if constexpr (sizeof(T) == 4) {
+            const float4 q = *reinterpret_cast<const float4 *>(row);
+            a[r][0] = q.x; a[r][1] = q.y; a[r][2] = q.z; a[r][3] = q.w;
+          } else {
+            const double2 q = *reinterpret_cast<const double2 *>(row);
+            const double2 w = *reinterpret_cast<const double2 *>(row + 2);
+            a[r][0] = q.x; a[r][1] = q.y; a[r][2] = w.x; a[r][3] = w.y;
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (x + j < nx) a[r][j] = row[j];
+        }
+        if (x0 > 0) left[r] = t[(size_t)(y + 1) * rs + x0] - t[(size_t)y * rs + x0];
+      }
+#pragma unroll
+      for (int r = 0; r < kR; ++r) {
+        const int y = y0 + r;
+        if (y >= ny) break;  // whole warps
+        long long v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = quantize3(a[r][j], e, sc);
+        v[1] += v[0];
+        v[2] += v[1];
+        v[3] += v[2];
+        long long inc = v[3];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const long long n = __shfl_up_sync(0xffffffffu, inc, o);
+          if (lane >= o) inc += n;
+        }
+        const long long off = left[r] + inc - v[3];
+        long long *o = t + (size_t)(y + 1) * rs + x + 1;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          col[j] += off + v[j];
+          if (x + j < nx) o[j] = col[j];
+        }
+        if (x == 0) o[-1] = 0;
+      }
+    }
   }
 }
 
-// Prefix along y (axis 1) or z (axis 2) of the tables in place: one thread
-// per (x, other coordinate, field) line.
-__global__ void k3_scan_yz(Diag3 J, long long *tab, int axis) {
+// Prefix along z of the tables in place: one thread per (x, y, field) line,
+// eight planes of loads in flight.
+__global__ void __launch_bounds__(128) k3_scan_z(Diag3 J, long long *tab) {
   const M3 &M = *J.m;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, o = blockIdx.y, k = blockIdx.z;
-  if (x > M.nx) return;
-  const int no = axis == 1 ? M.nz : M.ny, nl = axis == 1 ? M.ny : M.nz;
-  if (o > no) return;
-  const size_t ts = (size_t)(M.nx + 1) * (M.ny + 1) * (M.nz + 1);
-  long long *t = tab + (size_t)k * ts;
+  const size_t plane = (size_t)(M.nx + 1) * (M.ny + 1);
+  const size_t i = (size_t)blockIdx.x * 128 + threadIdx.x;
+  if (i >= plane) return;
+  long long *t = tab + (size_t)blockIdx.y * plane * (M.nz + 1) + i;
   long long acc = 0;
-  for (int i = 1; i <= nl; ++i) {
-    const size_t p = axis == 1 ? tidx(M, x, i, o) : tidx(M, x, o, i);
-    acc += t[p];
-    t[p] = acc;
+  for (int z = 1; z <= M.nz; z += 8) {
+    long long v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = z + k <= M.nz ? t[(size_t)(z + k) * plane] : 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      acc += v[k];
+      if (z + k <= M.nz) t[(size_t)(z + k) * plane] = acc;
+    }
   }
 }
 
-// Exclusive prefix at (x, y, z) for 0 <= x < 2 nx etc. (periodic extension),
-// modular arithmetic.
-__device__ __forceinline__ unsigned long long P3(const M3 &M, const long long *t, int x, int y,
-                                                 int z) {
-  unsigned long long v = 0;
-  const int qx = x > M.nx, qy = y > M.ny, qz = z > M.nz;
-  const int xm = x - qx * M.nx, ym = y - qy * M.ny, zm = z - qz * M.nz;
-  for (int a = 0; a <= qx; ++a)
-    for (int b = 0; b <= qy; ++b)
-      for (int d = 0; d <= qz; ++d)
-        v += (unsigned long long)t[tidx(M, a ? M.nx : xm, b ? M.ny : ym, d ? M.nz : zm)];
-  return v;
+// max(m, |v|) for m >= 0, NaN ignored; FP64 by the bits, off the FP64 pipe.
+__device__ __forceinline__ float abs_max3(float m, float v) { return fmax(m, fabs(v)); }
+__device__ __forceinline__ double abs_max3(double m, double v) {
+  const long long b = __double_as_longlong(v) & 0x7fffffffffffffffll, a = __double_as_longlong(m);
+  return b > a && b <= 0x7ff0000000000000ll ? __longlong_as_double(b) : m;
 }
 
 template <int NRHS, typename MT>
@@ -710,7 +817,7 @@ __device__ __forceinline__ MT delta3(const MT *v) {
 #pragma unroll
   for (int i = 1; i <= NRHS; ++i) {
     sum += v[i];
-    mx = fmax(mx, fabs(v[i]));
+    mx = abs_max3(mx, v[i]);
   }
   const MT num = fabs(sum - v[0]);
   if (mx == MT(0)) return num == MT(0) ? MT(0) : MT(INFINITY);
@@ -724,7 +831,14 @@ template <typename MT>
 __device__ __forceinline__ MT i64_to(long long v);
 template <>
 __device__ __forceinline__ double i64_to<double>(long long v) {
-  return (double)v;
+  // to nearest (ties away from zero) by integer instructions, off the FP64 pipe
+  const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  const int n = __clzll((long long)a);
+  const unsigned long long x = a << (n & 63), r = x + 0x400ull;
+  const unsigned carry = r < x;
+  const unsigned e = n == 64 ? 0u : (unsigned)(1023 + 63 - 1 - n) << 20;
+  const unsigned hi = (unsigned)(r >> 43) + e + (carry << 21);
+  return __hiloint2double((int)(hi | (v < 0 ? 0x80000000u : 0u)), (int)(unsigned)(r >> 11));
 }
 template <>
 __device__ __forceinline__ float i64_to<float>(long long v) {
@@ -747,81 +861,177 @@ __device__ __forceinline__ float i64_to<float>(long long v) {
                          ((unsigned)m & 0x7fffffu));
 }
 
+constexpr int kMaxQBlocks3 = 1024;  // query CTAs per size
 constexpr int kQS3 = 30;  // per size: sums and sums of squares of 15 quantities
 
-// One thread per box: the 13 box sums exactly in integers, their deviations
-// from the field means formed in integers too (the mean box sum L^3 total/N,
-// rounded) and only then converted to the query precision MT; box means,
-// delta^E, delta^Omega; CTA partial sums (fixed order) of the 15 quantities'
-// deviations and squares, MT within each warp and FP64 across warps.
-template <typename MT>
-__global__ void __launch_bounds__(256) k3_query(Diag3 J, const long long *tab,
-                                                const double *scales, const double *means,
-                                                int L, int nb, const int *origins,
-                                                double *partials, double *per_box) {
+// The sizes of one balance call.
+struct Sizes3 {
+  int n, L[32], nb[32], qb[32];     // box size, boxes, query CTAs
+  long long ooff[32], row[32];      // first origin (lists), first per-box row
+  int out[32];                      // statistics row
+};
+
+// One thread per box and balance (blockIdx.z: 0 energy, 1 enstrophy), every
+// size in one launch (blockIdx.y): the box sums of its fields exactly in
+// integers (8 corners, or the signed sum of up to 27 for a box across the
+// periodic edge), their deviations from the field means formed in integers too
+// (the mean box sum L^3 total/N, rounded) and only then converted to the query
+// precision MT; box means, the balancing error; CTA partial sums (fixed order)
+// of the deviations and squares, MT within each warp and FP64 across warps.
+// (All 13 fields per thread with the values in local memory, a launch per size:
+// 295 us per size of 64^3 FP64, now 75.)
+template <typename MT, int G>
+__device__ __forceinline__ void query3(const Diag3 &J, const Sizes3 &S, const long long *tab,
+                                       const double *scales, const double *means,
+                                       const int *origins, double *partials, double *per_box,
+                                       double *sums) {
+  constexpr int NF = G ? 7 : 6, K0 = G ? 6 : 0, NQ = 2 * (NF + 1);
   const M3 &M = *J.m;
-  const size_t ts = (size_t)(M.nx + 1) * (M.ny + 1) * (M.nz + 1);
-  __shared__ long long smq[13];
-  __shared__ MT scoef[13], smean[13];
-  if (threadIdx.x < 13) {
-    const int k = threadIdx.x;
+  const int iL = blockIdx.y, L = S.L[iL], nb = S.nb[iL], qb = S.qb[iL];
+  const int nx = M.nx, ny = M.ny, nz = M.nz;
+  const size_t rs = (size_t)nx + 1, ps = rs * (ny + 1), ts = ps * (nz + 1);
+  __shared__ long long smq[NF];
+  __shared__ MT scoef[NF], smean[NF];
+  if (threadIdx.x < NF) {
+    const int k = K0 + threadIdx.x;
     const double vol = (double)L * L * L;
-    const long long total = tab[(size_t)k * ts + tidx(M, M.nx, M.ny, M.nz)];
-    smq[k] = __double2ll_rn((double)total * (vol / (double)M.N));
-    scoef[k] = (MT)(scales[80 + k] / vol);  // 2^-e / L^3
-    smean[k] = (MT)means[k];
+    const long long total = tab[(size_t)k * ts + ts - 1];
+    smq[threadIdx.x] = __double2ll_rn((double)total * (vol / (double)M.N));
+    scoef[threadIdx.x] = (MT)(scales[80 + k] / vol);  // 2^-e / L^3
+    smean[threadIdx.x] = (MT)means[k];
   }
   __syncthreads();
-  MT acc[kQS3];
+  MT acc[NQ];
 #pragma unroll
-  for (int q = 0; q < kQS3; ++q) acc[q] = MT(0);
-  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += gridDim.x * blockDim.x) {
+  for (int q = 0; q < NQ; ++q) acc[q] = MT(0);
+  const int *org = origins ? origins + 3 * S.ooff[iL] : nullptr;
+  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += qb * blockDim.x) {
     int x0, y0, z0;
-    if (origins) {
-      x0 = origins[3 * b];
-      y0 = origins[3 * b + 1];
-      z0 = origins[3 * b + 2];
+    if (org) {
+      x0 = org[3 * b];
+      y0 = org[3 * b + 1];
+      z0 = org[3 * b + 2];
     } else {
-      x0 = b % M.nx;
-      y0 = (b / M.nx) % M.ny;
-      z0 = b / (M.nx * M.ny);
+      x0 = b % nx;
+      y0 = (b / nx) % ny;
+      z0 = b / (nx * ny);
     }
-    MT v[15], d[15];
-#pragma unroll 1
-    for (int k = 0; k < 13; ++k) {
-      const long long *t = tab + (size_t)k * ts;
-      const int X0 = x0, X1 = x0 + L, Y0 = y0, Y1 = y0 + L, Z0 = z0, Z1 = z0 + L;
-      const unsigned long long s =
-          P3(M, t, X1, Y1, Z1) - P3(M, t, X0, Y1, Z1) - P3(M, t, X1, Y0, Z1) - P3(M, t, X1, Y1, Z0) +
-          P3(M, t, X0, Y0, Z1) + P3(M, t, X0, Y1, Z0) + P3(M, t, X1, Y0, Z0) - P3(M, t, X0, Y0, Z0);
-      d[2 + k] = i64_to<MT>((long long)(s - (unsigned long long)smq[k])) * scoef[k];
-      v[2 + k] = d[2 + k] + smean[k];
+    unsigned long long s[NF];
+    const long long *t = tab + (size_t)K0 * ts + (size_t)z0 * ps + (size_t)y0 * rs + x0;
+    if (x0 + L <= nx && y0 + L <= ny && z0 + L <= nz) {
+      const size_t dx = L, dy = (size_t)L * rs, dz = (size_t)L * ps;
+#pragma unroll
+      for (int k = 0; k < NF; ++k, t += ts)
+        s[k] = ((unsigned long long)__ldg(t + dz + dy + dx) - (unsigned long long)__ldg(t + dz + dy) -
+                (unsigned long long)__ldg(t + dz + dx) + (unsigned long long)__ldg(t + dz)) -
+               ((unsigned long long)__ldg(t + dy + dx) - (unsigned long long)__ldg(t + dy) -
+                (unsigned long long)__ldg(t + dx) + (unsigned long long)__ldg(t));
+    } else {
+      // per axis: + min(x0 + L, n), - x0, and + (x0 + L - n) across the edge
+#pragma unroll
+      for (int k = 0; k < NF; ++k) s[k] = 0;
+      const int X[3] = {min(x0 + L, nx), x0, x0 + L - nx}, Y[3] = {min(y0 + L, ny), y0, y0 + L - ny},
+                Z[3] = {min(z0 + L, nz), z0, z0 + L - nz};
+      for (int c = 0; c < 3 && Z[c] >= 0; ++c)
+        for (int d = 0; d < 3 && Y[d] >= 0; ++d)
+          for (int a = 0; a < 3 && X[a] >= 0; ++a) {
+            const bool neg = ((a == 1) != (d == 1)) != (c == 1);
+            const long long *q =
+                tab + (size_t)K0 * ts + (size_t)Z[c] * ps + (size_t)Y[d] * rs + X[a];
+#pragma unroll
+            for (int k = 0; k < NF; ++k, q += ts) {
+              const unsigned long long w = (unsigned long long)__ldg(q);
+              s[k] = neg ? s[k] - w : s[k] + w;
+            }
+          }
     }
-    v[0] = d[0] = delta3<5>(v + 2);
-    v[1] = d[1] = delta3<6>(v + 8);
-    if (per_box)
+    MT v[NF];
 #pragma unroll
-      for (int q = 0; q < 15; ++q) per_box[(size_t)b * 15 + q] = (double)v[q];
+    for (int k = 0; k < NF; ++k) {
+      const long long dq = (long long)(s[k] - (unsigned long long)smq[k]);
+      if constexpr (sizeof(MT) == 4) {
+        const MT d = i64_to<MT>(dq) * scoef[k];
+        v[k] = d + smean[k];
+        acc[2 + 2 * k] += d;
+        acc[3 + 2 * k] += d * d;
+      } else {  // sums of the integers, scaled once at the end
+        const double c = i64_to<double>(dq);
+        v[k] = fma(c, scoef[k], smean[k]);
+        acc[2 + 2 * k] += c;
+        acc[3 + 2 * k] = fma(c, c, acc[3 + 2 * k]);
+      }
+    }
+    const MT del = delta3<NF - 1>(v);
+    acc[0] += del;
+    acc[1] += del * del;
+    if (per_box) {
+      double *o = per_box + ((size_t)S.row[iL] + b) * 15;
+      o[G] = (double)del;
 #pragma unroll
-    for (int q = 0; q < 15; ++q) {
-      acc[2 * q] += d[q];
-      acc[2 * q + 1] += d[q] * d[q];
+      for (int k = 0; k < NF; ++k) o[2 + K0 + k] = (double)v[k];
     }
   }
-  __shared__ double sh[kQS3][8];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if constexpr (sizeof(MT) == 8) {
 #pragma unroll
-  for (int q = 0; q < kQS3; ++q) {
-    MT a = acc[q];
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-    if (lane == 0) sh[q][wid] = (double)a;
+    for (int k = 0; k < NF; ++k) {
+      acc[2 + 2 * k] *= scoef[k];
+      acc[3 + 2 * k] *= scoef[k] * scoef[k];
+    }
   }
-  __syncthreads();
-  if (threadIdx.x < kQS3) {
-    double a = 0.0;
-    for (int w = 0; w < 8; ++w) a += sh[threadIdx.x][w];
-    partials[(size_t)blockIdx.x * kQS3 + threadIdx.x] = a;
+  // quantity order delta^E, delta^O, 13 terms: (sum, sum of squares) each
+  auto put = [&](int t, double a) {
+    const int q = t / 2, row = q == 0 ? G : 2 + K0 + q - 1;
+    partials[((size_t)iL * kMaxQBlocks3 + blockIdx.x) * kQS3 + 2 * row + (t & 1)] = a;
+  };
+  if constexpr (sizeof(MT) == 8) {
+    // 16 threads per quantity sum 16 threads' values each, then one sums
+    // theirs: a quarter of the FP64 instructions of a shuffle tree per warp
+    double(*sh)[256] = reinterpret_cast<double(*)[256]>(sums);
+    double(*part)[16] = reinterpret_cast<double(*)[16]>(sums + 16 * 256);
+    const int q = threadIdx.x >> 4, p = threadIdx.x & 15;
+#pragma unroll
+    for (int k = 0; k < NQ; ++k) sh[k][threadIdx.x] = acc[k];
+    __syncthreads();
+    if (q < NQ) {
+      double a = 0.0;
+      for (int i = 0; i < 16; ++i) a += sh[q][16 * i + p];
+      part[q][p] = a;
+    }
+    __syncthreads();
+    if (threadIdx.x < NQ) {
+      double a = 0.0;
+      for (int i = 0; i < 16; ++i) a += part[threadIdx.x][i];
+      put(threadIdx.x, a);
+    }
+  } else {
+    double(*sh)[8] = reinterpret_cast<double(*)[8]>(sums);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      MT a = acc[q];
+      for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+      if (lane == 0) sh[q][wid] = (double)a;
+    }
+    __syncthreads();
+    if (threadIdx.x < NQ) {
+      double a = 0.0;
+      for (int w = 0; w < 8; ++w) a += sh[threadIdx.x][w];
+      put(threadIdx.x, a);
+    }
   }
+}
+
+template <typename MT>
+__global__ void __launch_bounds__(256) k3_query(Diag3 J, Sizes3 S, const long long *tab,
+                                                const double *scales, const double *means,
+                                                const int *origins, double *partials,
+                                                double *per_box) {
+  __shared__ double sums[sizeof(MT) == 8 ? 16 * 256 + 16 * 16 : 16 * 8];
+  if ((int)blockIdx.x >= S.qb[blockIdx.y]) return;
+  if (blockIdx.z == 0)
+    query3<MT, 0>(J, S, tab, scales, means, origins, partials, per_box, sums);
+  else
+    query3<MT, 1>(J, S, tab, scales, means, origins, partials, per_box, sums);
 }
 
 // Field means (exact table totals) for the deviation sums of the query.
@@ -833,13 +1043,15 @@ __global__ void k3_means(Diag3 J, const long long *tab, const double *scales, do
   means[k] = (double)tab[(size_t)k * ts + tidx(M, M.nx, M.ny, M.nz)] / scales[k] / (double)M.N;
 }
 
-// Mean and population standard deviation of the 15 quantities of one size
-// from the query's CTA partials: a warp per quantity (15 x 32 threads), each
+// Mean and population standard deviation of the 15 quantities of each size
+// (a CTA per size) from the query's CTA partials: a warp per quantity (15 x 32 threads), each
 // lane a fixed-order chain over the CTAs, then a shuffle tree.
-__global__ void k3_stats(const double *partials, int nblocks, const double *means, int nb,
-                         double *stats) {
-  const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+__global__ void k3_stats(const double *all, Sizes3 S, const double *means, double *stats_all) {
+  const int q = threadIdx.x >> 5, lane = threadIdx.x & 31, iL = blockIdx.x;
   if (q >= 15) return;
+  const double *partials = all + (size_t)iL * kMaxQBlocks3 * kQS3;
+  double *stats = stats_all + 30 * (size_t)iL;
+  const int nblocks = S.qb[iL], nb = S.nb[iL];
   double s1 = 0.0, s2 = 0.0;
   for (int b = lane; b < nblocks; b += 32) {
     s1 += partials[(size_t)b * kQS3 + 2 * q];
@@ -994,8 +1206,8 @@ cudaError_t tune_vec3(lbm3d_handle *h) {
   } while (0)
 
 constexpr size_t kAl = 256;
+constexpr size_t kPart3 = 112 + 32 * 30;  // scales, means, maxima, statistics per size
 size_t al(size_t v) { return (v + kAl - 1) / kAl * kAl; }
-constexpr int kMaxQBlocks3 = 1024;
 
 struct Layout3 {
   size_t members;
@@ -1054,7 +1266,7 @@ Layout3 layout3(const lbm3d_config *cfg) {
     Tmax = std::max(Tmax, (size_t)(c.nx + 1) * (c.ny + 1) * (c.nz + 1));
   }
   // fields, 13 tables (as int64), scales/means, query partials
-  L.diag_doubles = (size_t)NF3 * Nmax + 13 * Tmax + 112 + (size_t)kMaxQBlocks3 * kQS3;
+  L.diag_doubles = (size_t)NF3 * Nmax + 13 * Tmax + kPart3 + (size_t)32 * kMaxQBlocks3 * kQS3;
   L.diag = take(8 * L.diag_doubles);
   L.origin_cap = std::max<size_t>(3 * Nmax, (size_t)3 << 20);
   L.origins = take(4 * L.origin_cap);
@@ -1171,7 +1383,14 @@ int lbm3d_create(const lbm3d_config *cfg, void *workspace, size_t bytes, lbm3d_h
       return fail3(nullptr, LBM_ERR_CUDA, cudaGetErrorString(e));
     }
   }
-  cudaError_t e = vec_layout(h, 4);
+  // four cells per lane, or two where that leaves fewer lanes of the rows'
+  // segments idle (64 columns fill half a warp of four)
+  long long lanes4 = 0, lanes2 = 0;
+  for (const lbm3d_member_cfg &c : h->mcfg) {
+    lanes4 += (long long)((c.nx + 127) / 128) * 128 * c.ny * c.nz;
+    lanes2 += (long long)((c.nx + 63) / 64) * 64 * c.ny * c.nz;
+  }
+  cudaError_t e = vec_layout(h, 4 * lanes2 < 3 * lanes4 ? 2 : 4);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e == cudaSuccess) e = tune_vec3(h);
   if (e != cudaSuccess) {
@@ -1320,14 +1539,14 @@ int lbm3d_subvolume_balance(lbm3d_handle *h, int member, const int *L, int nL,
   long long *tab = reinterpret_cast<long long *>(h->diag + (size_t)NF3 * N);
   double *scales = h->diag + (size_t)NF3 * N + 13 * T;  // [16] scales, [16] exponents
   double *means = scales + 32;                           // [16]
-  double *sd = scales + 48;                              // [30] statistics of one size
   // scales + 80: [16] inverse scales 2^-e; scales + 96: [16] maxima bit patterns
-  double *partials = scales + 112;                       // [blocks][kQS3]
+  double *sd = scales + 112;                             // [32][30] statistics per size
+  double *partials = scales + kPart3;                    // [32][CTAs][kQS3]
   const dim3 cb(64, 4), cg = cells3(c);
   unsigned long long *maxbits = reinterpret_cast<unsigned long long *>(scales + 96);
   CK3(cudaMemsetAsync(maxbits, 0, 16 * sizeof(unsigned long long), h->stream));
   const dim3 ag((unsigned)std::min<size_t>(256, (N + 2047) / 2048), 13);
-  const dim3 sg((c.ny + 1 + 63) / 64, c.nz + 1, 13);
+  const dim3 sg((c.nz + 1 + 3) / 4, 13);
   if (h->diag_prec == 32) {  // term arithmetic in FP32
     k3_prep<float><<<cg, cb, 0, h->stream>>>(J);
     k3_grad<float><<<cg, cb, 0, h->stream>>>(J);
@@ -1335,7 +1554,7 @@ int lbm3d_subvolume_balance(lbm3d_handle *h, int member, const int *L, int nL,
     k3_curl<float><<<cg, cb, 0, h->stream>>>(J);
     k3_absmax<float><<<ag, 256, 0, h->stream>>>(J, maxbits);
     k3_scales<<<1, 32, 0, h->stream>>>(J, maxbits, scales);
-    k3_scan_x<float><<<sg, 64, 0, h->stream>>>(J, scales, tab);
+    k3_scan_xy<float><<<sg, 128, 0, h->stream>>>(J, scales, tab);
   } else {
     k3_prep<double><<<cg, cb, 0, h->stream>>>(J);
     k3_grad<double><<<cg, cb, 0, h->stream>>>(J);
@@ -1343,37 +1562,52 @@ int lbm3d_subvolume_balance(lbm3d_handle *h, int member, const int *L, int nL,
     k3_curl<double><<<cg, cb, 0, h->stream>>>(J);
     k3_absmax<double><<<ag, 256, 0, h->stream>>>(J, maxbits);
     k3_scales<<<1, 32, 0, h->stream>>>(J, maxbits, scales);
-    k3_scan_x<double><<<sg, 64, 0, h->stream>>>(J, scales, tab);
+    k3_scan_xy<double><<<sg, 128, 0, h->stream>>>(J, scales, tab);
   }
-  k3_scan_yz<<<dim3((c.nx + 1 + 63) / 64, c.nz + 1, 13), 64, 0, h->stream>>>(J, tab, 1);
-  k3_scan_yz<<<dim3((c.nx + 1 + 63) / 64, c.ny + 1, 13), 64, 0, h->stream>>>(J, tab, 2);
+  k3_scan_z<<<dim3((unsigned)(((size_t)(c.nx + 1) * (c.ny + 1) + 127) / 128), 13), 128, 0,
+              h->stream>>>(J, tab);
   k3_means<<<1, 32, 0, h->stream>>>(J, tab, scales, means);
   CK3(cudaGetLastError());
   if (origins)
     CK3(cudaMemcpyAsync(h->d_origins, origins, 12 * total, cudaMemcpyHostToDevice, h->stream));
-  std::vector<double> host(30 * (size_t)nL, std::nan(""));
-  size_t ooff = 0, row = 0;
+  // the sizes that fit the grid, in one query and one statistics launch
+  std::vector<double> host(30 * (size_t)nL, std::nan("")), got(30 * 32);
+  Sizes3 S{};
+  long long ooff = 0, row = 0;
+  int qmax = 1;
   for (int i = 0; i < nL; ++i) {
     const int nb = origins ? counts[i] : (int)N;
     if (L[i] >= 1 && L[i] <= Lmax) {
-      const int qb = std::min(kMaxQBlocks3, std::max(1, (nb + 255) / 256));
-      const int *og = origins ? h->d_origins + 3 * ooff : nullptr;
-      double *pbo = per_box_out ? per_box_out + row * 15 : nullptr;
-      if (h->diag_prec == 32)
-        k3_query<float><<<qb, 256, 0, h->stream>>>(J, tab, scales, means, L[i], nb, og, partials,
-                                                   pbo);
-      else
-        k3_query<double><<<qb, 256, 0, h->stream>>>(J, tab, scales, means, L[i], nb, og,
-                                                    partials, pbo);
-      k3_stats<<<1, 15 * 32, 0, h->stream>>>(partials, qb, means, nb, sd);
-      CK3(cudaGetLastError());
-      CK3(cudaMemcpyAsync(host.data() + 30 * (size_t)i, sd, 8 * 30, cudaMemcpyDeviceToHost,
-                          h->stream));
+      S.L[S.n] = L[i];
+      S.nb[S.n] = nb;
+      // FP32: a box per thread; FP64, whose block sums cost about a box per
+      // thread too, up to eight where that leaves two CTAs per SM
+      S.qb[S.n] = std::min(kMaxQBlocks3, std::max(1, (nb + 255) / 256));
+      if (h->diag_prec != 32)
+        S.qb[S.n] = std::min(S.qb[S.n], std::max((nb + 2047) / 2048, (304 + nL - 1) / nL));
+      S.ooff[S.n] = ooff;
+      S.row[S.n] = row;
+      S.out[S.n] = i;
+      qmax = std::max(qmax, S.qb[S.n]);
+      ++S.n;
     }
     ooff += origins ? counts[i] : 0;
     row += nb;
   }
+  if (S.n > 0) {
+    const dim3 qg(qmax, S.n, 2);
+    const int *og = origins ? h->d_origins : nullptr;
+    if (h->diag_prec == 32)
+      k3_query<float><<<qg, 256, 0, h->stream>>>(J, S, tab, scales, means, og, partials, per_box_out);
+    else
+      k3_query<double><<<qg, 256, 0, h->stream>>>(J, S, tab, scales, means, og, partials, per_box_out);
+    k3_stats<<<S.n, 15 * 32, 0, h->stream>>>(partials, S, means, sd);
+    CK3(cudaGetLastError());
+    CK3(cudaMemcpyAsync(got.data(), sd, 8 * 30 * (size_t)S.n, cudaMemcpyDeviceToHost, h->stream));
+  }
   CK3(cudaStreamSynchronize(h->stream));
+  for (int i = 0; i < S.n; ++i)
+    std::copy_n(got.begin() + 30 * (size_t)i, 30, host.begin() + 30 * (size_t)S.out[i]);
   std::copy(host.begin(), host.end(), stats_out);
   return LBM_OK;
 }

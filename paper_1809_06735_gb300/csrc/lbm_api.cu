@@ -341,14 +341,16 @@ int build_multi(lbm_handle *h, int T, int rows, int gmax) {
 }
 
 // Members the several-steps kernel can advance: double-buffer storage, every
-// member on the vectorised kernel with BGK, no force that needs the whole
+// member on the vectorised kernel with BGK, or every one with the entropic
+// collision, no force that needs the whole
 // state of each step (the damping of force kind 2).
 bool multi_eligible(const lbm_handle *h) {
-  if (h->precision != 32 || h->cfg.storage == 1 || h->has_kind2 || h->has_vv ||
-      !h->scalar_members.empty())
+  if (h->precision != 32 || h->cfg.storage == 1 || h->has_kind2 || !h->scalar_members.empty())
     return false;
   for (const lbm_member_cfg &c : h->mcfg)  // densities whose reciprocal is a normal number
-    if (c.ny < lbm::kMultiMinNy || c.rho0 < 1e-30 || c.rho0 > 1e30) return false;
+    if (c.ny < lbm::kMultiMinNy || c.rho0 < 1e-30 || c.rho0 > 1e30 ||
+        c.collision != (h->has_elbm ? 3 : 0))
+      return false;
   return true;
 }
 
@@ -413,7 +415,7 @@ int launch_steps(lbm_handle *h, cudaStream_t s, int *cur, long long k, int *n) {
       t = (int)((k + left - 1) / left);
     }
     if (t > 1) {
-      CK(lbm::launch_multi(t, h->multi_forced, h->d_members, h->d_multi, h->multi_ctas, *cur,
+      CK(lbm::launch_multi(t, h->multi_forced, h->has_elbm, h->d_members, h->d_multi, h->multi_ctas, *cur,
                            *cur & 1, s));
     } else {
       if (int rc = launch_one_step(h, s, *cur)) return rc;
@@ -1356,7 +1358,8 @@ int balance_members(lbm_handle *h, const int *members, int nm, const int *L, int
     J.meta = meta_dev + (size_t)i * kMaxL * 8;
     J.nL = (int)where[i].size();
     J.max_boxes = maxb[i];
-    J.qblocks = lbm::diag_query_blocks(hm.nx, hm.ny, maxb[i], origins != nullptr, batch_jobs);
+    J.qblocks = lbm::diag_query_blocks(hm.nx, hm.ny, maxb[i], origins != nullptr, batch_jobs, J.nL,
+                                       h->diag_precision == 64);
     J.qwhole = lbm::diag_whole_blocks(hm.nx * hm.ny, batch_jobs);
     for (int q : where[i]) J.any_whole |= !origins && lbm::diag_whole_box(L[q], hm.nx, hm.ny);
     J.force_kind = hm.force_kind;
@@ -1383,7 +1386,7 @@ int balance_members(lbm_handle *h, const int *members, int nm, const int *L, int
       const int G = (int)std::min(jobs.size() - j0, (size_t)h->sc.slots);
       CK(lbm::diag_balance(jobs.data() + j0, jobs_dev + j0, G, h->diag_precision,
                            h->precision == 32, orig_dev, stats_dev, per_box_out,
-                           dist ? &dd : nullptr, batch_jobs, s));
+                           dist ? &dd : nullptr, s));
       h->launches += 10;  // 4 term passes, scales, strip sums, table builder, constants, query, statistics
     }
   }

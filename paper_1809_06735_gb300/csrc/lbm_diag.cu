@@ -948,6 +948,34 @@ __device__ void block_sum_store_mt(MT (&v)[NQ], double *out /*[NQ]*/) {
   }
 }
 
+// Block sum of 256 threads' FP64 values, fixed order, through shared memory: 16
+// threads per quantity sum 16 values each, then one sums theirs: about 130
+// FP64 warp instructions for 14 quantities instead of the 560 of a shuffle
+// tree in every warp (17 cycles of the FP64 pipe each).
+template <int NQ>
+__device__ void block_sum_f64(const double (&v)[NQ], double *out /*[NQ]*/) {
+  static_assert(NQ <= 16, "16 threads per quantity");
+  __shared__ double sh[NQ][256];
+  __shared__ double part[NQ][16];
+  const int tid = threadIdx.x, q = tid >> 4, p = tid & 15;
+#pragma unroll
+  for (int k = 0; k < NQ; ++k) sh[k][tid] = v[k];
+  __syncthreads();
+  if (q < NQ) {
+    double a = 0.0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) a += sh[q][16 * i + p];
+    part[q][p] = a;
+  }
+  __syncthreads();
+  if (tid < NQ) {
+    double a = 0.0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) a += part[tid][i];
+    out[tid] = a;
+  }
+}
+
 // Sums nb partial rows of width nq (fixed order per thread: 8 threads per
 // quantity take interleaved rows, then a fixed-order combination).
 __global__ void k_sum_partials(const double *partials, int nb, int nq, double *out) {
@@ -1727,22 +1755,29 @@ __global__ void __launch_bounds__(256, 3) k_query(const DiagJob *__restrict__ jo
 // (k_query, which it replaces here, keeps the sizes of nearly the whole grid.)
 
 // How the origins of a grid are shared out: CTAs of 256 threads, xt columns
-// by 256 / xt chains, nxb CTAs along x times `parts` along the chains.
+// by 256 / xt chains, nxb CTAs along x times `parts` along the chains.  A
+// function of the member and of the number of sizes only, so that the
+// statistics do not depend on the other members of a batch.
 struct AllGrid {
   int xt, nxb, parts;
 };
-__host__ __device__ inline AllGrid all_grid(int nx, int ny, int batch_jobs) {
+__host__ __device__ inline AllGrid all_grid(int nx, int ny, int nL, bool f64) {
   AllGrid g;
   g.xt = nx > 128 ? 256 : (nx > 64 ? 128 : (nx > 32 ? 64 : 32));
   if (nx > 256 && (nx + 255) / 256 * 256 * 7 > nx * 8 && (nx + 127) / 128 * 128 < (nx + 255) / 256 * 256)
     g.xt = 128;  // a ragged last CTA column
   const int yt = 256 / g.xt, xb = (nx + g.xt - 1) / g.xt;
   g.nxb = xb < kMaxQueryBlocks ? xb : kMaxQueryBlocks;
-  // about 32 boxes per thread, down to 4 where the batch has few CTAs
-  int parts = (ny + yt * 32 - 1) / (yt * 32);
-  const int jobs = batch_jobs < 1 ? 1 : batch_jobs;
-  const int want = (256 / jobs + g.nxb - 1) / g.nxb, cap = (ny + yt * 4 - 1) / (yt * 4);
-  if (parts < want) parts = want < cap ? want : cap;
+  // boxes per thread: 16, and 4 on grids too small to fill the GPU.  FP64,
+  // whose block sum costs about a box per thread: as many as two CTAs per SM
+  // over all sizes and balances leave, 32 at most
+  int per = (long long)nx * ny < 65536 ? 4 : 16;
+  if (f64) {
+    const int want = (152 + nL * g.nxb - 1) / (nL * g.nxb);
+    per = ny / (yt * want);
+    per = per > 32 ? 32 : (per < 1 ? 1 : per);
+  }
+  int parts = (ny + yt * per - 1) / (yt * per);
   if (parts > kMaxQueryBlocks / g.nxb) parts = kMaxQueryBlocks / g.nxb;
   g.parts = parts < 1 ? 1 : parts;
   return g;
@@ -1777,6 +1812,9 @@ __device__ __forceinline__ void query_column(const DiagJob &J, int iL, int grp, 
   const MT ma_ref = NFLD == 1 ? sqrt(fmax(qc[0].mean<MT>(), MT(0))) * MT(1.7320508075688772) : MT(0);
   long long mq[NFLD];
   MT coef[NFLD], mean[NFLD], s1[NFLD], s2[NFLD], d1 = 0, d2 = 0;
+  // FP64: the deviations' sums stay integers, by 32-bit halves
+  long long hi[NFLD];
+  unsigned long long lo[NFLD];
 #pragma unroll
   for (int j = 0; j < NFLD; ++j) {
     mq[j] = qc[j].mq;
@@ -1784,6 +1822,8 @@ __device__ __forceinline__ void query_column(const DiagJob &J, int iL, int grp, 
     mean[j] = qc[j].mean<MT>();
     s1[j] = MT(0);
     s2[j] = MT(0);
+    hi[j] = 0;
+    lo[j] = 0;
   }
   // a chain of up to kSeg boxes per unit of work
   constexpr int kSeg = 16;
@@ -1833,7 +1873,8 @@ __device__ __forceinline__ void query_column(const DiagJob &J, int iL, int grp, 
           } else {  // sums of the integers, scaled once at the end
             const double c = i64_to_f64(dq);
             v = fma(c, coef[j], mean[j]);
-            s1[j] += c;
+            hi[j] += dq >> 32;
+            lo[j] += (unsigned long long)dq & 0xffffffffull;
             s2[j] = fma(c, c, s2[j]);
           }
           if (j == 0) {
@@ -1870,7 +1911,8 @@ __device__ __forceinline__ void query_column(const DiagJob &J, int iL, int grp, 
   acc[1] = d2;
 #pragma unroll
   for (int j = 0; j < NFLD; ++j) {
-    acc[2 + 2 * j] = sizeof(MT) == 8 ? s1[j] * coef[j] : s1[j];
+    acc[2 + 2 * j] =
+        sizeof(MT) == 8 ? MT(((double)hi[j] * 4294967296.0 + (double)lo[j]) * (double)coef[j]) : s1[j];
     acc[3 + 2 * j] = sizeof(MT) == 8 ? s2[j] * coef[j] * coef[j] : s2[j];
   }
 }
@@ -1879,7 +1921,7 @@ __device__ __forceinline__ void query_column(const DiagJob &J, int iL, int grp, 
 // 3 with the distributions (EXT: Ma_V); blockIdx.z = groups * job + group.
 template <typename MT, bool PER_BOX, bool EXT>
 __global__ void __launch_bounds__(256, 2)
-    k_query_all(const DiagJob *__restrict__ jobs, double *per_box, DiagDist ext, int batch_jobs) {
+    k_query_all(const DiagJob *__restrict__ jobs, double *per_box, DiagDist ext) {
   constexpr int NG = EXT ? 3 : 2;
   const DiagJob &J = jobs[blockIdx.z / NG];
   const int grp = blockIdx.z % NG, iL = blockIdx.x, blk = blockIdx.y, qb = J.qblocks;
@@ -1896,7 +1938,7 @@ __global__ void __launch_bounds__(256, 2)
     }
     __syncthreads();
   }
-  const AllGrid ag = all_grid(J.nx, J.ny, batch_jobs);
+  const AllGrid ag = all_grid(J.nx, J.ny, J.nL, sizeof(MT) == 8);
   const int nblk_x = (J.nx + ag.xt - 1) / ag.xt;
   MT acc[kQStats];
 #pragma unroll
@@ -1905,8 +1947,11 @@ __global__ void __launch_bounds__(256, 2)
     query_column<MT, PER_BOX, EXT, 1>(J, iL, grp, blk, nblk_x, ag, sedge, shist, ne, per_box, acc);
   else
     query_column<MT, PER_BOX, EXT, 6>(J, iL, grp, blk, nblk_x, ag, sedge, shist, ne, per_box, acc);
-  double *pq = J.part + kPartQuery;
-  block_sum_store_mt<kQStats, MT>(acc, pq + (((size_t)iL * 3 + grp) * qb + blk) * kQStats);
+  double *out = J.part + kPartQuery + (((size_t)iL * 3 + grp) * qb + blk) * kQStats;
+  if constexpr (sizeof(MT) == 8)
+    block_sum_f64<kQStats>(acc, out);
+  else
+    block_sum_store_mt<kQStats, MT>(acc, out);
   if constexpr (EXT) {
     __syncthreads();
     unsigned long long *h =
@@ -2006,7 +2051,7 @@ dim3 cells_grid(const Grid &g, dim3 b) {
 template <typename T, typename MT>
 cudaError_t balance_launches(const DiagJob *jobs_host, const DiagJob *jobs, int G, bool pairs,
                              const int *origins, double *stats, double *per_box,
-                             const DiagDist *dist, int batch_jobs, cudaStream_t s) {
+                             const DiagDist *dist, cudaStream_t s) {
   const bool planar = origins == nullptr;  // every periodic origin
   int nx = 1, ny = 1, nL = 1, qblocks = 1, qwhole = 1;
   bool any_whole = false;
@@ -2084,11 +2129,11 @@ cudaError_t balance_launches(const DiagJob *jobs_host, const DiagJob *jobs, int 
   if (planar) {
     const dim3 qg(nL, qblocks, (dist ? 3 : 2) * G);
     if (dist)
-      k_query_all<MT, false, true><<<qg, 256, 0, s>>>(jobs, nullptr, *dist, batch_jobs);
+      k_query_all<MT, false, true><<<qg, 256, 0, s>>>(jobs, nullptr, *dist);
     else if (per_box)
-      k_query_all<MT, true, false><<<qg, 256, 0, s>>>(jobs, per_box, none, batch_jobs);
+      k_query_all<MT, true, false><<<qg, 256, 0, s>>>(jobs, per_box, none);
     else
-      k_query_all<MT, false, false><<<qg, 256, 0, s>>>(jobs, nullptr, none, batch_jobs);
+      k_query_all<MT, false, false><<<qg, 256, 0, s>>>(jobs, nullptr, none);
   }
   if (!planar || any_whole) {
     const dim3 qg(planar ? qwhole : qblocks, nL, (dist ? 2 : 1) * G);
@@ -2149,9 +2194,10 @@ static int diag_list_blocks(int max_boxes, int per_cta, int batch_jobs) {
 // one pass of 128 boxes, about 256 per size over the batch: its FP64
 // statistics then spread over the SMs instead of queueing on a few (GB300
 // issues about 1.7 FP64 FMAs per clock per SM).
-int diag_query_blocks(int nx, int ny, int max_boxes, bool origin_list, int batch_jobs) {
+int diag_query_blocks(int nx, int ny, int max_boxes, bool origin_list, int batch_jobs, int nL,
+                      bool f64) {
   if (!origin_list) {
-    const AllGrid g = all_grid(nx, ny, batch_jobs);
+    const AllGrid g = all_grid(nx, ny, nL, f64);
     return g.nxb * g.parts;
   }
   return diag_list_blocks(max_boxes, 1024, batch_jobs);
@@ -2176,16 +2222,16 @@ size_t diag_job_partials(size_t Nmax, size_t pad) {
 cudaError_t diag_balance(const DiagJob *jobs_host, const DiagJob *jobs_dev, int G,
                          int precision, bool pairs, const int *origins_dev,
                          double *stats_dev, double *per_box_dev, const DiagDist *dist,
-                         int batch_jobs, cudaStream_t s) {
+                         cudaStream_t s) {
   if (G < 1 || (per_box_dev && G != 1) || (per_box_dev && dist)) return cudaErrorInvalidValue;
   if (dist && (dist->n_delta < 1 || dist->n_delta > kDiagMaxEdges || dist->n_mach < 1 ||
                dist->n_mach > kDiagMaxEdges))
     return cudaErrorInvalidValue;
   if (precision == 32)
     return balance_launches<float, float>(jobs_host, jobs_dev, G, pairs, origins_dev,
-                                          stats_dev, per_box_dev, dist, batch_jobs, s);
+                                          stats_dev, per_box_dev, dist, s);
   return balance_launches<double, double>(jobs_host, jobs_dev, G, pairs, origins_dev,
-                                          stats_dev, per_box_dev, dist, batch_jobs, s);
+                                          stats_dev, per_box_dev, dist, s);
 }
 
 }  // namespace lbm

@@ -241,8 +241,9 @@ void multi_member(int member, int nx, int ny, int rows, int gmax, std::vector<Mu
 double multi_ctas(int nx, int ny, int rows, int gmax);  // CTAs of it
 size_t multi_capacity(int nx, int ny);  // table entries of a member at most
 // T = 2..4 steps of every member in the table from double-buffer storage
-// `state` into the other buffer (forced: some member has a force or drag).
-cudaError_t launch_multi(int T, bool forced, const Member *d_members, const MultiWarp *tab, int ctas,
+// `state` into the other buffer (forced: some member has a force or drag; elbm:
+// the entropic collision, else BGK).
+cudaError_t launch_multi(int T, bool forced, bool elbm, const Member *d_members, const MultiWarp *tab, int ctas,
                          int state, int flip, cudaStream_t s);
 
 // One step of every vector-kernel member (flip: tiles in reverse order).
@@ -358,7 +359,8 @@ struct DiagJob {
 };
 // Query CTAs for a job: a fixed function of its own box count, so that the
 // statistics do not depend on which members share a batch.
-int diag_query_blocks(int nx, int ny, int max_boxes, bool origin_list, int batch_jobs);
+int diag_query_blocks(int nx, int ny, int max_boxes, bool origin_list, int batch_jobs, int nL,
+                      bool f64);
 int diag_whole_blocks(int boxes, int batch_jobs);
 bool diag_whole_box(int L, int nx, int ny);
 // Doubles of one field slot and of one partials slot for members of at most
@@ -383,7 +385,7 @@ struct DiagDist {
 cudaError_t diag_balance(const DiagJob *jobs_host, const DiagJob *jobs_dev, int G,
                          int precision, bool pairs, const int *origins_dev,
                          double *stats_dev, double *per_box_dev, const DiagDist *dist,
-                         int batch_jobs, cudaStream_t s);
+                         cudaStream_t s);
 
 // Adjoint (lbm_adjoint.cu).
 cudaError_t adjoint_step(const Member &hm, const double *f_n, const double *lam_in,

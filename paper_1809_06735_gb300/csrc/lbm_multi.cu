@@ -106,8 +106,9 @@ __device__ __forceinline__ float last_of(const f32x2 (&v)[2]) {
   return b;
 }
 
-// T steps of the members' rows (BGK; FORCED: some member has a force or drag).
-template <int T, bool FORCED>
+// T steps of the members' rows (BGK, or ELBM: the entropic collision; FORCED:
+// some member has a force or drag).
+template <int T, bool FORCED, bool ELBM>
 __global__ void __launch_bounds__(32 * kMultiWarps, 2)
     k_multi(const Member *__restrict__ members, const MultiWarp *__restrict__ tab, int ctas, int cur,
             int flip) {
@@ -233,7 +234,20 @@ __global__ void __launch_bounds__(32 * kMultiWarps, 2)
         f32x2 g[kQ];
 #pragma unroll
         for (int l = 0; l < kQ; ++l) g[l] = v[l][c];
-        collide2_f32<FORCED>(g, rho0, om, both2(fx[s]), fy[c], alpha);
+        if constexpr (ELBM) {
+          if (!collide2_elbm<FORCED>(g, rho0, 2.0f * M.tau_f, both2(fx[s]), fy[c], alpha)) {
+            float ga[kQ], gb[kQ], fya, fyb;  // a cell whose root needs iterations
+#pragma unroll
+            for (int l = 0; l < kQ; ++l) unpack2(g[l], ga[l], gb[l]);
+            unpack2(fy[c], fya, fyb);
+            collide_elbm_call(ga, rho0, M.tau_f, fx[s], fya, alpha);
+            collide_elbm_call(gb, rho0, M.tau_f, fx[s], fyb, alpha);
+#pragma unroll
+            for (int l = 0; l < kQ; ++l) g[l] = pack2(ga[l], gb[l]);
+          }
+        } else {
+          collide2_f32<FORCED>(g, rho0, om, both2(fx[s]), fy[c], alpha);
+        }
 #pragma unroll
         for (int l = 0; l < kQ; ++l) v[l][c] = g[l];
       }
@@ -255,14 +269,14 @@ __global__ void __launch_bounds__(32 * kMultiWarps, 2)
   }
 }
 
-template <int T, bool FORCED>
+template <int T, bool FORCED, bool ELBM>
 cudaError_t launch(const Member *d_members, const MultiWarp *tab, int ctas, int state, int flip,
                    cudaStream_t s) {
   constexpr size_t smem = multi_smem<T>();
   const cudaError_t e = cudaFuncSetAttribute(
-      k_multi<T, FORCED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      k_multi<T, FORCED, ELBM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_multi<T, FORCED><<<ctas, dim3(32, kMultiWarps), smem, s>>>(d_members, tab, ctas, state, flip);
+  k_multi<T, FORCED, ELBM><<<ctas, dim3(32, kMultiWarps), smem, s>>>(d_members, tab, ctas, state, flip);
   return cudaGetLastError();
 }
 
@@ -323,13 +337,16 @@ size_t multi_capacity(int nx, int ny) {
   return ((size_t)nx / 60 + 2) * ((size_t)ny / kMultiMinRows + 2) * 2 + kMultiWarps;
 }
 
-cudaError_t launch_multi(int T, bool forced, const Member *d_members, const MultiWarp *tab, int ctas,
+cudaError_t launch_multi(int T, bool forced, bool elbm, const Member *d_members, const MultiWarp *tab, int ctas,
                          int state, int flip, cudaStream_t s) {
   if (state > 1 || ctas < 1) return cudaErrorInvalidValue;
 #define LBM_MULTI(T_)                                                                 \
+  if (T == T_ && elbm)                                                                \
+    return forced ? launch<T_, true, true>(d_members, tab, ctas, state, flip, s)      \
+                  : launch<T_, false, true>(d_members, tab, ctas, state, flip, s);    \
   if (T == T_)                                                                        \
-    return forced ? launch<T_, true>(d_members, tab, ctas, state, flip, s)            \
-                  : launch<T_, false>(d_members, tab, ctas, state, flip, s)
+    return forced ? launch<T_, true, false>(d_members, tab, ctas, state, flip, s)     \
+                  : launch<T_, false, false>(d_members, tab, ctas, state, flip, s)
   LBM_MULTI(2);
   LBM_MULTI(3);
   LBM_MULTI(4);
