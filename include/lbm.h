@@ -230,7 +230,7 @@ int lbm_set_launch(lbm_handle *h, int warps, int rows, int grid, int proj_rows);
  * steps of a call that do not fill a launch, and the steps that record a
  * snapshot, run as shorter launches.  Results do not depend on it.
  * LBM_ERR_ARG for steps > 1 unless every member is FP32 with nx % 4 == 0,
- * ny >= 4, collision 0, force kind 0 or 1 and rho0 in [1e-30, 1e30], in
+ * ny >= 4, collision 0 (or 3 in all), force kind 0 or 1 and rho0 in [1e-30, 1e30], in
  * double-buffer storage (storage 2, or 0 where the tuner chose it); the
  * previous setting is then kept. */
 int lbm_set_steps_per_launch(lbm_handle *h, int steps, int rows);

@@ -897,6 +897,10 @@ int lbm_create(const lbm_config *cfg, void *workspace, size_t bytes, lbm_handle 
     return cleanup(fail(nullptr, LBM_ERR_CUDA, std::string("create: ") + cudaGetErrorString(e)));
   h->cur = cfg->storage == 1 ? 2 : 0;
   h->lc.paper_force = h->has_elbm ? 3 : (h->has_vv ? 2 : (h->has_kind2 ? 1 : 0));
+  if (h->has_elbm)
+    for (const lbm_member_cfg &c : h->mcfg)
+      if (c.collision == 3 && (c.alpha != 0.0 || c.force_kind == 2 || (c.force_kind == 1 && c.F0 != 0.0)))
+        h->lc.paper_force = 4;
   for (const lbm_member_cfg &c : h->mcfg)
     h->multi_forced |= c.alpha != 0.0 || (c.force_kind != 0 && c.F0 != 0.0);
   {

@@ -219,7 +219,8 @@ struct LaunchCfg {
   int paper_force;    // kernel variant: 0 plain; 1 some member has force kind 2
                       // (BGK collisions); 2 some member has a variable-viscosity
                       // collision (any force); 3 some member has the entropic
-                      // collision (with any other collision and force)
+                      // collision (with any other collision), those members
+                      // without force and drag; 4 the same with any force
   int proj_rows;      // rows per thread of the FP32 four-cell projection (force
                       // kind 2): a block covers 128 x 8 proj_rows cells
 };

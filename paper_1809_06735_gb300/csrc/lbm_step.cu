@@ -171,17 +171,42 @@ __device__ __forceinline__ void step_tile(const Member *__restrict__ members, co
           fyc[c] = fy[c];
         }
       }
+      bool two_done = false;
+      if constexpr (PF >= 3) {
+        if (M.collision == 3) {  // two cells per instruction
+          two_done = true;
+          const bool normal = rho0 > 1e-30f && rho0 < 1e30f;
+#pragma unroll
+          for (int c = 0; c < 4; c += 2) {
+            f32x2 g[kQ];
+#pragma unroll
+            for (int l = 0; l < kQ; ++l) g[l] = pack2(v[l][c], v[l][c + 1]);
+            if (normal &&
+                collide2_elbm<PF == 4>(g, rho0, 2.0f * M.tau_f, pack2(fxc[c], fxc[c + 1]),
+                                       pack2(fyc[c], fyc[c + 1]), alpha)) {
+#pragma unroll
+              for (int l = 0; l < kQ; ++l) unpack2(g[l], v[l][c], v[l][c + 1]);
+            } else {  // a cell whose root needs iterations
+#pragma unroll
+              for (int i = c; i < c + 2; ++i) {
+                float a[kQ];
+#pragma unroll
+                for (int l = 0; l < kQ; ++l) a[l] = v[l][i];
+                collide_elbm_call(a, rho0, M.tau_f, fxc[i], fyc[i], alpha);
+#pragma unroll
+                for (int l = 0; l < kQ; ++l) v[l][i] = a[l];
+              }
+            }
+          }
+        }
+      }
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
+        if (two_done) break;
         float g[kQ];
 #pragma unroll
         for (int l = 0; l < kQ; ++l) g[l] = v[l][c];
-        if constexpr (PF == 3) {
-          if (M.collision == 3)
-            collide_elbm<float>(g, rho0, M.tau_f, fxc[c], fyc[c], alpha);
-          else
-            collide_f32<true>(g, rho0, om, fxc[c], fyc[c], alpha, M.collision, M.tau_f, M.Cs_f);
-        } else if constexpr (PF == 2)
+        if constexpr (PF >= 2)
           collide_f32<true>(g, rho0, om, fxc[c], fyc[c], alpha, M.collision, M.tau_f, M.Cs_f);
         else
           collide_f32(g, rho0, om, fxc[c], fyc[c], alpha);
@@ -243,7 +268,7 @@ __device__ __forceinline__ void step_tile(const Member *__restrict__ members, co
 }
 
 template <int ROWS, int MODE, int PF, bool SNAP = false>
-__global__ void __launch_bounds__(256, PF == 1 || PF == 2 ? 3 : (PF == 3 || SNAP ? 2 : 1)) k_step_f32_vec(const Member *__restrict__ members,
+__global__ void __launch_bounds__(256, PF == 1 || PF == 2 ? 3 : (PF >= 3 || SNAP ? 2 : 1)) k_step_f32_vec(const Member *__restrict__ members,
                                                       const Tile *__restrict__ tiles,
                                                       int ntiles, int cur, int flip, int snap_slot) {
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
@@ -269,11 +294,14 @@ static void launch_vec_rows(const Member *d_members, const Tile *d_tiles, int nt
 
 // pf: 0 no member with force kind 2 or a variable viscosity; 1 force kind 2
 // with the BGK collision only; 2 variable-viscosity collisions (any force);
-// 3 some member with the entropic collision (any other collision, any force)
+// 3 some member with the entropic collision (any other collision), no force
+// or drag on those members, 4 the same with any force
 template <int ROWS>
 static void launch_vec_rows(const Member *d_members, const Tile *d_tiles, int ntiles, int state,
                             int flip, int grid, dim3 block, int pf, cudaStream_t s) {
-  if (pf == 3)
+  if (pf == 4)
+    launch_vec_rows<ROWS, 4>(d_members, d_tiles, ntiles, state, flip, grid, block, s);
+  else if (pf == 3)
     launch_vec_rows<ROWS, 3>(d_members, d_tiles, ntiles, state, flip, grid, block, s);
   else if (pf == 2)
     launch_vec_rows<ROWS, 2>(d_members, d_tiles, ntiles, state, flip, grid, block, s);

@@ -54,6 +54,28 @@ def test_equals_single_steps(P, T, rows, forced):
     b.close()
 
 
+@pytest.mark.parametrize("forced", [False, True])
+@pytest.mark.parametrize("T,rows", [(2, 8), (3, 27), (4, 100)])
+def test_entropic_equals_single_steps(P, T, rows, forced):
+    """The entropic collision likewise, with members whose cells are close to
+    equilibrium, far from it (the root iterated) and at rest."""
+    kw = dict(force_kind=1, kf=2, F0=1e-5, alpha=1e-4) if forced else {}
+    members = [P.Member(nx, ny, 0.52, collision=3, **kw) for nx, ny in ((132, 70), (256, 65), (8, 8))]
+    a, b = _pair(P, members, T, rows)
+    far = li.random_populations(256, 65, seed=4, rel_noise=0.04)
+    rest = np.tile(li.random_populations(1, 1, seed=1, rel_noise=0.0), (1, 8, 8))
+    for lat in (a, b):
+        lat.set_populations(1, far)
+        lat.set_populations(2, rest)
+    for n in (1, 2, 3, 5):
+        a.step(n)
+        b.step(n)
+        for m in range(3):
+            assert np.array_equal(a.get_populations_host(m), b.get_populations_host(m)), (n, m)
+    a.close()
+    b.close()
+
+
 @pytest.mark.parametrize("graph", [0, 5, 6])
 def test_snapshots_and_graphs(P, graph):
     """Snapshot steps, graph replay and remainders around them."""
