@@ -21,8 +21,9 @@
 // whose adjoint uses D^T = -D (antisymmetric periodic eq. (18) stencil).
 // All arithmetic is FP64; reductions are block-deterministic.
 #include <algorithm>
+#include <cmath>
 
-#include "lbm_internal.cuh"
+#include "lbm_collide.cuh"
 
 namespace lbm {
 
@@ -36,6 +37,8 @@ struct AGrid {
   int nx, ny, kf, force;
   double nu, alpha, tau, omega, F0;
   const double *fxt, *fyt;  // F_ext tables (F0 included)
+  FixedBgk fixed;           // constants of the fixed-point forms
+  long long w1, keep;       // (omega - 1) 2^63, (1 - omega) 2^63
 };
 
 __device__ __forceinline__ int wrapn(int i, int n) {
@@ -281,6 +284,167 @@ __device__ __forceinline__ MuMoments mu_moments(const double (&mu)[kQ]) {
   return M;
 }
 
+// One cell of the adjoint of a step in FP64: lambda_out from the state fl, the
+// pulled adjoint mu and the objective's (d_rho, d_jx, d_jy); t and (bx, by)
+// receive sum mu (f - feq) and the adjoint of m'.
+__device__ __forceinline__ void adjoint_cell_f64(const AGrid &g, int x, int y,
+                                                 const double (&fl)[kQ], const double (&mu)[kQ],
+                                                 double d_rho, double d_jx, double d_jy,
+                                                 double (&out)[kQ], double &t, double &bx,
+                                                 double &by) {
+  // moments from the opposite pairs' sums and differences
+  const double d57 = fl[5] - fl[7], d68 = fl[6] - fl[8];
+  const double rho = fl[0] + ((fl[1] + fl[3]) + (fl[2] + fl[4])) + ((fl[5] + fl[7]) + (fl[6] + fl[8]));
+  const double jx = (fl[1] - fl[3]) + (d57 - d68), jy = (fl[2] - fl[4]) + (d57 + d68);
+  const double ir = 1.0 / rho;
+  const double mpx = (1.0 - g.alpha) * jx + g.fxt[y];
+  const double mpy = (1.0 - g.alpha) * jy + g.fyt[x];
+  const MuMoments M = mu_moments(mu);
+  // equilibrium at (rho, j): q_a = m.M2.m, p_a = M2.m
+  const double pax = M.mxx * jx + M.mxy * jy, pay = M.mxy * jx + M.myy * jy;
+  const double qa = (4.5 * (jx * pax + jy * pay) - 1.5 * (jx * jx + jy * jy) * M.m0) * ir;
+  // at (rho, m')
+  const double pbx = M.mxx * mpx + M.mxy * mpy, pby = M.mxy * mpx + M.myy * mpy;
+  const double qb = (4.5 * (mpx * pbx + mpy * pby) - 1.5 * (mpx * mpx + mpy * mpy) * M.m0) * ir;
+  const double w1 = g.omega - 1.0;
+  const double Sa_rho = M.m0 - qa * ir, Sb_rho = M.m0 - qb * ir;
+  // S_a = 3 M_a + 9 p_a / rho - 3 m_a M0 / rho with 9 / rho and 3 M0 / rho
+  // formed once
+  const double ir9 = 9.0 * ir, k0 = 3.0 * M.m0 * ir, mx3 = 3.0 * M.mx, my3 = 3.0 * M.my;
+  const double Sa_x = fma(ir9, pax, fma(-jx, k0, mx3));
+  const double Sa_y = fma(ir9, pay, fma(-jy, k0, my3));
+  bx = fma(ir9, pbx, fma(-mpx, k0, mx3));
+  by = fma(ir9, pby, fma(-mpy, k0, my3));
+  const double Arho = w1 * Sa_rho + Sb_rho + d_rho;
+  const double Ajx = w1 * Sa_x + (1.0 - g.alpha) * bx + d_jx;
+  const double Ajy = w1 * Sa_y + (1.0 - g.alpha) * by + d_jy;
+  // sum mu (f - feq(rho, j)) for dJ/dtau
+  double muf = 0.0;
+#pragma unroll
+  for (int l = 0; l < kQ; ++l) muf += mu[l] * fl[l];
+  t = muf - (rho * M.m0 + 3.0 * (jx * M.mx + jy * M.my) + qa);
+  const double keep = 1.0 - g.omega;
+  // lambda_l = keep mu_l + Arho + c_l . A, by opposite pairs (c . A once
+  // per pair; a product by c = 0 still costs an FMA under IEEE arithmetic)
+  const double cA[4] = {Ajx, Ajy, Ajx + Ajy, Ajy - Ajx};  // c of 1, 2, 5, 6
+  out[0] = fma(keep, mu[0], Arho);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int l = k < 2 ? 1 + k : 5 + (k - 2), m = opposite(l);
+    out[l] = fma(keep, mu[l], Arho + cA[k]);
+    out[m] = fma(keep, mu[m], Arho - cA[k]);
+  }
+}
+
+// The same in 64-bit fixed point (collide_fixed's reasons and range; 256^2:
+// 13.6 us per adjoint step against 22.8).  The populations of the adjoint have no
+// scale of their own: they are taken in units of 2^-53 of the exponent of the
+// largest one of the warp's 32 cells (emax), sums and products with three to
+// five more bits, so that the warp's largest values keep FP64's 53 bits.  With u = j / rho and v = m' / rho the terms are
+//   S_rho = M0 - Q(u), S = 3 M1 + 9 M2.u - 3 u M0,
+//   Q(u) = 4.5 u.M2.u - 1.5 |u|^2 M0,
+// (36 M are exact integer sums of the mu), sum mu feq = rho (M0 + 3 u.M1 +
+// Q(u)).  Returns false where the cell needs the FP64 form.
+__device__ __forceinline__ long long adj_fixed(double v, int emax) {
+  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+  const int e = (int)((hi >> 20) & 0x7ffu), r = emax - e;
+  const unsigned long long m =
+      (((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo) << 2;  // 2 x 2^53 .. 2^54
+  // to nearest, ties to even: ties are frequent here (r = 2 drops one bit), and
+  // rounding them one way would bias every step's adjoint
+  const unsigned long long h = m >> (r & 63), odd = (h >> 1) & 1ull;
+  const unsigned long long sticky = m & ((1ull << (r & 63)) - 1);
+  const long long q = r > 57 || e == 0 ? 0 : (long long)((h + (sticky ? 1ull : odd)) >> 1);
+  return (int)hi < 0 ? -q : q;
+}
+// v 2^(emax - 1023 - 53) to double, to nearest even
+__device__ __forceinline__ double adj_double(long long v, int emax) {
+  const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  const int n = __clzll((long long)a);
+  const unsigned long long x = a << (n & 63), r = x + 0x3ffull + ((x >> 11) & 1ull);
+  const unsigned carry = r < x;
+  const unsigned e = (unsigned)(emax - 53 + 63 - 1 - n) << 20;
+  const unsigned hi = n == 64 ? 0u : (unsigned)(r >> 43) + e + (carry << 21);
+  return __hiloint2double((int)(hi | (v < 0 ? 0x80000000u : 0u)),
+                          n == 64 ? 0 : (int)(unsigned)(r >> 11));
+}
+__device__ __forceinline__ bool adjoint_cell_fixed(const AGrid &g, int x, int y, int emax,
+                                                   const double (&fl)[kQ], const double (&mu)[kQ],
+                                                   double (&out)[kQ], double &t, double &bx,
+                                                   double &by) {
+  int bad;
+  FixedCell C;
+  fixed_cell(fl, g.fixed.k, C, bad);
+  long long vx = C.ux, vy = C.uy;
+  const Dig al = dig(g.fixed.alpha);
+  if (g.fixed.forced) {
+    const Dig Fx = dig(small_fixed(g.fxt[y], g.fixed.k, bad) - mulr(C.djx, al));
+    const Dig Fy = dig(small_fixed(g.fyt[x], g.fixed.k, bad) - mulr(C.djy, al));
+    const long long dx = mulr(Fx, C.ir), dy = mulr(Fy, C.ir);  // in 2^-60
+    bad |= (unsigned long long)(dx + (1ll << 57)) > (1ull << 58) ||
+           (unsigned long long)(dy + (1ll << 57)) > (1ull << 58);
+    vx += dx << 4;
+    vy += dy << 4;
+  }
+  if (bad) return false;
+  long long m[kQ];
+#pragma unroll
+  for (int l = 0; l < kQ; ++l) m[l] = adj_fixed(mu[l], emax);  // |m| < 2^54
+  const long long s13 = m[1] + m[3], d13 = m[1] - m[3], s24 = m[2] + m[4], d24 = m[2] - m[4];
+  const long long s57 = m[5] + m[7], d57 = m[5] - m[7], s68 = m[6] + m[8], d68 = m[6] - m[8];
+  const long long dg = s57 + s68;
+  // 36 times the t-weighted moments, below 2^59.2
+  const long long m0 = 16 * m[0] + 4 * (s13 + s24) + dg;
+  const long long m1x = 4 * d13 + (d57 - d68), m1y = 4 * d24 + (d57 + d68);
+  const Dig D0 = dig(m0), Dxx = dig(4 * s13 + dg), Dyy = dig(4 * s24 + dg), Dxy = dig(s57 - s68);
+  struct Part {
+    long long q2, px, py;  // 2 Q, 9 M2.w - 3 w M0
+  };
+  auto part = [&](long long wx, long long wy) {
+    const Dig ax = dig(wx), ay = dig(wy);
+    const long long px = mulr(Dxx, ax) + mulr(Dxy, ay), py = mulr(Dxy, ax) + mulr(Dyy, ay);
+    const long long w2 = mulr(ax, ax) + mulr(ay, ay);
+    const long long up = mulr(dig(px), ax) + mulr(dig(py), ay);
+    Part P;
+    P.q2 = 9 * up - 3 * mulr(D0, dig(w2));
+    P.px = 9 * px - 3 * mulr(D0, ax);
+    P.py = 9 * py - 3 * mulr(D0, ay);
+    return P;
+  };
+  const Part A = part(C.ux, C.uy), B = part(vx, vy);
+  const Dig w1 = dig(g.w1);  // omega - 1 in 2^-63
+  const long long sbx = 3 * m1x + B.px, sby = 3 * m1y + B.py;
+  const long long ar2 = 2 * mulr(dig(2 * m0 - A.q2), w1) + (2 * m0 - B.q2);  // 2 x 36 A_rho
+  const long long ax = 2 * mulr(dig(3 * m1x + A.px), w1) + sbx - mulr(dig(sbx), al);
+  const long long ay = 2 * mulr(dig(3 * m1y + A.py), w1) + sby - mulr(dig(sby), al);
+  // back from 36 times, eight times over for one rounding at the end
+  const Dig c836 = dig(4099276460824344804ll), c436 = dig(2049638230412172402ll);  // 2^67, 2^66 / 36
+  const Dig kp = dig(g.keep);  // (1 - omega) 2^63
+  const long long r = mulr(dig(ar2), c436), cx = mulr(dig(ax), c836), cy = mulr(dig(ay), c836);
+  auto put = [&](int l, long long add) {
+    out[l] = adj_double(mulr(dig(m[l] << 4), kp) + add, emax - 3);
+  };
+  put(0, r);
+  put(1, r + cx);
+  put(3, r - cx);
+  put(2, r + cy);
+  put(4, r - cy);
+  put(5, r + cx + cy);
+  put(7, r - cx - cy);
+  put(6, r - cx + cy);
+  put(8, r + cx - cy);
+  // sum mu f - rho (M0 + 3 u.M1 + Q), eight times over
+  long long muf = mulr(dig(m[0] << 3), dig(C.n[0] << 2));
+#pragma unroll
+  for (int l = 1; l < kQ; ++l) muf += mulr(dig(m[l] << 3), dig(C.n[l]));
+  const long long u1 = 3 * (mulr(dig(m1x), dig(C.ux)) + mulr(dig(m1y), dig(C.uy)));
+  muf -= 2 * mulr(dig(mulr(dig(2 * (m0 + u1) + A.q2), c436)), dig(2 * C.rho));
+  t = adj_double(muf, emax + g.fixed.k - 3);
+  bx = adj_double(mulr(dig(sbx), c836), emax - 3);
+  by = adj_double(mulr(dig(sby), c836), emax - 3);
+  return true;
+}
+
 // Adjoint of one step (see the header comment).  with_obj adds dJ_n/df on
 // the objective region R.  Each CTA's (dJ/dtau, dJ/dF0) sums go to its slot
 // of `partials`, added to what is there when `add` (a sweep's running sums;
@@ -291,63 +455,33 @@ __global__ void k_adjoint(AGrid g, Region R, const double *f, const double *lam_
   double acc[2] = {0.0, 0.0};
   FOR_CELLS {
     const int x = (int)(c % g.nx), y = (int)(c / g.nx);
-    double fl[kQ], mu[kQ];
+    double fl[kQ], mu[kQ], out[kQ], t, bx, by;
+    unsigned em = 0, ef = 0;
 #pragma unroll
     for (int l = 0; l < kQ; ++l) {
       fl[l] = f[(size_t)l * N + c];
       const int xd = wr(x + cx_of(l), g.nx), yd = wr(y + cy_of(l), g.ny);
       mu[l] = lam_in ? lam_in[(size_t)l * N + (size_t)yd * g.nx + xd] : 0.0;
+      if (mu[l] != 0.0) em = max(em, max(1u, ((unsigned)__double2hiint(mu[l]) >> 20) & 0x7ffu));
+      ef = max(ef, ((unsigned)__double2hiint(fl[l]) >> 20) & 0x7ffu);
     }
-    // moments from the opposite pairs' sums and differences
-    const double d57 = fl[5] - fl[7], d68 = fl[6] - fl[8];
-    const double rho = fl[0] + ((fl[1] + fl[3]) + (fl[2] + fl[4])) + ((fl[5] + fl[7]) + (fl[6] + fl[8]));
-    const double jx = (fl[1] - fl[3]) + (d57 - d68), jy = (fl[2] - fl[4]) + (d57 + d68);
-    const double ir = 1.0 / rho;
-    const double mpx = (1.0 - g.alpha) * jx + g.fxt[y];
-    const double mpy = (1.0 - g.alpha) * jy + g.fyt[x];
-    const MuMoments M = mu_moments(mu);
-    // equilibrium at (rho, j): q_a = m.M2.m, p_a = M2.m
-    const double pax = M.mxx * jx + M.mxy * jy, pay = M.mxy * jx + M.myy * jy;
-    const double qa = (4.5 * (jx * pax + jy * pay) - 1.5 * (jx * jx + jy * jy) * M.m0) * ir;
-    // at (rho, m')
-    const double pbx = M.mxx * mpx + M.mxy * mpy, pby = M.mxy * mpx + M.myy * mpy;
-    const double qb = (4.5 * (mpx * pbx + mpy * pby) - 1.5 * (mpx * mpx + mpy * mpy) * M.m0) * ir;
-    const double w1 = g.omega - 1.0;
-    const double Sa_rho = M.m0 - qa * ir, Sb_rho = M.m0 - qb * ir;
-    // S_a = 3 M_a + 9 p_a / rho - 3 m_a M0 / rho with 9 / rho and 3 M0 / rho
-    // formed once
-    const double ir9 = 9.0 * ir, k0 = 3.0 * M.m0 * ir, mx3 = 3.0 * M.mx, my3 = 3.0 * M.my;
-    const double Sa_x = fma(ir9, pax, fma(-jx, k0, mx3));
-    const double Sa_y = fma(ir9, pay, fma(-jy, k0, my3));
-    const double Sb_x = fma(ir9, pbx, fma(-mpx, k0, mx3));
-    const double Sb_y = fma(ir9, pby, fma(-mpy, k0, my3));
-    double Arho = w1 * Sa_rho + Sb_rho;
-    double Ajx = w1 * Sa_x + (1.0 - g.alpha) * Sb_x;
-    double Ajy = w1 * Sa_y + (1.0 - g.alpha) * Sb_y;
-    // sum mu (f - feq(rho, j)) for dJ/dtau
-    double muf = 0.0;
+    const unsigned emax = __reduce_max_sync(__activemask(), em);
+    const bool obj = with_obj && in_region(x, y, R, g);
+    if (emax == 0 && !obj && ef < 0x7ffu) {  // no adjoint here yet
 #pragma unroll
-    for (int l = 0; l < kQ; ++l) muf += mu[l] * fl[l];
-    const double mufeq = rho * M.m0 + 3.0 * (jx * M.mx + jy * M.my) + qa;
+      for (int l = 0; l < kQ; ++l) lam_out[(size_t)l * N + c] = 0.0;
+      continue;
+    }
+    // a common scale for the warp, away from the ends of the exponent range
+    if (obj || !g.fixed.ok || emax < 200u || emax > 1800u ||
+        !adjoint_cell_fixed(g, x, y, (int)emax, fl, mu, out, t, bx, by))
+      adjoint_cell_f64(g, x, y, fl, mu, obj ? F[D_TOT * N + c] : 0.0, obj ? F[D_JX * N + c] : 0.0,
+                       obj ? F[D_JY * N + c] : 0.0, out, t, bx, by);
     const double sx = F[S_TAB * N + y], sy = F[S_TAB * N + g.ny + x];
-    acc[0] += (muf - mufeq) * g.omega * g.omega;  // / tau^2
-    acc[1] += Sb_x * sx + Sb_y * sy;
-    if (with_obj && in_region(x, y, R, g)) {
-      Arho += F[D_TOT * N + c];
-      Ajx += F[D_JX * N + c];
-      Ajy += F[D_JY * N + c];
-    }
-    const double keep = 1.0 - g.omega;
-    // lambda_l = keep mu_l + Arho + c_l . A, by opposite pairs (c . A once
-    // per pair; a product by c = 0 still costs an FMA under IEEE arithmetic)
-    const double cA[4] = {Ajx, Ajy, Ajx + Ajy, Ajy - Ajx};  // c of 1, 2, 5, 6
-    lam_out[c] = fma(keep, mu[0], Arho);
+    acc[0] += t * g.omega * g.omega;  // / tau^2
+    acc[1] += bx * sx + by * sy;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int l = k < 2 ? 1 + k : 5 + (k - 2), m = opposite(l);
-      lam_out[(size_t)l * N + c] = fma(keep, mu[l], Arho + cA[k]);
-      lam_out[(size_t)m * N + c] = fma(keep, mu[m], Arho - cA[k]);
-    }
+    for (int l = 0; l < kQ; ++l) lam_out[(size_t)l * N + c] = out[l];
   }
   block_sums<2>(acc, partials + 2 * blockIdx.x, add);
 }
@@ -514,6 +648,10 @@ AGrid agrid(const Member &hm) {
   g.F0 = hm.F0;
   g.fxt = hm.fx_tab64;
   g.fyt = hm.fy_tab64;
+  g.fixed = hm.fixed;
+  g.fixed.ok = g.fixed.ok && std::abs(g.fixed.k) < 100 && std::fabs(hm.omega - 1.0) < 1.0 - 1e-9;
+  g.w1 = g.fixed.ok ? std::llrint(std::ldexp(hm.omega - 1.0, 63)) : 0;
+  g.keep = -g.w1;
   return g;
 }
 

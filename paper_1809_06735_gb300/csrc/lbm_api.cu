@@ -837,7 +837,7 @@ int lbm_create(const lbm_config *cfg, void *workspace, size_t bytes, lbm_handle 
       h->has_kind2 = true;
       if (h->precision != 32 || c.nx % 4 != 0) h->proj_quad = false;
     }
-    if (h->precision == 64 && c.collision == 0) {  // see collide_fixed
+    if (c.collision == 0) {  // see collide_fixed; the adjoint of either precision uses it
       lbm::FixedBgk &B = M.fixed;
       B.k = std::ilogb(c.rho0) + 2;
       B.om = std::llrint(std::ldexp(M.omega, 62));

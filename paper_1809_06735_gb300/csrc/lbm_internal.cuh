@@ -80,7 +80,7 @@ struct Member {
   double Cs;
   void *nu_ring;         // local viscosity at each snapshot slot [3][N]
                          // (storage precision), collision != 0
-  FixedBgk fixed;        // FP64 storage
+  FixedBgk fixed;
 };
 
 // Local relaxation time of a cell from its non-equilibrium stress
