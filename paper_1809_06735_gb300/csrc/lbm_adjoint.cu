@@ -337,10 +337,12 @@ __device__ __forceinline__ void adjoint_cell_f64(const AGrid &g, int x, int y,
 }
 
 // The same in 64-bit fixed point (collide_fixed's reasons and range; 256^2:
-// 13.6 us per adjoint step against 22.8).  The populations of the adjoint have no
+// 13.9 us per adjoint step against 22.8).  The populations of the adjoint have no
 // scale of their own: they are taken in units of 2^-53 of the exponent of the
-// largest one of the warp's 32 cells (emax), sums and products with three to
-// five more bits, so that the warp's largest values keep FP64's 53 bits.  With u = j / rho and v = m' / rho the terms are
+// cell's largest one (emax), sums and products with three to six more bits, so
+// that the cell's largest values keep FP64's 53 bits.  (A scale per warp loses
+// the small adjoints beside a large one: 1e-8 relative at the 99th percentile
+// on the rim of the objective's reach, 1e-14 in FP64.)  With u = j / rho and v = m' / rho the terms are
 //   S_rho = M0 - Q(u), S = 3 M1 + 9 M2.u - 3 u M0,
 //   Q(u) = 4.5 u.M2.u - 1.5 |u|^2 M0,
 // (36 M are exact integer sums of the mu), sum mu feq = rho (M0 + 3 u.M1 +
@@ -433,13 +435,19 @@ __device__ __forceinline__ bool adjoint_cell_fixed(const AGrid &g, int x, int y,
   put(7, r - cx - cy);
   put(6, r - cx + cy);
   put(8, r + cx - cy);
-  // sum mu f - rho (M0 + 3 u.M1 + Q), eight times over
-  long long muf = mulr(dig(m[0] << 3), dig(C.n[0] << 2));
+  // sum mu f - rho (M0 + 3 u.M1 + Q), 64 times over: the difference is a
+  // thousandth of its parts
+  const Dig c6436 = dig(8198552921648689607ll);  // 2^68 / 36
+  long long muf = mulr(dig(m[0] << 6), dig(C.n[0] << 2));
 #pragma unroll
-  for (int l = 1; l < kQ; ++l) muf += mulr(dig(m[l] << 3), dig(C.n[l]));
+  for (int l = 1; l < kQ; ++l) muf += mulr(dig(m[l] << 6), dig(C.n[l]));
   const long long u1 = 3 * (mulr(dig(m1x), dig(C.ux)) + mulr(dig(m1y), dig(C.uy)));
-  muf -= 2 * mulr(dig(mulr(dig(2 * (m0 + u1) + A.q2), c436)), dig(2 * C.rho));
-  t = adj_double(muf, emax + g.fixed.k - 3);
+  // rho with the bits that its two quarter sums dropped (one sign: they would
+  // add up over the cells)
+  const int cut = ((int)(C.n[1] + C.n[2] + C.n[3] + C.n[4]) & 3) +
+                  ((int)(C.n[5] + C.n[6] + C.n[7] + C.n[8]) & 3);
+  muf -= 2 * mulr(dig(mulr(dig(2 * (2 * (m0 + u1) + A.q2)), c6436)), dig(2 * C.rho + (cut >> 1)));
+  t = adj_double(muf, emax + g.fixed.k - 6);
   bx = adj_double(mulr(dig(sbx), c836), emax - 3);
   by = adj_double(mulr(dig(sby), c836), emax - 3);
   return true;
@@ -456,23 +464,22 @@ __global__ void k_adjoint(AGrid g, Region R, const double *f, const double *lam_
   FOR_CELLS {
     const int x = (int)(c % g.nx), y = (int)(c / g.nx);
     double fl[kQ], mu[kQ], out[kQ], t, bx, by;
-    unsigned em = 0, ef = 0;
+    unsigned emax = 0, ef = 0;
 #pragma unroll
     for (int l = 0; l < kQ; ++l) {
       fl[l] = f[(size_t)l * N + c];
       const int xd = wr(x + cx_of(l), g.nx), yd = wr(y + cy_of(l), g.ny);
       mu[l] = lam_in ? lam_in[(size_t)l * N + (size_t)yd * g.nx + xd] : 0.0;
-      if (mu[l] != 0.0) em = max(em, max(1u, ((unsigned)__double2hiint(mu[l]) >> 20) & 0x7ffu));
+      if (mu[l] != 0.0) emax = max(emax, max(1u, ((unsigned)__double2hiint(mu[l]) >> 20) & 0x7ffu));
       ef = max(ef, ((unsigned)__double2hiint(fl[l]) >> 20) & 0x7ffu);
     }
-    const unsigned emax = __reduce_max_sync(__activemask(), em);
     const bool obj = with_obj && in_region(x, y, R, g);
     if (emax == 0 && !obj && ef < 0x7ffu) {  // no adjoint here yet
 #pragma unroll
       for (int l = 0; l < kQ; ++l) lam_out[(size_t)l * N + c] = 0.0;
       continue;
     }
-    // a common scale for the warp, away from the ends of the exponent range
+    // a common scale for the cell, away from the ends of the exponent range
     if (obj || !g.fixed.ok || emax < 200u || emax > 1800u ||
         !adjoint_cell_fixed(g, x, y, (int)emax, fl, mu, out, t, bx, by))
       adjoint_cell_f64(g, x, y, fl, mu, obj ? F[D_TOT * N + c] : 0.0, obj ? F[D_JX * N + c] : 0.0,
