@@ -29,9 +29,13 @@ namespace lbm {
 
 namespace {
 
-enum AdjField { A_RHO = 0, A_JX, A_JY, A_U, A_V, GAM_XX, GAM_XY, GAM_YY, D_RHO, D_JX, D_JY,
-                D_TOT, S_TAB, A_NFIELDS };  // S_TAB: sin(2 pi kf y/ny) [ny], then of x [nx]
-static_assert(A_NFIELDS <= kDiagFields, "scratch too small");
+// Fields of the objective on its region, one set per level of a batch:
+// kObjFields planes of region cells.
+enum ObjField { A_RHO = 0, A_U, A_V, GAM_XX, GAM_XY, GAM_YY, D_RHO, D_JX, D_JY, D_TOT, kObjFields };
+constexpr int kObjLevels = 256;  // levels of one batch at most
+struct ObjWeights {
+  double cw[kObjLevels];  // weight / L^2 per level, 0: no objective at that level
+};
 
 struct AGrid {
   int nx, ny, kf, force;
@@ -116,14 +120,25 @@ __device__ __forceinline__ bool in_region(int x, int y, const Region &r, const A
   return wrapi(x - r.x0, g.nx) < r.w && wrapi(y - r.y0, g.ny) < r.h;
 }
 
-#define FOR_REGION(R)                                                                  \
-  const size_t N = (size_t)g.nx * g.ny;                                                \
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < (R).w * (R).h;               \
-       i += gridDim.x * blockDim.x)
+// Index of cell (x, y) of the region in its planes.
+__device__ __forceinline__ int region_index(int x, int y, const Region &r, const AGrid &g) {
+  return wrapi(y - r.y0, g.ny) * r.w + wrapi(x - r.x0, g.nx);
+}
 
-// rho, j and u = (j + F/2)/rho of the public state f[9][ny][nx] on R.
-__global__ void k_region_velocity(AGrid g, Region R, const double *f, double *F) {
-  FOR_REGION(R) {
+// The objective's kernels run over the levels of a batch at once (blockIdx.y):
+// they read the recorded states only, so nothing of them has to wait for the
+// adjoint.  One launch per level and kernel cost 14.4 us per weighted level of
+// 256^2, L = 16, between the adjoint steps.
+
+// rho, j and u = (j + F/2)/rho of the public states f[level][9][ny][nx] on R.
+__global__ void k_region_velocity(AGrid g, Region R, const double *states, double *fields,
+                                  ObjWeights W) {
+  const int q = blockIdx.y, nreg = R.w * R.h;
+  if (W.cw[q] == 0.0) return;
+  const size_t N = (size_t)g.nx * g.ny;
+  const double *f = states + (size_t)q * kQ * N;
+  double *F = fields + (size_t)q * kObjFields * nreg;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nreg; i += gridDim.x * blockDim.x) {
     const int x = wrapi(R.x0 + i % R.w, g.nx), y = wrapi(R.y0 + i / R.w, g.ny);
     const size_t c = (size_t)y * g.nx + x;
     double r = 0, a = 0, b = 0;
@@ -136,9 +151,9 @@ __global__ void k_region_velocity(AGrid g, Region R, const double *f, double *F)
     }
     const double Fx = g.fxt[y] - g.alpha * a, Fy = g.fyt[x] - g.alpha * b;
     const double ir = 1.0 / r;
-    F[A_RHO * N + c] = r;
-    F[A_U * N + c] = (a + 0.5 * Fx) * ir;
-    F[A_V * N + c] = (b + 0.5 * Fy) * ir;
+    F[A_RHO * nreg + i] = r;
+    F[A_U * nreg + i] = (a + 0.5 * Fx) * ir;
+    F[A_V * nreg + i] = (b + 0.5 * Fy) * ir;
   }
 }
 
@@ -158,11 +173,13 @@ __device__ __forceinline__ double quad_get(double v, int qb, int k) {
   return __shfl_sync(0xffffffffu, v, qb + k);
 }
 
-// The eq. (18) stencil derivative of A along x (dir 0) or y (dir 1) at (x, y),
-// one code path for both directions (no divergence within a quad).
-__device__ __forceinline__ double D_dir(const double *A, const AGrid &g, int x, int y, int dir) {
+// The eq. (18) stencil derivative of the region plane A along x (dir 0) or y
+// (dir 1) at (x, y), one code path for both directions (no divergence within
+// a quad).
+__device__ __forceinline__ double D_dir(const double *A, const AGrid &g, const Region &R, int x,
+                                        int y, int dir) {
   auto at = [&](int k) {
-    return dir ? A[(size_t)wr(y + k, g.ny) * g.nx + x] : A[(size_t)y * g.nx + wr(x + k, g.nx)];
+    return A[dir ? region_index(x, wr(y + k, g.ny), R, g) : region_index(wr(x + k, g.nx), y, R, g)];
   };
   return 0.8 * (at(1) - at(-1)) - 0.2 * (at(2) - at(-2)) + (4.0 / 105.0) * (at(3) - at(-3)) -
          (1.0 / 280.0) * (at(4) - at(-4));
@@ -171,32 +188,34 @@ __device__ __forceinline__ double D_dir(const double *A, const AGrid &g, int x, 
 // Objective pass 1, over V0: Gamma_ij = dJ/dG_ij = -2 c nu rho S_ij
 // (c = weight / L^2); explicit dJ/dtau part -c rho Q / 3 (d nu / d tau = 1/3).
 // Four lanes per cell (FOR_QUADS): d/dx u, d/dy u, d/dx v, d/dy v.
-__global__ void k_obj_gamma(AGrid g, double *F, double cw, int bx, int by, int L,
-                            double *partials, int add) {
+__global__ void k_obj_gamma(AGrid g, Region R, double *fields, ObjWeights W, int bx, int by, int L,
+                            double *partials) {
+  const int q = blockIdx.y, nreg = R.w * R.h;
+  const double cw = W.cw[q];
+  double *F = fields + (size_t)q * kObjFields * nreg;
   double acc[1] = {0.0};
-  const size_t N = (size_t)g.nx * g.ny;
-  const int nc = L * L;
+  const int nc = cw == 0.0 ? 0 : L * L;
   FOR_QUADS(nc) {
     const int iq = i0 + (lane >> 2), i = iq < nc ? iq : nc - 1;
     const int x = wrapi(bx + i % L, g.nx), y = wrapi(by + i / L, g.ny);
-    const size_t c = (size_t)y * g.nx + x;
-    const double d = D_dir(F + (p < 2 ? A_U : A_V) * N, g, x, y, p & 1);
+    const int c = region_index(x, y, R, g);
+    const double d = D_dir(F + (p < 2 ? A_U : A_V) * nreg, g, R, x, y, p & 1);
     const double dxu = quad_get(d, qb, 0), dyu = quad_get(d, qb, 1);
     const double dxv = quad_get(d, qb, 2), dyv = quad_get(d, qb, 3);
     if (iq < nc) {
       const double sxx = 2 * dxu, sxy = dyu + dxv, syy = 2 * dyv;
-      const double r = F[A_RHO * N + c];
+      const double r = F[A_RHO * nreg + c];
       if (p < 3) {  // Gamma_xx, Gamma_xy, Gamma_yy: one per lane
         const double sp = p == 0 ? sxx : (p == 1 ? sxy : syy);
-        F[(GAM_XX + p) * N + c] = -2.0 * cw * g.nu * r * sp;
+        F[(GAM_XX + p) * nreg + c] = -2.0 * cw * g.nu * r * sp;
       } else {
         const double Q = sxx * dxu + sxy * dyu + sxy * dxv + syy * dyv;
-        F[D_RHO * N + c] = -cw * g.nu * Q;
+        F[D_RHO * nreg + c] = -cw * g.nu * Q;
         acc[0] += -cw * r * Q / 3.0;
       }
     }
   }
-  block_sums<1>(acc, partials + blockIdx.x, add);
+  block_sums<1>(acc, partials + (size_t)q * gridDim.x + blockIdx.x);
 }
 
 // Objective pass 2, over R: dJ/du_i = -sum_j D_j Gamma_ij (D^T = -D), then
@@ -205,56 +224,71 @@ __global__ void k_obj_gamma(AGrid g, double *F, double cw, int bx, int by, int L
 // (FOR_QUADS): D_x Gamma_xx, D_y Gamma_xy, D_x Gamma_xy, D_y Gamma_yy, Gamma
 // zero outside V0; then one quotient per lane (dJ/djx, dJ/djy, the velocity
 // part of dJ/drho, the dJ/dF0 term) and the force direction s from the
-// sine tables at F[S_TAB].
-__global__ void k_obj_velocity_adjoint(AGrid g, Region R, double *F, int bx, int by, int L,
-                                       double *partials, int add) {
+// sine tables.
+__global__ void k_obj_velocity_adjoint(AGrid g, Region R, double *fields, ObjWeights W,
+                                       const double *sines, int bx, int by, int L,
+                                       double *partials) {
+  const int q = blockIdx.y, nreg = R.w * R.h;
+  double *F = fields + (size_t)q * kObjFields * nreg;
   double acc[1] = {0.0};
-  const size_t N = (size_t)g.nx * g.ny;
-  const int nc = R.w * R.h;
+  const int nc = W.cw[q] == 0.0 ? 0 : nreg;
   FOR_QUADS(nc) {
     const int iq = i0 + (lane >> 2), i = iq < nc ? iq : nc - 1;
     const int x = wrapi(R.x0 + i % R.w, g.nx), y = wrapi(R.y0 + i / R.w, g.ny);
-    const size_t c = (size_t)y * g.nx + x;
     // box-relative coordinates: the stencil point k along dir is in V0 when
     // its along coordinate wraps into [0, L) and the cross one already is
     const int rx = wrapi(x - bx, g.nx), ry = wrapi(y - by, g.ny);
     const int dir = p & 1;
-    const double *G = F + (p == 0 ? GAM_XX : (p == 3 ? GAM_YY : GAM_XY)) * N;
+    const double *G = F + (p == 0 ? GAM_XX : (p == 3 ? GAM_YY : GAM_XY)) * nreg;
     const int ra = dir ? ry : rx, na = dir ? g.ny : g.nx;
     const bool cross_in = (dir ? rx : ry) < L;
     auto at = [&](int k) {
-      const int t = wr(ra + k, na);
-      const size_t e = dir ? (size_t)wr(y + k, g.ny) * g.nx + x : (size_t)y * g.nx + wr(x + k, g.nx);
-      return (cross_in && t < L) ? G[e] : 0.0;
+      if (!(cross_in && wr(ra + k, na) < L)) return 0.0;
+      return G[dir ? region_index(x, wr(y + k, g.ny), R, g) : region_index(wr(x + k, g.nx), y, R, g)];
     };
     const double d = 0.8 * (at(1) - at(-1)) - 0.2 * (at(2) - at(-2)) +
                      (4.0 / 105.0) * (at(3) - at(-3)) - (1.0 / 280.0) * (at(4) - at(-4));
     const double Ux = -(quad_get(d, qb, 0) + quad_get(d, qb, 1));
     const double Uy = -(quad_get(d, qb, 2) + quad_get(d, qb, 3));
-    const double r = F[A_RHO * N + c];
+    const double r = F[A_RHO * nreg + i];
     double num;
     if (p == 0) {
       num = Ux * (1.0 - 0.5 * g.alpha);
     } else if (p == 1) {
       num = Uy * (1.0 - 0.5 * g.alpha);
     } else if (p == 2) {
-      num = Ux * F[A_U * N + c] + Uy * F[A_V * N + c];
+      num = Ux * F[A_U * nreg + i] + Uy * F[A_V * nreg + i];
     } else {
-      num = Ux * F[S_TAB * N + y] + Uy * F[S_TAB * N + g.ny + x];
+      num = Ux * sines[y] + Uy * sines[g.ny + x];
     }
-    const double q = num / (p == 3 ? 2.0 * r : r);
+    const double qt = num / (p == 3 ? 2.0 * r : r);
     if (iq < nc) {
       if (p < 2) {
-        F[(D_JX + p) * N + c] = q;
+        F[(D_JX + p) * nreg + i] = qt;
       } else if (p == 2) {
-        const double direct = (rx < L && ry < L) ? F[D_RHO * N + c] : 0.0;
-        F[D_TOT * N + c] = direct - q;
+        const double direct = (rx < L && ry < L) ? F[D_RHO * nreg + i] : 0.0;
+        F[D_TOT * nreg + i] = direct - qt;
       } else {
-        acc[0] += q;
+        acc[0] += qt;
       }
     }
   }
-  block_sums<1>(acc, partials + blockIdx.x, add);
+  block_sums<1>(acc, partials + (size_t)q * gridDim.x + blockIdx.x);
+}
+
+// Adds a batch's objective partials to the sweep's running sums, fixed order.
+__global__ void __launch_bounds__(256) k_obj_sum(const double *pt, int nt, const double *pf, int nf,
+                                                 double *tau, double *F0) {
+  double acc[2] = {0.0, 0.0};
+  for (int i = threadIdx.x; i < nt; i += 256) acc[0] += pt[i];
+  for (int i = threadIdx.x; i < nf; i += 256) acc[1] += pf[i];
+  __shared__ double out[2];
+  block_sums<2>(acc, out);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    *tau += out[0];
+    *F0 += out[1];
+  }
 }
 
 // t_l-weighted sums over the populations of the pulled adjoint mu_l and
@@ -453,13 +487,13 @@ __device__ __forceinline__ bool adjoint_cell_fixed(const AGrid &g, int x, int y,
   return true;
 }
 
-// Adjoint of one step (see the header comment).  with_obj adds dJ_n/df on
-// the objective region R.  Each CTA's (dJ/dtau, dJ/dF0) sums go to its slot
-// of `partials`, added to what is there when `add` (a sweep's running sums;
-// steps are stream-ordered, so a slot has one writer at a time).
+// Adjoint of one step (see the header comment).  obj_fields (or NULL) adds
+// dJ_n/df on the objective region R.  Each CTA's (dJ/dtau, dJ/dF0) sums are
+// added to its slot of `partials` (a sweep's running sums; steps are
+// stream-ordered, so a slot has one writer at a time).
 __global__ void k_adjoint(AGrid g, Region R, const double *f, const double *lam_in,
-                          double *lam_out, const double *F, int with_obj, double *partials,
-                          int add) {
+                          double *lam_out, const double *sines, const double *obj_fields,
+                          double *partials) {
   double acc[2] = {0.0, 0.0};
   FOR_CELLS {
     const int x = (int)(c % g.nx), y = (int)(c / g.nx);
@@ -473,7 +507,7 @@ __global__ void k_adjoint(AGrid g, Region R, const double *f, const double *lam_
       if (mu[l] != 0.0) emax = max(emax, max(1u, ((unsigned)__double2hiint(mu[l]) >> 20) & 0x7ffu));
       ef = max(ef, ((unsigned)__double2hiint(fl[l]) >> 20) & 0x7ffu);
     }
-    const bool obj = with_obj && in_region(x, y, R, g);
+    const bool obj = obj_fields && in_region(x, y, R, g);
     if (emax == 0 && !obj && ef < 0x7ffu) {  // no adjoint here yet
 #pragma unroll
       for (int l = 0; l < kQ; ++l) lam_out[(size_t)l * N + c] = 0.0;
@@ -481,16 +515,19 @@ __global__ void k_adjoint(AGrid g, Region R, const double *f, const double *lam_
     }
     // a common scale for the cell, away from the ends of the exponent range
     if (obj || !g.fixed.ok || emax < 200u || emax > 1800u ||
-        !adjoint_cell_fixed(g, x, y, (int)emax, fl, mu, out, t, bx, by))
-      adjoint_cell_f64(g, x, y, fl, mu, obj ? F[D_TOT * N + c] : 0.0, obj ? F[D_JX * N + c] : 0.0,
-                       obj ? F[D_JY * N + c] : 0.0, out, t, bx, by);
-    const double sx = F[S_TAB * N + y], sy = F[S_TAB * N + g.ny + x];
+        !adjoint_cell_fixed(g, x, y, (int)emax, fl, mu, out, t, bx, by)) {
+      const int nreg = R.w * R.h, i = obj ? region_index(x, y, R, g) : 0;
+      const double *F = obj_fields + i;
+      adjoint_cell_f64(g, x, y, fl, mu, obj ? F[D_TOT * nreg] : 0.0, obj ? F[D_JX * nreg] : 0.0,
+                       obj ? F[D_JY * nreg] : 0.0, out, t, bx, by);
+    }
+    const double sx = sines[y], sy = sines[g.ny + x];
     acc[0] += t * g.omega * g.omega;  // / tau^2
     acc[1] += bx * sx + by * sy;
 #pragma unroll
     for (int l = 0; l < kQ; ++l) lam_out[(size_t)l * N + c] = out[l];
   }
-  block_sums<2>(acc, partials + 2 * blockIdx.x, add);
+  block_sums<2>(acc, partials + 2 * blockIdx.x, 1);
 }
 
 // Adds every partial into the two accumulators: thread i sums the partials
@@ -685,42 +722,20 @@ int adjoint_threads(size_t N) { return N < ((size_t)1 << 17) ? 64 : 256; }
 cudaError_t adjoint_step(const Member &hm, const double *f_n, const double *lam_in,
                          double *lam_out, double w, int bx, int by, int L, double *dJ_dtau,
                          double *dJ_dF0, const DiagScratch &sc, cudaStream_t s) {
-  const AGrid g = agrid(hm);
-  const size_t N = (size_t)hm.nx * hm.ny;
-  const int tpb = adjoint_threads(N), nb = nblocks_for(N, tpb);
-  double *F = sc.f;
-  double *p_step = sc.partials;                         // [nb][2]
-  double *p_tau = p_step + 2 * kMaxPartialBlocks;       // [nbo]
-  double *p_F0 = p_tau + kMaxPartialBlocks;             // [nbr]
-  const int with_obj = w != 0.0;
-  const Region R = objective_region(hm.nx, hm.ny, bx, by, L);
-  int nbo = 0, nbr = 0;
-  k_sine_tables<<<(hm.nx + hm.ny + 255) / 256, 256, 0, s>>>(g, F + S_TAB * N);
-  if (with_obj) {
-    const double cw = w / ((double)L * (double)L);
-    const size_t nreg = (size_t)R.w * R.h;
-    nbr = nblocks_for(4 * nreg, kObjThreads);  // four lanes per cell
-    nbo = nblocks_for(4 * (size_t)L * L, kObjThreads);
-    k_region_velocity<<<nblocks_for(nreg, kObjThreads), kObjThreads, 0, s>>>(g, R, f_n, F);
-    k_obj_gamma<<<nbo, kObjThreads, 0, s>>>(g, F, cw, bx, by, L, p_tau, 0);
-    k_obj_velocity_adjoint<<<nbr, kObjThreads, 0, s>>>(g, R, F, bx, by, L, p_F0, 0);
-  }
-  k_adjoint<<<nb, tpb, 0, s>>>(g, R, f_n, lam_in, lam_out, F, with_obj, p_step, 0);
-  k_adjoint_final<<<1, 256, 0, s>>>(p_step, nb, p_tau, nbo, p_F0, nbr, with_obj, dJ_dtau,
-                                    dJ_dF0);
-  return cudaGetLastError();
+  return adjoint_sweep(hm, f_n, 1, lam_in, lam_out, nullptr, &w, bx, by, L, dJ_dtau, dJ_dF0, sc, s,
+                       nullptr);
 }
 
-int adjoint_kernel_count(double w) { return w != 0.0 ? 6 : 3; }
+int adjoint_kernel_count(double w) { return w != 0.0 ? 7 : 3; }
 
 // The adjoint steps of states[nstates - 1] .. states[0] (each [9][ny][nx]),
 // the adjoint ping-ponging between lam_out and lam_tmp so that the last
 // (state 0) lands in lam_out; weights[k] (host) the objective weight of
-// step k.  Each CTA keeps running sums of its (dJ/dtau, dJ/dF0) partials
-// over the whole sweep and one reduction at the end adds them into the
-// accumulators; the force-direction tables are built once.  The adjoint
-// fields are those of per-step adjoint_step calls; the two gradients differ
-// from theirs only by the order of the FP64 sums.
+// step k.  The objective's fields of a batch of levels (as many as the
+// scratch holds) come from three launches before the batch's adjoint steps.
+// Each CTA keeps running sums of its (dJ/dtau, dJ/dF0) partials over the
+// whole sweep and one reduction at the end adds them into the accumulators;
+// the force-direction tables are built once.
 cudaError_t adjoint_sweep(const Member &hm, const double *states, int nstates,
                           const double *lam_in, double *lam_out, double *lam_tmp,
                           const double *weights, int bx, int by, int L, double *dJ_dtau,
@@ -729,38 +744,60 @@ cudaError_t adjoint_sweep(const Member &hm, const double *states, int nstates,
   const AGrid g = agrid(hm);
   const size_t N = (size_t)hm.nx * hm.ny;
   const int tpb = adjoint_threads(N), nb = nblocks_for(N, tpb);
-  double *F = sc.f;
+  double *sines = sc.f, *fields = sc.f + (hm.nx + hm.ny);
   double *p_step = sc.partials;                    // [nb][2]
-  double *p_tau = p_step + 2 * kMaxPartialBlocks;  // [nbo]
-  double *p_F0 = p_tau + kMaxPartialBlocks;        // [nbr]
+  double *p_tau = p_step + 2 * kMaxPartialBlocks;  // the objective's running sums
+  double *p_F0 = p_tau + kMaxPartialBlocks;
   int any_obj = 0;
   for (int k = 0; k < nstates; ++k) any_obj |= weights[k] != 0.0;
-  const Region R = objective_region(hm.nx, hm.ny, bx, by, L);
+  const Region R = any_obj ? objective_region(hm.nx, hm.ny, bx, by, L) : Region{0, 0, 1, 1};
   const size_t nreg = (size_t)R.w * R.h;
   const int nbv = nblocks_for(nreg, kObjThreads);
-  const int nbr = any_obj ? nblocks_for(4 * nreg, kObjThreads) : 0;  // four lanes per cell
-  const int nbo = any_obj ? nblocks_for(4 * (size_t)L * L, kObjThreads) : 0;
+  const int nbr = any_obj ? nblocks_for(4 * nreg, kObjThreads) : 1;  // four lanes per cell
+  const int nbo = any_obj ? nblocks_for(4 * (size_t)L * L, kObjThreads) : 1;
+  // per level: the fields and the two passes' partials
+  const size_t per = kObjFields * nreg + nbr + nbo;
+  const size_t room = (size_t)kDiagFields * sc.N - (hm.nx + hm.ny);
+  const int batch = (int)std::min<size_t>({room / per, (size_t)kObjLevels, (size_t)nstates});
+  if (any_obj && batch < 1) return cudaErrorInvalidValue;
   cudaError_t e = cudaMemsetAsync(p_step, 0, sizeof(double) * 4 * kMaxPartialBlocks, s);
   if (e != cudaSuccess) return e;
-  k_sine_tables<<<(hm.nx + hm.ny + 255) / 256, 256, 0, s>>>(g, F + S_TAB * N);
+  k_sine_tables<<<(hm.nx + hm.ny + 255) / 256, 256, 0, s>>>(g, sines);
   long long n = 2;
   const double *in = lam_in;
-  for (int k = nstates - 1; k >= 0; --k) {
-    double *out = (k % 2 == 0) ? lam_out : lam_tmp;
-    const double *f_k = states + (size_t)k * kQ * N;
-    const int with_obj = weights[k] != 0.0;
-    if (with_obj) {
-      const double cw = weights[k] / ((double)L * (double)L);
-      k_region_velocity<<<nbv, kObjThreads, 0, s>>>(g, R, f_k, F);
-      k_obj_gamma<<<nbo, kObjThreads, 0, s>>>(g, F, cw, bx, by, L, p_tau, 1);
-      k_obj_velocity_adjoint<<<nbr, kObjThreads, 0, s>>>(g, R, F, bx, by, L, p_F0, 1);
-      n += 3;
+  for (int hi = nstates; hi > 0;) {
+    const int lo = any_obj ? std::max(0, hi - batch) : 0, cnt = hi - lo;
+    if (any_obj) {
+      ObjWeights W{};
+      bool some = false;
+      for (int q = 0; q < cnt; ++q) {
+        W.cw[q] = weights[lo + q] / ((double)L * (double)L);
+        some |= W.cw[q] != 0.0;
+      }
+      if (some) {
+        double *pt = fields + (size_t)cnt * kObjFields * nreg, *pf = pt + (size_t)cnt * nbo;
+        const double *f0 = states + (size_t)lo * kQ * N;
+        k_region_velocity<<<dim3(nbv, cnt), kObjThreads, 0, s>>>(g, R, f0, fields, W);
+        k_obj_gamma<<<dim3(nbo, cnt), kObjThreads, 0, s>>>(g, R, fields, W, bx, by, L, pt);
+        k_obj_velocity_adjoint<<<dim3(nbr, cnt), kObjThreads, 0, s>>>(g, R, fields, W, sines, bx,
+                                                                      by, L, pf);
+        k_obj_sum<<<1, 256, 0, s>>>(pt, cnt * nbo, pf, cnt * nbr, p_tau, p_F0);
+        n += 4;
+      }
     }
-    k_adjoint<<<nb, tpb, 0, s>>>(g, R, f_k, in, out, F, with_obj, p_step, 1);
-    n += 1;
-    in = out;
+    for (int k = hi - 1; k >= lo; --k) {
+      double *out = (k % 2 == 0) ? lam_out : lam_tmp;
+      k_adjoint<<<nb, tpb, 0, s>>>(g, R, states + (size_t)k * kQ * N, in, out, sines,
+                                   weights[k] / ((double)L * (double)L) != 0.0
+                                       ? fields + (size_t)(k - lo) * kObjFields * nreg
+                                       : nullptr,
+                                   p_step);
+      n += 1;
+      in = out;
+    }
+    hi = lo;
   }
-  k_adjoint_final<<<1, 256, 0, s>>>(p_step, nb, p_tau, nbo, p_F0, nbr, any_obj, dJ_dtau, dJ_dF0);
+  k_adjoint_final<<<1, 256, 0, s>>>(p_step, nb, p_tau, 1, p_F0, 1, any_obj, dJ_dtau, dJ_dF0);
   if (launches) *launches += n;
   return cudaGetLastError();
 }

@@ -1,6 +1,7 @@
 """One adjoint step against extended precision, cell by cell: the fixed-point
 form (its scale is the cell's own largest adjoint) and the FP64 form that
-takes the cells outside its range."""
+takes the cells outside its range; and the objective's fields over several
+batches of levels."""
 import numpy as np
 import pytest
 
@@ -74,3 +75,37 @@ def test_adjoint_step_exact(nx, ny, adjoint, rho0, tau):
     assert (np.abs(out.cpu().numpy() - ref) <= eps * top).all()
     assert abs(float(dt) - rt) <= eps * (top * np.maximum(rho, 1)).sum() / tau ** 2
     assert abs(float(dF) - rF) <= eps * top.sum()
+
+
+@pytest.mark.parametrize("nx,ny,L,nstates,every", [
+    (40, 28, 28, 13, 1),   # region = grid: five levels fit the scratch at once
+    (40, 28, 20, 13, 5),   # batches with weighted, partly weighted and no levels
+    (16, 12, 2, 300, 7),   # more levels than one batch may have
+    (3, 2, 2, 9, 2)])
+def test_objective_batches_match_single_steps(nx, ny, L, nstates, every):
+    """A sweep whose levels take several batches against single steps: the
+    adjoint bit for bit, the gradients to the rounding of their sums (2^-53
+    per level and partial, 1e-12 covers 300 levels)."""
+    import torch
+
+    import paper_1809_06735_gb300 as P
+
+    lat = P.Lattice([P.Member(nx, ny, 0.56, 1.0, 1, 1, 2e-4, 1e-3)], precision=64)
+    rng = np.random.default_rng(nx)
+    u = 0.03 * rng.standard_normal((2, ny, nx)).clip(-2, 2)
+    lat.init_fields(0, np.ones((ny, nx)), u[0], u[1])
+    states = torch.empty((nstates, 9, ny, nx), dtype=torch.float64, device="cuda")
+    lat.record_trajectory(0, states)
+    w = np.where(np.arange(nstates) % every == 0, 0.1 + np.arange(nstates) / nstates, 0.0)
+    acc = torch.zeros(4, dtype=torch.float64, device="cuda")
+    new = lambda: torch.empty((9, ny, nx), dtype=torch.float64, device="cuda")
+    out, box = new(), (nx - 1, 1)
+    lat.adjoint_sweep(0, states, None, out, new(), w, box, L, acc[0:1], acc[1:2])
+    lam = None
+    for k in range(nstates - 1, -1, -1):
+        nxt = new()
+        lat.adjoint_step(0, states[k], lam, nxt, float(w[k]), box, L, acc[2:3], acc[3:4])
+        lam = nxt
+    assert torch.equal(out, lam) and bool(out.isfinite().all())
+    a = acc.cpu().numpy()
+    assert abs(a[0] - a[2]) <= 1e-12 * abs(a[2]) and abs(a[1] - a[3]) <= 1e-12 * abs(a[3])
