@@ -118,6 +118,17 @@ def profiled_traffic():
     return d.get("dram_bytes_per_full_launch")
 
 
+def bytes_per_lu_f32(lat) -> float:
+    """Algorithmic bytes of one FP32 update: a launch that advances T steps
+    reads and writes the populations once for all of them (72 / T)."""
+    return BYTES_PER_LU_F32 / lat.steps_per_launch
+
+
+def step_kernel_name(lat) -> str:
+    t = lat.steps_per_launch
+    return "k_multi (%d steps per launch)" % t if t > 1 else "k_step_f32_vec"
+
+
 class ClockSampler:
     """nvidia-smi clocks and throttle reasons sampled during the timed region."""
 
@@ -446,7 +457,7 @@ def collision_models_leg(P, stream, dev, peak):
     """The variable-viscosity collisions (Sec. 1) on 16 FP32 members of
     512^2 (tau0 = 0.51): Smagorinsky (Cs = 0.1), eq. (7) and the entropic
     LBM (its per-cell root of the entropy condition) on the vectorised
-    kernel.  Every step moves 72 algorithmic bytes per update.  Median of
+    kernel.  An update moves 72 algorithmic bytes over the steps of a launch.  Median of
     five timed 40-step runs."""
     n, M, steps = 512, 16, 40
     fields = li.random_phase(n, seed=4000, u_rms=0.02)
@@ -459,13 +470,13 @@ def collision_models_leg(P, stream, dev, peak):
         lat.step(20)
         secs = median_timed(stream, lambda: lat.step(steps))
         lu = M * n * n * steps
-        gbs = BYTES_PER_LU_F32 * lu / secs / 1e9
+        gbs = bytes_per_lu_f32(lat) * lu / secs / 1e9
         out[name] = {"glups": lu / secs / 1e9, "achieved_gbs": gbs, "frac": gbs / peak,
-                     "kernel": "k_step_f32_vec (entropic)" if coll == 3 else "k_step_f32_vec (extended)",
+                     "kernel": step_kernel_name(lat) + (" (entropic)" if coll == 3 else " (extended)"),
                      "bound": "hbm"}
         if coll == 3:  # the entropic root keeps the issue slots busy: ALU-bound
             out[name].update({"bound": "alu", "hbm_frac": gbs / peak})
-            wi = issue_counts().get("k_step_f32_vec (entropic)")
+            wi = issue_counts().get(out[name]["kernel"])
             if wi is not None:
                 rate = wi * lu / secs
                 pk = issue_peak(dev.index or 0)
@@ -732,12 +743,13 @@ def forced_sweep_leg(P, stream, dev, peak):
     event_s = c.elapsed_time(d) / 1e3
     tot = sum(cells)
     glups = tot / pure_s / 1e9
-    gbs = BYTES_PER_LU_F32 * glups
+    bpl = bytes_per_lu_f32(lat)
+    gbs = bpl * glups
     lat.close()
     return {"members": len(mem), "cells": tot, "glups": glups,
             "per_member_glups": [{"n": m["n"], "tau": m["tau"], "glups": c_ / pure_s / 1e9}
                                  for m, c_ in zip(mem, cells)],
-            "bytes_per_lu": BYTES_PER_LU_F32, "achieved_gbs": gbs, "frac": gbs / peak,
+            "bytes_per_lu": bpl, "achieved_gbs": gbs, "frac": gbs / peak,
             "diagnostic_event_ms_all_origins": 1e3 * event_s, "sizes": list(wl["Ls"]),
             "glups_with_diagnostic": tot * PERIOD / (period_s + event_s) / 1e9}
 
@@ -774,11 +786,12 @@ def large_grid_leg(P, stream, dev, peak):
     assert np.all(np.isfinite(st[:, 2:, 0]))
     pure_s = a.elapsed_time(b) / 1e3 / (D - 3)
     glups = n * n / pure_s / 1e9
-    gbs = BYTES_PER_LU_F32 * glups
+    bpl = bytes_per_lu_f32(lat)
+    gbs = bpl * glups
     event_s = c.elapsed_time(d) / 1e3
     period_s = a.elapsed_time(c) / 1e3
     lat.close()
-    return {"grid": [n, n], "glups": glups, "bytes_per_lu": BYTES_PER_LU_F32,
+    return {"grid": [n, n], "glups": glups, "bytes_per_lu": bpl,
             "achieved_gbs": gbs, "frac": gbs / peak, "sizes": list(wl["Ls"]),
             "diagnostic_event_ms_all_origins": 1e3 * event_s,
             "boxes_per_event": n * n * len(wl["Ls"]),
@@ -1162,7 +1175,9 @@ def run_ours(args):
     kern_s = pure / (args.steps * PURE_STEPS)
     step_glups = M * n * n / kern_s / 1e9
     peak, peak_kind = measured_peaks()
-    achieved = BYTES_PER_LU_F32 * M * n * n / kern_s / 1e9
+    # per launch of `spl` steps: kern_s is the time of one step
+    spl, kernel = lat.steps_per_launch, step_kernel_name(lat)
+    achieved = bytes_per_lu_f32(lat) * M * n * n / kern_s / 1e9
 
     # one diagnostic event of all members on its own: the Table 1 boxes of the
     # timed steps, and every periodic origin (2.1 M boxes per member)
@@ -1262,19 +1277,19 @@ def run_ours(args):
         cpu = cpu_baseline_all_cores()
 
     if rank == 0:
-        traffic = profiled_traffic()
+        traffic = profiled_traffic() if spl == 1 else None
         line = {
             "metric": METRIC, "value": value, "unit": "GLUPS", "n_gpus": ws,
             "steps": args.steps, "warmup": args.warmup,
             "ms_per_step": 1e3 * elapsed / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": workload_config(),
-            "roofline": {"bound": "hbm", "kernel": "k_step_f32_vec", "achieved": achieved,
+            "roofline": {"bound": "hbm", "kernel": kernel, "achieved": achieved,
                          "peak": peak, "peak_kind": peak_kind, "unit": "GB/s",
                          "frac": achieved / peak,
                          "traffic": traffic,
                          "algorithmic_bytes_per_launch": BYTES_PER_LU_F32 * M * n * n,
-                         "avg_launch_ms": kern_s * 1e3},
+                         "steps_per_launch": spl, "avg_launch_ms": kern_s * spl * 1e3},
             "step_only_glups_per_gpu": step_glups,
             "diagnostic_event_ms": dict(diag_ms, members=M, sizes=list(Ls)),
             "fp64_plain_single_instance": {"glups": fp64_glups, "grid": [n, n],

@@ -5,7 +5,7 @@
 //
 // Storage: double buffer, pull layout pop[b][l][z][y][x] (x fastest): the
 // pre-collision f_l(x, n) = pop[cur][l][x - c_l].  FP32 stores deviations
-// g = f - t rho0, FP64 f.  One thread per cell; one launch per member.
+// g = f - t rho0, FP64 f.
 //
 // Diagnostic (FP64 arithmetic): snapshots (rho, j_x, j_y, j_z) of the levels
 // n, n-1, n-2 (FP32 storage: compensated sums of the FP32 populations, so

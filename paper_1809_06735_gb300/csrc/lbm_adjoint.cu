@@ -19,7 +19,9 @@
 //   eps = -nu rho S_ij G_ij, G_ij = D_j u_i, S_ij = G_ij + G_ji,
 //   u = (j + F/2)/rho, F = F_ext - alpha j, nu = (tau - 1/2)/3,
 // whose adjoint uses D^T = -D (antisymmetric periodic eq. (18) stencil).
-// All arithmetic is FP64; reductions are block-deterministic.
+// The step's adjoint is formed in 64-bit fixed point (the FP64 pipe is narrow)
+// with FP64 as the fallback, the objective in FP64; reductions are
+// block-deterministic.
 #include <algorithm>
 #include <cmath>
 
