@@ -130,3 +130,25 @@ def test_refusals(P):
     lat.set_launch(8, 1)
     assert lat.steps_per_launch == 1
     lat.close()
+
+
+@pytest.mark.parametrize("forced", [False, True])
+@pytest.mark.parametrize("T,rows", [(2, 8), (3, 27), (4, 100)])
+def test_entropic_far_cells_at_the_rim(P, T, rows, forced):
+    """Cells whose root is iterated in rows that no warp width divides and in
+    strips with halos: lanes past the row and the rims of the strips iterate
+    nothing, every stored cell does."""
+    kw = dict(force_kind=1, kf=2, F0=1e-5, alpha=1e-4) if forced else {}
+    grids = ((132, 70), (392, 33), (1500, 20), (4, 40))
+    members = [P.Member(nx, ny, 0.52, collision=3, **kw) for nx, ny in grids]
+    a, b = _pair(P, members, T, rows)
+    for lat in (a, b):
+        for m, (nx, ny) in enumerate(grids):
+            lat.set_populations(m, li.random_populations(nx, ny, seed=m, rel_noise=0.04))
+    for n in (1, 2, 3, 5):
+        a.step(n)
+        b.step(n)
+        for m in range(len(grids)):
+            assert np.array_equal(a.get_populations_host(m), b.get_populations_host(m)), (n, m)
+    a.close()
+    b.close()
