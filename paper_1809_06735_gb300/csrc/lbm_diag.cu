@@ -1724,10 +1724,10 @@ __global__ void __launch_bounds__(256, 3) k_query(const DiagJob *__restrict__ jo
   }
   double *pq = J.part + kPartQuery;
   if (mpart)
-    block_sum_store_mt<kQStats, MT>(acc, pq + (((size_t)iL * 3 + 2) * qb + blockIdx.x) * kQStats);
+    block_sum_store_mt<kQStats, MT>(acc, pq + (((size_t)iL * 3 + 2) * kMaxQueryBlocks + blockIdx.x) * kQStats);
   else
-    block_sum_store_pairs<kQStats, MT>(acc, pq + (((size_t)iL * 3 + 0) * qb + blockIdx.x) * kQStats,
-                                       pq + (((size_t)iL * 3 + 1) * qb + blockIdx.x) * kQStats);
+    block_sum_store_pairs<kQStats, MT>(acc, pq + (((size_t)iL * 3 + 0) * kMaxQueryBlocks + blockIdx.x) * kQStats,
+                                       pq + (((size_t)iL * 3 + 1) * kMaxQueryBlocks + blockIdx.x) * kQStats);
   if constexpr (EXT) {
     __syncthreads();
     const int ng = mpart ? 1 : 2;
@@ -1947,7 +1947,7 @@ __global__ void __launch_bounds__(256, 2)
     query_column<MT, PER_BOX, EXT, 1>(J, iL, grp, blk, nblk_x, ag, sedge, shist, ne, per_box, acc);
   else
     query_column<MT, PER_BOX, EXT, 6>(J, iL, grp, blk, nblk_x, ag, sedge, shist, ne, per_box, acc);
-  double *out = J.part + kPartQuery + (((size_t)iL * 3 + grp) * qb + blk) * kQStats;
+  double *out = J.part + kPartQuery + (((size_t)iL * 3 + grp) * kMaxQueryBlocks + blk) * kQStats;
   if constexpr (sizeof(MT) == 8)
     block_sum_f64<kQStats>(acc, out);
   else
@@ -1981,7 +1981,7 @@ __global__ void k_stats_final(const DiagJob *__restrict__ jobs, double *stats, d
   if (q < ngrp * kQStats) {
     const int grp = q / kQStats, slot = q % kQStats;
     for (int b = j; b < nblocks; b += 8)
-      a += partials[(((size_t)iL * 3 + grp) * nblocks + b) * kQStats + slot];
+      a += partials[(((size_t)iL * 3 + grp) * kMaxQueryBlocks + b) * kQStats + slot];
     sh[q][j] = a;
   }
   __syncthreads();

@@ -68,3 +68,15 @@ def test_distributions_equal_the_list(P):
     assert np.all(a["mach_hist"].sum(-1) == 131 * 77)
     np.testing.assert_allclose(a["mach"], b["mach"], rtol=1e-5, atol=1e-9)
     lat.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(1000, 1000), (512, 512), (260, 260)])
+def test_sizes_together_equal_sizes_alone(P, nx, ny):
+    """Sizes of nearly the whole grid use another number of CTAs than the
+    rest: the partial sums of one size must not reach another's.  FP32: the
+    CTAs of a size do not depend on the other sizes, so the same bits."""
+    lat = _lattice(P, nx, ny, 32)
+    Ls = [2, 10, nx // 3, nx - 1, nx]
+    s = lat.subvolume_balance(0, Ls)
+    for i, L in enumerate(Ls):
+        assert np.array_equal(s[i], lat.subvolume_balance(0, [L])[0], equal_nan=True), L
