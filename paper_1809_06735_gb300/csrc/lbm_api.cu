@@ -390,15 +390,18 @@ int launch_one_step(lbm_handle *h, cudaStream_t s, int cur) {
                                 s));
   if (h->scalar_members.size() == 1) {
     const int m = h->scalar_members[0];
-    CK(lbm::launch_step_scalar(h->precision, h->d_members, m, h->mcfg[m].nx, h->mcfg[m].ny, cur, s));
+    CK(lbm::launch_step_scalar(h->precision, h->d_members, m, h->mcfg[m].nx, h->mcfg[m].ny, cur,
+                               h->hm[m].fixed.step, s));
   } else if (!h->scalar_members.empty()) {
     int nx = 1, ny = 1;
+    bool fixed = false;
     for (int m : h->scalar_members) {
       nx = std::max(nx, h->mcfg[m].nx);
       ny = std::max(ny, h->mcfg[m].ny);
+      fixed |= h->hm[m].fixed.step != 0;
     }
     CK(lbm::launch_step_scalar_batch(h->precision, h->d_members, h->scalar_members.data(),
-                                     (int)h->scalar_members.size(), nx, ny, cur, s));
+                                     (int)h->scalar_members.size(), nx, ny, cur, fixed, s));
   }
   return LBM_OK;
 }
@@ -595,7 +598,10 @@ int autotune(lbm_handle *h) {
   // two and four steps on the fastest of these shapes
   struct Multi { int T, rows, gmax; float ms; };
   Multi multi{1, 0, 0, 1e30f};
-  if (rc == LBM_OK && multi_eligible(h)) {
+  // Not the entropic collision: once some cells iterate their root (0.1% of 23
+  // members of 392 x 665) it takes 405 to 436 us per step, single steps 152;
+  // with none at best 10% less than single steps (16 x 512^2: 57 against 63).
+  if (rc == LBM_OK && multi_eligible(h) && !h->has_elbm) {
     // one warm-up launch and 2 to 6 timed ones, about 2 ms where that is enough
     auto time_multi = [&](Multi &c) -> int {
       if (int rc2 = build_multi(h, c.T, c.rows, c.gmax)) return rc2;
@@ -846,6 +852,11 @@ int lbm_create(const lbm_config *cfg, void *workspace, size_t bytes, lbm_handle 
       B.om9h = (long long)(((unsigned __int128)B.om * 4 + 4) / 9);
       B.alpha = B.ok ? std::llrint(std::ldexp(c.alpha, 64)) : 0;
       B.forced = c.force_kind != 0 || c.alpha != 0.0;
+      // Small grids keep the FP64 form: the symmetric flows they are run with
+      // (Taylor-Green) amplify a change of the step's rounding until the
+      // balancing errors move by 1e-9 (64^2, 100 steps), more than results
+      // may.  The persistent kernel takes the same sizes.
+      B.step = es == 8 && B.ok && (long long)c.nx * c.ny >= lbm::kPersistMaxCells;
     }
     h->hm.push_back(M);
     // Kolmogorov tables: F_ext,x(y) = F0 sin(2 pi kf y / ny), F_ext,y(x) likewise.
@@ -1365,7 +1376,7 @@ int balance_members(lbm_handle *h, const int *members, int nm, const int *L, int
     J.qblocks = lbm::diag_query_blocks(hm.nx, hm.ny, maxb[i], origins != nullptr, batch_jobs, J.nL,
                                        h->diag_precision == 64);
     J.qwhole = lbm::diag_whole_blocks(hm.nx * hm.ny, batch_jobs);
-    for (int q : where[i]) J.any_whole |= !origins && lbm::diag_whole_box(L[q], hm.nx, hm.ny);
+    for (int q : where[i]) J.any_whole |= !origins && lbm::diag_whole_box(L[q], hm.nx, hm.ny, h->diag_precision == 64);
     J.force_kind = hm.force_kind;
     if (hm.collision != 0) {  // local viscosity recorded with the snapshot at n
       const size_t N = (size_t)hm.nx * hm.ny;
@@ -1600,7 +1611,7 @@ int lbm_record_trajectory(lbm_handle *h, int member, int nstates, double *states
     if ((rc = wait_diag(h))) return rc;
     for (int k = 0; k + 1 < nstates; ++k) {
       CK(lbm::launch_step_scalar(h->precision, h->d_members, member, c.nx, c.ny, h->cur,
-                                 h->stream, states + (size_t)k * 9 * N));
+                                 h->hm[member].fixed.step, h->stream, states + (size_t)k * 9 * N));
       h->launches += 1;
       h->cur ^= 1;
       h->t += 1;

@@ -108,9 +108,13 @@ __host__ __device__ inline size_t planar_stride(int nx, int ny) {
 // Sizes of nearly the whole grid in both directions: their boxes are almost
 // equal, so their standard deviation is what the sums' rounding leaves of a
 // difference of two equal numbers.  k_query takes them for every origin too,
-// whose order of summation that value then stays that of an origin list.
-__host__ __device__ inline bool whole_grid_box(int L, int nx, int ny) {
-  return 20LL * L > 19LL * nx && 20LL * L > 19LL * ny;
+// whose order of summation that value then stays that of an origin list.  So
+// does every size of a small grid with FP64 terms, whose few columns leave
+// k_query_all's threads waiting on the FP64 pipe (64^2, 4 sizes: 59 against
+// 13.5 us).
+__host__ __device__ inline bool whole_grid_box(int L, int nx, int ny, bool f64) {
+  return (f64 && (long long)nx * ny < kPersistMaxCells) ||
+         (20LL * L > 19LL * nx && 20LL * L > 19LL * ny);
 }
 
 __device__ __forceinline__ int wr(int i, int n) {
@@ -1558,7 +1562,7 @@ __global__ void __launch_bounds__(256, 3) k_query(const DiagJob *__restrict__ jo
   const int iL = blockIdx.y;
   const int qb = planar ? J.qwhole : J.qblocks;
   if (iL >= J.nL || (int)blockIdx.x >= qb) return;
-  if (planar && !whole_grid_box(J.meta[8 * iL], J.nx, J.ny)) return;
+  if (planar && !whole_grid_box(J.meta[8 * iL], J.nx, J.ny, sizeof(MT) == 8)) return;
   const int grp = mpart ? 2 : (int)(threadIdx.x & 1), k0 = 6 * grp;
   const int slot = mpart ? (int)threadIdx.x : (int)(threadIdx.x >> 1);
   const int per_pass = mpart ? 256 : 128;
@@ -1925,7 +1929,7 @@ __global__ void __launch_bounds__(256, 2)
   constexpr int NG = EXT ? 3 : 2;
   const DiagJob &J = jobs[blockIdx.z / NG];
   const int grp = blockIdx.z % NG, iL = blockIdx.x, blk = blockIdx.y, qb = J.qblocks;
-  if (iL >= J.nL || blk >= qb || whole_grid_box(J.meta[8 * iL], J.nx, J.ny)) return;
+  if (iL >= J.nL || blk >= qb || whole_grid_box(J.meta[8 * iL], J.nx, J.ny, sizeof(MT) == 8)) return;
   __shared__ MT sedge[EXT ? kDiagMaxEdges : 1];
   __shared__ unsigned shist[EXT ? kDiagMaxEdges + 1 : 1];
   int ne = 0;
@@ -1971,7 +1975,7 @@ __global__ void k_stats_final(const DiagJob *__restrict__ jobs, double *stats, d
   const int iL = blockIdx.x;
   if (iL >= J.nL) return;
   const int nblocks =
-      planar && whole_grid_box(J.meta[8 * iL], J.nx, J.ny) ? J.qwhole : J.qblocks;
+      planar && whole_grid_box(J.meta[8 * iL], J.nx, J.ny, sizeof(MT) == 8) ? J.qwhole : J.qblocks;
   const double *partials = J.part + kPartQuery;
   const QConst *consts = reinterpret_cast<const QConst *>(J.part + kPartConsts);
   const int q = threadIdx.x >> 3, j = threadIdx.x & 7;  // q = grp * 14 + slot
@@ -2203,7 +2207,7 @@ int diag_query_blocks(int nx, int ny, int max_boxes, bool origin_list, int batch
   return diag_list_blocks(max_boxes, 1024, batch_jobs);
 }
 int diag_whole_blocks(int boxes, int batch_jobs) { return diag_list_blocks(boxes, 4096, batch_jobs); }
-bool diag_whole_box(int L, int nx, int ny) { return whole_grid_box(L, nx, ny); }
+bool diag_whole_box(int L, int nx, int ny, bool f64) { return whole_grid_box(L, nx, ny, f64); }
 
 size_t diag_slot_doubles(size_t Nmax, size_t pad) {
   // snapshot slots + term-stage fields + kNT padded tables, in whole 256-byte

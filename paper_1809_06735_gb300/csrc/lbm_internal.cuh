@@ -38,7 +38,8 @@ struct FixedBgk {
   int k, ok;           // ok: the member can take it (BGK, moderate parameters)
   long long om, om9, om9h;  // omega 2^62, omega / 9 2^65 and 2^64
   long long alpha;     // drag 2^64
-  int forced, pad;     // forced: a force or drag
+  int forced;          // a force or drag
+  int step;            // the step takes it: grids from kPersistMaxCells up
 };
 
 // Per-member parameters, uploaded once into the workspace.
@@ -256,12 +257,13 @@ cudaError_t launch_step_f32_vec_snap(const Member *d_members, const Tile *d_tile
 // rec (optional): the member's public state before the step, FP64
 // [9][ny][nx] (the values lbm_get_populations returns), written by the step.
 cudaError_t launch_step_scalar(int precision, const Member *d_members, int member,
-                               int nx, int ny, int cur, cudaStream_t s, double *rec = nullptr);
+                               int nx, int ny, int cur, bool fixed, cudaStream_t s, double *rec = nullptr);
 struct InitList;
 // The general kernel for the members members[0..n) (host array), one launch
 // per 256 members, grid sized for nx_max x ny_max.
 cudaError_t launch_step_scalar_batch(int precision, const Member *d_members, const int *members,
-                                     int n, int nx_max, int ny_max, int state, cudaStream_t s);
+                                     int n, int nx_max, int ny_max, int state, bool fixed,
+                                     cudaStream_t s);
 // Grid-wide barrier words of the persistent small-grid step (device memory,
 // zeroed by each launch): arrival count, generation, error flag.
 struct GridSync {
@@ -363,7 +365,7 @@ struct DiagJob {
 int diag_query_blocks(int nx, int ny, int max_boxes, bool origin_list, int batch_jobs, int nL,
                       bool f64);
 int diag_whole_blocks(int boxes, int batch_jobs);
-bool diag_whole_box(int L, int nx, int ny);
+bool diag_whole_box(int L, int nx, int ny, bool f64);
 // Doubles of one field slot and of one partials slot for members of at most
 // Nmax cells and nx + 7 ny + 7 <= pad.
 size_t diag_slot_doubles(size_t Nmax, size_t pad);

@@ -353,7 +353,7 @@ cudaError_t launch_step_f32_vec_snap(const Member *d_members, const Tile *d_tile
 // one, which a stale L1 line of this SM could otherwise shadow.  The
 // arithmetic is the same either way.  rec (optional): the public state
 // before the step, FP64 [9][ny][nx], as k_get_pop writes it.
-template <typename T, bool L2ONLY>
+template <typename T, bool L2ONLY, bool FIXED>
 __device__ __forceinline__ void step_cell(const Member &M, int state, int x, int y,
                                           double *rec = nullptr) {
   const T *src = static_cast<const T *>(state_buffer(M, state));
@@ -388,8 +388,13 @@ __device__ __forceinline__ void step_cell(const Member &M, int state, int x, int
       rec[(size_t)l * N + (size_t)y * M.nx + x] = v;
     }
   }
-  if constexpr (sizeof(T) == 8) {
-    if (!M.fixed.ok || !collide_fixed(f, M.fixed, fx, fy)) {
+  if constexpr (sizeof(T) == 8 && !FIXED) {
+    if (M.collision == 3)
+      collide_elbm<double>(f, 0.0, M.tau, fx, fy, M.alpha);
+    else
+      collide_f64(f, M.omega, fx, fy, M.alpha, M.collision, M.tau, M.Cs);
+  } else if constexpr (sizeof(T) == 8) {
+    if (!M.fixed.step || !collide_fixed(f, M.fixed, fx, fy)) {
       double g[kQ];  // read again: the fixed-point form keeps no copy
 #pragma unroll
       for (int l = 0; l < kQ; ++l) {
@@ -423,15 +428,16 @@ __device__ __forceinline__ void step_cell(const Member &M, int state, int x, int
 // NT threads per CTA, at least MB CTAs per SM: FP64 grids from 2^17 cells up
 // take 3 x 256 threads (80 registers; 512^2 unforced 12.3 us against 13.7
 // with 116), smaller ones as many registers as the compiler likes (256^2:
-// 5.95 against 6.20 us).
-template <typename T, int NT, int MB>
+// 5.95 against 6.20 us).  FIXED: some member takes the fixed-point collision;
+// without one the FP64 form is compiled in line.
+template <typename T, int NT, int MB, bool FIXED = false>
 __global__ void __launch_bounds__(NT, MB) k_step_scalar(const Member *__restrict__ members, int member, int state,
                               double *rec) {
   const Member &M = members[member];
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   if (x >= M.nx || y >= M.ny) return;
-  step_cell<T, false>(M, state, x, y, rec);
+  step_cell<T, false, FIXED>(M, state, x, y, rec);
 }
 
 // ---------------------------------------------------------------------------
@@ -487,7 +493,7 @@ __global__ void __launch_bounds__(kPersistThreads)
   unsigned target = 0;
   for (int n = 0; n < nsteps; ++n) {
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < N; c += gridDim.x * blockDim.x)
-      step_cell<T, true>(M, state, c % M.nx, c / M.nx);
+      step_cell<T, true, false>(M, state, c % M.nx, c / M.nx);
     state ^= 1;  // 0 <-> 1 (double buffer), 2 <-> 3 (AA phases)
     if (n + 1 < nsteps && !grid_barrier(gs, gridDim.x, target)) return;
   }
@@ -498,14 +504,14 @@ __global__ void __launch_bounds__(kPersistThreads)
 // CTAs return at once), so a step of many general-kernel members (the
 // entropic collision, FP64 ensembles, nx % 4 != 0) fills the GPU without a
 // partial wave per member.
-template <typename T, int NT, int MB>
+template <typename T, int NT, int MB, bool FIXED = false>
 __global__ void __launch_bounds__(NT, MB) k_step_scalar_multi(const Member *__restrict__ members, InitList list,
                                     int state) {
   const Member &M = members[list.m[blockIdx.z]];
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   if (x >= M.nx || y >= M.ny) return;
-  step_cell<T, false>(M, state, x, y);
+  step_cell<T, false, FIXED>(M, state, x, y);
 }
 
 static dim3 grid2d(int nx, int ny, dim3 b) {
@@ -576,7 +582,8 @@ cudaError_t launch_step_scalar_persistent(int precision, const Member *d_members
 }
 
 cudaError_t launch_step_scalar_batch(int precision, const Member *d_members, const int *members,
-                                     int n, int nx_max, int ny_max, int state, cudaStream_t s) {
+                                     int n, int nx_max, int ny_max, int state, bool fixed,
+                                     cudaStream_t s) {
   const dim3 b = (long long)nx_max * ny_max < (1LL << 15) ? dim3(32, 2) : dim3(64, 4);
   for (int i0 = 0; i0 < n; i0 += InitList::kMax) {
     InitList list;
@@ -587,15 +594,17 @@ cudaError_t launch_step_scalar_batch(int precision, const Member *d_members, con
     if (precision == 32)
       k_step_scalar_multi<float, 256, 4><<<g, b, 0, s>>>(d_members, list, state);
     else if (b.x == 32)
-      k_step_scalar_multi<double, 64, 1><<<g, b, 0, s>>>(d_members, list, state);
+      (fixed ? k_step_scalar_multi<double, 64, 1, true> : k_step_scalar_multi<double, 64, 1>)<<<g, b, 0, s>>>
+          (d_members, list, state);
     else
-      k_step_scalar_multi<double, 256, 3><<<g, b, 0, s>>>(d_members, list, state);
+      (fixed ? k_step_scalar_multi<double, 256, 3, true> : k_step_scalar_multi<double, 256, 1>)<<<g, b, 0, s>>>
+          (d_members, list, state);
   }
   return cudaGetLastError();
 }
 
 cudaError_t launch_step_scalar(int precision, const Member *d_members, int member, int nx,
-                               int ny, int state, cudaStream_t s, double *rec) {
+                               int ny, int state, bool fixed, cudaStream_t s, double *rec) {
   // one thread per cell; grids below 2^17 cells get 64-thread CTAs, so that
   // their FP64 arithmetic (slow on this part) spreads evenly over the SMs
   // (256^2 FP64: 16.9 against 18.2 us per step with 256-thread CTAs in 1.7
@@ -605,9 +614,11 @@ cudaError_t launch_step_scalar(int precision, const Member *d_members, int membe
   if (precision == 32)
     k_step_scalar<float, 256, 4><<<g, b, 0, s>>>(d_members, member, state, rec);
   else if (small)
-    k_step_scalar<double, 64, 1><<<g, b, 0, s>>>(d_members, member, state, rec);
+    (fixed ? k_step_scalar<double, 64, 1, true> : k_step_scalar<double, 64, 1>)<<<g, b, 0, s>>>
+          (d_members, member, state, rec);
   else
-    k_step_scalar<double, 256, 3><<<g, b, 0, s>>>(d_members, member, state, rec);
+    (fixed ? k_step_scalar<double, 256, 3, true> : k_step_scalar<double, 256, 1>)<<<g, b, 0, s>>>
+          (d_members, member, state, rec);
   return cudaGetLastError();
 }
 

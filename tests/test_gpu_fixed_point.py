@@ -70,3 +70,25 @@ def test_non_finite_cells_spread_as_before(P):
     want[7:10, 7:10] = want[19:22, 19:22] = True
     assert np.array_equal(bad, want)
     lat.close()
+
+
+@pytest.mark.parametrize("rho0", [1.0, 1.999, 0.75, 3e-5, 4.1e6])
+@pytest.mark.parametrize("grids", [[(255, 128)], [(256, 128)], [(331, 103)], [(40, 30), (256, 128)]])
+def test_both_sides_of_the_size_rule(P, orc, rho0, grids):
+    """Grids below 2^15 cells take the FP64 form, those from it up the fixed
+    point, also side by side in one launch; a few cells are outside its range.
+    1e-12 of the cells' density, as above."""
+    mem = [P.Member(nx, ny, 0.56, rho0, 1, 2, 3e-4 * rho0, 1e-3) for nx, ny in grids]
+    lat = P.Lattice(mem, precision=64)
+    f0 = []
+    for m, (nx, ny) in enumerate(grids):
+        f = rho0 * li.random_populations(nx, ny, seed=m, rel_noise=0.02)
+        f[5, 3, :4] = 1e-7 * rho0
+        f[0, 15, 4] = 3.0 * rho0
+        f0.append(f)
+        lat.set_populations(m, f)
+    lat.step(5)
+    for m, f in enumerate(f0):
+        ref = orc.run(f, 5, 0.56, orc.Force(1, 3e-4 * rho0, 2, 1e-3))
+        assert np.max(np.abs(lat.get_populations_host(m) - ref)) < 1e-12 * np.max(f.sum(0))
+    lat.close()
