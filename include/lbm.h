@@ -218,8 +218,10 @@ long long lbm_kernels_per_step(const lbm_handle *h);
  * the populations and the storage are kept): for the batched FP32 kernel
  * warps 1..8 per CTA, rows 1, 2 or 4 per warp and grid CTAs (0: one CTA per
  * tile); proj_rows 1..64 rows per thread of the FP32 eq. (16) projection
- * (force kind 2, nx % 4 == 0: a CTA covers 128 x 8 proj_rows cells), 0 to
- * keep the current value.  Results do not depend on any of these.
+ * (force kind 2, nx % 4 == 0: whole groups of 8 rows, so a CTA covers 128 x
+ * 64 ceil(proj_rows / 8) cells), 0 to keep the current value.  Results do not
+ * depend on any of these, but for collisions 1 and 2: there the last bits
+ * depend on the storage and on the rows per warp.
  * LBM_ERR_ARG for other values, with the previous configuration kept. */
 int lbm_set_launch(lbm_handle *h, int warps, int rows, int grid, int proj_rows);
 

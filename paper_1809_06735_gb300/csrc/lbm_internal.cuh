@@ -223,7 +223,8 @@ struct LaunchCfg {
                       // collision (with any other collision), those members
                       // without force and drag; 4 the same with any force
   int proj_rows;      // rows per thread of the FP32 four-cell projection (force
-                      // kind 2): a block covers 128 x 8 proj_rows cells
+                      // kind 2), in whole groups of 8: a block covers 128 x 64
+                      // cells per group
 };
 
 // One warp of the several-steps kernel (lbm_multi.cu): the columns [x0, xend)

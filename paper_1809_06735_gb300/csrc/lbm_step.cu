@@ -802,16 +802,17 @@ __global__ void k_snapshot_ring(const Member *__restrict__ members, int state, i
   }
 }
 
-// The member's last projection CTA to finish (a counter in
+// The member's last of `nctas` projection CTAs to finish (a counter in
 // Member::proj_count; the caller wrote its partials and fenced) reduces the
-// nblk CTA partials in a fixed order into the damping coefficients and, for
+// nblk partials in a fixed order into the damping coefficients and, for
 // the running step of FP32 storage, the per-row factors.  Every thread of
 // the CTA calls it (256 threads: tid, lane, wid of the CTA).
-__device__ void project_finalize(const Member &M, int nblk, int slot, int tid, int lane, int wid) {
+__device__ void project_finalize(const Member &M, int nctas, int nblk, int slot, int tid, int lane,
+                                 int wid) {
   const int nx = M.nx, ny = M.ny;
   __shared__ int is_last;
   __syncthreads();
-  if (tid == 0) is_last = atomicAdd(M.proj_count, 1u) == (unsigned)(nblk - 1);
+  if (tid == 0) is_last = atomicAdd(M.proj_count, 1u) == (unsigned)(nctas - 1);
   __syncthreads();
   if (!is_last) return;
   __threadfence();
@@ -941,12 +942,12 @@ __global__ void __launch_bounds__(256) k_project(const Member *__restrict__ memb
     M.proj_part[(size_t)blk * kDamp + tid] = (double)a;
     __threadfence();
   }
-  project_finalize(M, nblk, slot, tid, lane, wid);
+  project_finalize(M, nblk, nblk, slot, tid, lane, wid);
 }
 
 // FP32 projection with 4 consecutive cells per lane (every kind-2 member
 // with nx % 4 == 0): CTA (32, 8), a warp per 128-cell row segment, each
-// thread kProj4Rows rows 8 apart, so a CTA covers 128 x 8 kProj4Rows cells.
+// thread rows 8 apart in groups of kProj4Group, a CTA 128 x 64 cells per group.
 // The populations of the state are pulled as in k_step_f32_vec (MODE 0:
 // double buffer `state`, 1: AA even, 2: AA odd): one float4 per population
 // and lane, the x-shift by shuffles.  Same sums per cell as k_project.
@@ -1065,10 +1066,19 @@ __device__ __forceinline__ void proj4_moments(float rho0, const float4 (&o)[kQ],
   }
 }
 // Block (bx, by) of the projection of member M: cells [128 bx, 128 bx + 128)
-// x [8 prow by, 8 prow (by + 1)), CTA (32, 8), prow rows per thread.
-template <int MODE>
+// x [64 ng by, 64 ng (by + 1)), CTA (32, 8), ng groups of kProj4Group rows per
+// thread.  A group is what is summed in FP32: its sum, widened, is one partial
+// of the member, so the partials and with them the damping coefficients do not
+// depend on ng.  (With one partial per CTA, whatever its rows, the FP32 sums
+// were grouped as the tuner's choice of rows had it, and the statistics of 64 x
+// 256^2 differed by 7e-4 between two handles that had tuned differently.)
+constexpr int kProj4Group = 8;
+// ONE: ng is 1, without the group loop (its registers, up to 144, would leave
+// one CTA per SM: 64 x 256^2 13.2 against 12.9 ms per 100 steps).
+template <int MODE, bool ONE>
 __device__ __forceinline__ void proj4_block(const Member &M, int bx, int by, int state, int slot,
-                                            int prow) {
+                                            int ngroups) {
+  const int ng = ONE ? 1 : ngroups;
   const int nx = M.nx, ny = M.ny, lane = threadIdx.x;
   const int x = bx * 128 + 4 * lane;
   const bool active = x < nx;
@@ -1086,53 +1096,57 @@ __device__ __forceinline__ void proj4_block(const Member &M, int bx, int by, int
       s2x[i] = tr[3 * nx + x + i];
     }
   }
-  float acc[kDamp];
-#pragma unroll
-  for (int q = 0; q < kDamp; ++q) acc[q] = 0.f;
-  // software-pipelined over the thread's rows: the loads of the next row are
-  // issued before the mode sums of the current one
-  float4 o[kQ];
-  float e[kQ];
-  const int yb = by * 8 * prow + threadIdx.y;
-  if (yb < ny) proj4_load<MODE>(M, src, yb, x, xprev, xnext, active, last, lane, o, e);
-#pragma unroll 1
-  for (int r = 0; r < prow; ++r) {
-    const int y = yb + 8 * r;
-    if (y >= ny) break;  // whole warps
-    float rho[4], jx[4], jy[4];
-    proj4_moments<MODE>(M.rho0_f, o, e, active, last, lane, rho, jx, jy);
-    if (r + 1 < prow && y + 8 < ny)
-      proj4_load<MODE>(M, src, y + 8, x, xprev, xnext, active, last, lane, o, e);
-    if (active) proj_row_accumulate(M, rho, jx, jy, cx, sx, c2x, s2x, y, acc);
-  }
   __shared__ float sh[kDamp][8];
   const int tid = threadIdx.y * 32 + threadIdx.x, wid = threadIdx.y;
+  const int gx = (nx + 127) / 128, groups = (ny + 8 * kProj4Group - 1) / (8 * kProj4Group);
+  // software-pipelined over the thread's rows, across the groups too: the loads
+  // of the next row are issued before the mode sums of the current one
+  float4 o[kQ];
+  float e[kQ];
+  const int g0 = by * ng, g1 = ONE ? by + 1 : min(g0 + ng, groups);
+  int yb = g0 * 8 * kProj4Group + threadIdx.y;
+  if (yb < ny) proj4_load<MODE>(M, src, yb, x, xprev, xnext, active, last, lane, o, e);
+#pragma unroll 1
+  for (int g = g0; g < g1; ++g, yb += 8 * kProj4Group) {
+    float acc[kDamp];
 #pragma unroll
-  for (int q = 0; q < kDamp; ++q) {
-    float a = acc[q];
+    for (int q = 0; q < kDamp; ++q) acc[q] = 0.f;
+#pragma unroll 1
+    for (int r = 0; r < kProj4Group; ++r) {
+      const int y = yb + 8 * r;
+      if (y >= ny) break;  // whole warps
+      float rho[4], jx[4], jy[4];
+      proj4_moments<MODE>(M.rho0_f, o, e, active, last, lane, rho, jx, jy);
+      if ((r + 1 < kProj4Group || (!ONE && g + 1 < g1)) && y + 8 < ny)
+        proj4_load<MODE>(M, src, y + 8, x, xprev, xnext, active, last, lane, o, e);
+      if (active) proj_row_accumulate(M, rho, jx, jy, cx, sx, c2x, s2x, y, acc);
+    }
+    if (!ONE && g > g0) __syncthreads();  // the previous group's sums have been read
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-    if (lane == 0) sh[q][wid] = a;
+    for (int q = 0; q < kDamp; ++q) {
+      float a = acc[q];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+      if (lane == 0) sh[q][wid] = a;
+    }
+    __syncthreads();
+    if (tid < kDamp) {
+      float a = sh[tid][0];
+      for (int w = 1; w < 8; ++w) a += sh[tid][w];
+      M.proj_part[(size_t)(g * gx + bx) * kDamp + tid] = (double)a;
+    }
   }
-  __syncthreads();
-  const int gx = (nx + 127) / 128;
-  const int nblk = gx * ((ny + 8 * prow - 1) / (8 * prow));
-  if (tid < kDamp) {
-    float a = sh[tid][0];
-    for (int w = 1; w < 8; ++w) a += sh[tid][w];
-    M.proj_part[(size_t)(by * gx + bx) * kDamp + tid] = (double)a;
-    __threadfence();
-  }
-  project_finalize(M, nblk, slot, tid, lane, wid);
+  if (tid < kDamp) __threadfence();
+  project_finalize(M, gx * ((groups + ng - 1) / ng), gx * groups, slot, tid, lane, wid);
 }
 
-template <int MODE>
-__global__ void __launch_bounds__(256) k_project4(const Member *__restrict__ members, int state,
-                                                  int slot, int prow) {
+template <int MODE, bool ONE>
+__global__ void __launch_bounds__(256, 2) k_project4(const Member *__restrict__ members, int state,
+                                                     int slot, int ng) {
   const Member &M = members[blockIdx.z];
   if (M.force_kind != 2) return;
-  if ((int)(blockIdx.x * 128) >= M.nx || (int)(blockIdx.y * 8 * prow) >= M.ny) return;
-  proj4_block<MODE>(M, blockIdx.x, blockIdx.y, state, slot, prow);
+  if ((int)(blockIdx.x * 128) >= M.nx || (int)(blockIdx.y * 8 * kProj4Group * ng) >= M.ny) return;
+  proj4_block<MODE, ONE>(M, blockIdx.x, blockIdx.y, state, slot, ng);
 }
 
 
@@ -1311,14 +1325,15 @@ cudaError_t launch_projection(int precision, const Member *d_members, int n_memb
                               cudaStream_t s) {
   if (quad && precision == 32) {  // four cells per lane
     if (prow < 1) return cudaErrorInvalidValue;
-    dim3 g((nx_max + 127) / 128, (ny_max + 8 * prow - 1) / (8 * prow), n_members);
+    const int ng = (prow + kProj4Group - 1) / kProj4Group, rows = 8 * kProj4Group * ng;
+    dim3 g((nx_max + 127) / 128, (ny_max + rows - 1) / rows, n_members);
     const dim3 b4(32, 8);
     if (state < 2)
-      k_project4<0><<<g, b4, 0, s>>>(d_members, state, slot, prow);
+      (ng == 1 ? k_project4<0, true> : k_project4<0, false>)<<<g, b4, 0, s>>>(d_members, state, slot, ng);
     else if (state == 2)
-      k_project4<1><<<g, b4, 0, s>>>(d_members, state, slot, prow);
+      (ng == 1 ? k_project4<1, true> : k_project4<1, false>)<<<g, b4, 0, s>>>(d_members, state, slot, ng);
     else
-      k_project4<2><<<g, b4, 0, s>>>(d_members, state, slot, prow);
+      (ng == 1 ? k_project4<2, true> : k_project4<2, false>)<<<g, b4, 0, s>>>(d_members, state, slot, ng);
     return cudaGetLastError();
   }
   const dim3 b(64, 4);
