@@ -681,7 +681,7 @@ cudaError_t launch_obj_tiles(const Member *d_members, int member, int state, con
   return cudaGetLastError();
 }
 
-AGrid agrid(const Member &hm) {
+AGrid agrid(const Member &hm, const FixedBgk &fixed) {
   AGrid g;
   g.nx = hm.nx;
   g.ny = hm.ny;
@@ -694,7 +694,7 @@ AGrid agrid(const Member &hm) {
   g.F0 = hm.F0;
   g.fxt = hm.fx_tab64;
   g.fyt = hm.fy_tab64;
-  g.fixed = hm.fixed;
+  g.fixed = fixed;
   g.fixed.ok = g.fixed.ok && std::abs(g.fixed.k) < 100 && std::fabs(hm.omega - 1.0) < 1.0 - 1e-9;
   g.w1 = g.fixed.ok ? std::llrint(std::ldexp(hm.omega - 1.0, 63)) : 0;
   g.keep = -g.w1;
@@ -721,10 +721,10 @@ int adjoint_threads(size_t N) { return N < ((size_t)1 << 17) ? 64 : 256; }
 
 }  // namespace
 
-cudaError_t adjoint_step(const Member &hm, const double *f_n, const double *lam_in,
+cudaError_t adjoint_step(const Member &hm, const FixedBgk &fixed, const double *f_n, const double *lam_in,
                          double *lam_out, double w, int bx, int by, int L, double *dJ_dtau,
                          double *dJ_dF0, const DiagScratch &sc, cudaStream_t s) {
-  return adjoint_sweep(hm, f_n, 1, lam_in, lam_out, nullptr, &w, bx, by, L, dJ_dtau, dJ_dF0, sc, s,
+  return adjoint_sweep(hm, fixed, f_n, 1, lam_in, lam_out, nullptr, &w, bx, by, L, dJ_dtau, dJ_dF0, sc, s,
                        nullptr);
 }
 
@@ -738,12 +738,12 @@ int adjoint_kernel_count(double w) { return w != 0.0 ? 7 : 3; }
 // Each CTA keeps running sums of its (dJ/dtau, dJ/dF0) partials over the
 // whole sweep and one reduction at the end adds them into the accumulators;
 // the force-direction tables are built once.
-cudaError_t adjoint_sweep(const Member &hm, const double *states, int nstates,
+cudaError_t adjoint_sweep(const Member &hm, const FixedBgk &fixed, const double *states, int nstates,
                           const double *lam_in, double *lam_out, double *lam_tmp,
                           const double *weights, int bx, int by, int L, double *dJ_dtau,
                           double *dJ_dF0, const DiagScratch &sc, cudaStream_t s,
                           long long *launches) {
-  const AGrid g = agrid(hm);
+  const AGrid g = agrid(hm, fixed);
   const size_t N = (size_t)hm.nx * hm.ny;
   const int tpb = adjoint_threads(N), nb = nblocks_for(N, tpb);
   double *sines = sc.f, *fields = sc.f + (hm.nx + hm.ny);
@@ -808,7 +808,7 @@ cudaError_t adjoint_sweep(const Member &hm, const double *states, int nstates,
 cudaError_t objective_tiles(int precision, const Member *d_members, int member,
                             const Member &hm, int state, double w, int bx, int by, int L,
                             double *acc, const DiagScratch &sc, cudaStream_t s) {
-  const AGrid g = agrid(hm);
+  const AGrid g = agrid(hm, FixedBgk{});
   const double cw = w / ((double)L * (double)L);
   if (precision == 32)
     return launch_obj_tiles<float>(d_members, member, state, g, bx, by, L, cw, sc.partials,

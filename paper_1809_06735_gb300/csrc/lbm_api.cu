@@ -32,7 +32,7 @@ size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 thread_local std::string g_last_error = "no error";
 
 struct Layout {
-  size_t members, tiles, multi, status, sync;
+  size_t members, tiles, multi, fixed, status, sync;
   size_t multi_cap;  // entries of the several-steps table
   std::vector<size_t> pop0, pop1, fx, fy, fx64, fy64, snap;
   std::vector<size_t> ft, ft64, trig, trig64, damp, damp_f, damp_ring, proj, drows, pcount;
@@ -174,7 +174,6 @@ Layout make_layout(const lbm_config *cfg) {
   }
   // the several-steps kernel needs the two arrays of a double buffer
   if (cfg->storage == 1) L.multi_cap = 0;
-  L.multi = take(sizeof(MultiWarp) * std::max<size_t>(L.multi_cap, 1));
   L.tiles = take(sizeof(Tile) * std::max<size_t>(max_tiles, 1));
   L.status = take(sizeof(int) * n);
   L.sync = take(4 * sizeof(unsigned));  // persistent small-grid step: count, gen, err
@@ -231,6 +230,9 @@ Layout make_layout(const lbm_config *cfg) {
   L.out7 = take(8 * 8);
   L.origin_cap = std::max<size_t>(4 * L.Nmax, (size_t)1 << 20);
   L.origins = take(8 * L.origin_cap);
+  // last: the populations keep their place
+  L.multi = take(sizeof(MultiWarp) * std::max<size_t>(L.multi_cap, 1));
+  L.fixed = take(sizeof(lbm::FixedBgk) * n);
   L.total = off;
   return L;
 }
@@ -241,9 +243,11 @@ struct lbm_handle {
   lbm_config cfg;
   std::vector<lbm_member_cfg> mcfg;
   std::vector<Member> hm;
+  std::vector<lbm::FixedBgk> fixed;  // of each member
   Layout lay;
   char *ws = nullptr;
   Member *d_members = nullptr;
+  lbm::FixedBgk *d_fixed = nullptr;
   Tile *d_tiles = nullptr;
   int ntiles = 0;
   std::vector<int> scalar_members;
@@ -391,17 +395,18 @@ int launch_one_step(lbm_handle *h, cudaStream_t s, int cur) {
   if (h->scalar_members.size() == 1) {
     const int m = h->scalar_members[0];
     CK(lbm::launch_step_scalar(h->precision, h->d_members, m, h->mcfg[m].nx, h->mcfg[m].ny, cur,
-                               h->hm[m].fixed.step, s));
+                               h->fixed[m].step ? h->d_fixed : nullptr, s));
   } else if (!h->scalar_members.empty()) {
     int nx = 1, ny = 1;
     bool fixed = false;
     for (int m : h->scalar_members) {
       nx = std::max(nx, h->mcfg[m].nx);
       ny = std::max(ny, h->mcfg[m].ny);
-      fixed |= h->hm[m].fixed.step != 0;
+      fixed |= h->fixed[m].step != 0;
     }
     CK(lbm::launch_step_scalar_batch(h->precision, h->d_members, h->scalar_members.data(),
-                                     (int)h->scalar_members.size(), nx, ny, cur, fixed, s));
+                                     (int)h->scalar_members.size(), nx, ny, cur,
+                                     fixed ? h->d_fixed : nullptr, s));
   }
   return LBM_OK;
 }
@@ -760,6 +765,7 @@ int lbm_create(const lbm_config *cfg, void *workspace, size_t bytes, lbm_handle 
   h->stream = static_cast<cudaStream_t>(cfg->cuda_stream);
   h->graph_k = cfg->graph_steps > 0 ? (cfg->graph_steps + 1) / 2 * 2 : 0;
   h->d_members = reinterpret_cast<Member *>(ws_at(h, lay.members));
+  h->d_fixed = reinterpret_cast<lbm::FixedBgk *>(ws_at(h, lay.fixed));
   h->d_tiles = reinterpret_cast<Tile *>(ws_at(h, lay.tiles));
   h->d_multi = reinterpret_cast<MultiWarp *>(ws_at(h, lay.multi));
   h->sc.f = reinterpret_cast<double *>(ws_at(h, lay.scratch));
@@ -838,8 +844,8 @@ int lbm_create(const lbm_config *cfg, void *workspace, size_t bytes, lbm_handle 
       h->has_kind2 = true;
       if (h->precision != 32 || c.nx % 4 != 0) h->proj_quad = false;
     }
+    lbm::FixedBgk B{};
     if (c.collision == 0) {  // see collide_fixed; the adjoint of either precision uses it
-      lbm::FixedBgk &B = M.fixed;
       B.k = std::ilogb(c.rho0) + 2;
       B.om = std::llrint(std::ldexp(M.omega, 62));
       B.ok = B.k > -900 && B.k < 900 && std::fabs(c.alpha) < 0.25 && M.omega < 2.0 - 1e-9;
@@ -854,6 +860,7 @@ int lbm_create(const lbm_config *cfg, void *workspace, size_t bytes, lbm_handle 
       B.step = es == 8 && B.ok && (long long)c.nx * c.ny >= lbm::kPersistMaxCells;
     }
     h->hm.push_back(M);
+    h->fixed.push_back(B);
     // Kolmogorov tables: F_ext,x(y) = F0 sin(2 pi kf y / ny), F_ext,y(x) likewise.
     std::vector<double> fx(c.ny, 0.0), fy(c.nx, 0.0);
     if (c.force_kind == 1) {
@@ -896,6 +903,9 @@ int lbm_create(const lbm_config *cfg, void *workspace, size_t bytes, lbm_handle 
   }
   cudaError_t e = cudaMemcpyAsync(h->d_members, h->hm.data(), sizeof(Member) * h->hm.size(),
                                   cudaMemcpyHostToDevice, h->stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(h->d_fixed, h->fixed.data(), sizeof(lbm::FixedBgk) * h->fixed.size(),
+                        cudaMemcpyHostToDevice, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ws_at(h, lay.status), 0, sizeof(int) * cfg->n_members, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->sc.count, 0, sizeof(unsigned), h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
@@ -1557,7 +1567,7 @@ int lbm_adjoint_step(lbm_handle *h, int member, const double *f_n, const double 
       (L < 1 || L > c.nx || L > c.ny || bx < 0 || bx >= c.nx || by < 0 || by >= c.ny))
     return fail(h, LBM_ERR_ARG, "objective box outside the grid");
   if ((rc = wait_diag(h))) return rc;
-  CK(lbm::adjoint_step(h->hm[member], f_n, lambda_in, lambda_out, obj_weight, bx, by, L,
+  CK(lbm::adjoint_step(h->hm[member], h->fixed[member], f_n, lambda_in, lambda_out, obj_weight, bx, by, L,
                        dJ_dtau, dJ_dF0, h->sc, h->stream));
   h->launches += lbm::adjoint_kernel_count(obj_weight);
   return LBM_OK;
@@ -1606,7 +1616,7 @@ int lbm_record_trajectory(lbm_handle *h, int member, int nstates, double *states
     if ((rc = wait_diag(h))) return rc;
     for (int k = 0; k + 1 < nstates; ++k) {
       CK(lbm::launch_step_scalar(h->precision, h->d_members, member, c.nx, c.ny, h->cur,
-                                 h->hm[member].fixed.step, h->stream, states + (size_t)k * 9 * N));
+                                 h->fixed[member].step ? h->d_fixed : nullptr, h->stream, states + (size_t)k * 9 * N));
       h->launches += 1;
       h->cur ^= 1;
       h->t += 1;
@@ -1646,7 +1656,7 @@ int lbm_adjoint_sweep(lbm_handle *h, int member, const double *states, int nstat
   if (any_obj && (L < 1 || L > c.nx || L > c.ny || bx < 0 || bx >= c.nx || by < 0 || by >= c.ny))
     return fail(h, LBM_ERR_ARG, "objective box outside the grid");
   if ((rc = wait_diag(h))) return rc;
-  CK(lbm::adjoint_sweep(h->hm[member], states, nstates, lambda_in, lambda_out, lambda_tmp,
+  CK(lbm::adjoint_sweep(h->hm[member], h->fixed[member], states, nstates, lambda_in, lambda_out, lambda_tmp,
                         weights, bx, by, L, dJ_dtau, dJ_dF0, h->sc, h->stream, &h->launches));
   return LBM_OK;
 }

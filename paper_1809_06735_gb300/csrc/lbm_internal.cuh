@@ -32,7 +32,10 @@ __host__ __device__ constexpr int opposite(int l) {
   return l == 0 ? 0 : (l <= 4 ? ((l + 1) % 4) + 1 : ((l - 5 + 2) % 4) + 5);
 }
 
-// Constants of the fixed-point form of the FP64 collision (collide_fixed):
+// Constants of the fixed-point form of the FP64 collision (collide_fixed), one
+// per member and an array of their own: as a part of Member (328 bytes in place
+// of 280) they cost the FP32 steps 0.5% (16 x 512^2, Smagorinsky: 6.63 against
+// 6.59 ms per 100 steps).
 // k = exponent of rho0 plus two, so that rho0 lies in [1/4, 1/2) 2^k.
 struct FixedBgk {
   int k, ok;           // ok: the member can take it (BGK, moderate parameters)
@@ -81,7 +84,6 @@ struct Member {
   double Cs;
   void *nu_ring;         // local viscosity at each snapshot slot [3][N]
                          // (storage precision), collision != 0
-  FixedBgk fixed;
 };
 
 // Local relaxation time of a cell from its non-equilibrium stress
@@ -255,16 +257,19 @@ cudaError_t launch_step_f32_vec(const Member *d_members, const Tile *d_tiles, in
 cudaError_t launch_step_f32_vec_snap(const Member *d_members, const Tile *d_tiles, int ntiles,
                                      int state, int flip, const LaunchCfg &lc, int slot,
                                      cudaStream_t s);
+// fixed: the members' fixed-point constants (device, by member), or null where no
+// member steps in fixed point.
 // rec (optional): the member's public state before the step, FP64
 // [9][ny][nx] (the values lbm_get_populations returns), written by the step.
 cudaError_t launch_step_scalar(int precision, const Member *d_members, int member,
-                               int nx, int ny, int cur, bool fixed, cudaStream_t s, double *rec = nullptr);
+                               int nx, int ny, int cur, const FixedBgk *fixed, cudaStream_t s,
+                               double *rec = nullptr);
 struct InitList;
 // The general kernel for the members members[0..n) (host array), one launch
 // per 256 members, grid sized for nx_max x ny_max.
 cudaError_t launch_step_scalar_batch(int precision, const Member *d_members, const int *members,
-                                     int n, int nx_max, int ny_max, int state, bool fixed,
-                                     cudaStream_t s);
+                                     int n, int nx_max, int ny_max, int state,
+                                     const FixedBgk *fixed, cudaStream_t s);
 // Grid-wide barrier words of the persistent small-grid step (device memory,
 // zeroed by each launch): arrival count, generation, error flag.
 struct GridSync {
@@ -392,7 +397,7 @@ cudaError_t diag_balance(const DiagJob *jobs_host, const DiagJob *jobs_dev, int 
                          cudaStream_t s);
 
 // Adjoint (lbm_adjoint.cu).
-cudaError_t adjoint_step(const Member &hm, const double *f_n, const double *lam_in,
+cudaError_t adjoint_step(const Member &hm, const FixedBgk &fixed, const double *f_n, const double *lam_in,
                          double *lam_out, double w, int bx, int by, int L,
                          double *dJ_dtau, double *dJ_dF0, const DiagScratch &sc,
                          cudaStream_t s);
@@ -404,7 +409,7 @@ cudaError_t objective_tiles(int precision, const Member *d_members, int member,
 int adjoint_kernel_count(double w);
 // The adjoint steps of a recorded interval, last state first, with one
 // gradient reduction per call (weights: host array of nstates).
-cudaError_t adjoint_sweep(const Member &hm, const double *states, int nstates,
+cudaError_t adjoint_sweep(const Member &hm, const FixedBgk &fixed, const double *states, int nstates,
                           const double *lam_in, double *lam_out, double *lam_tmp,
                           const double *weights, int bx, int by, int L, double *dJ_dtau,
                           double *dJ_dF0, const DiagScratch &sc, cudaStream_t s,

@@ -355,7 +355,8 @@ cudaError_t launch_step_f32_vec_snap(const Member *d_members, const Tile *d_tile
 // before the step, FP64 [9][ny][nx], as k_get_pop writes it.
 template <typename T, bool L2ONLY, bool FIXED>
 __device__ __forceinline__ void step_cell(const Member &M, int state, int x, int y,
-                                          double *rec = nullptr) {
+                                          double *rec = nullptr,
+                                          const FixedBgk *fixed = nullptr) {
   const T *src = static_cast<const T *>(state_buffer(M, state));
   T *dst = static_cast<T *>(state < 2 ? M.pop[state ^ 1] : M.pop[0]);
   T fx = static_cast<const T *>(M.fx_tab)[y];
@@ -394,7 +395,7 @@ __device__ __forceinline__ void step_cell(const Member &M, int state, int x, int
     else
       collide_f64(f, M.omega, fx, fy, M.alpha, M.collision, M.tau, M.Cs);
   } else if constexpr (sizeof(T) == 8) {
-    if (!M.fixed.step || !collide_fixed(f, M.fixed, fx, fy)) {
+    if (!fixed->step || !collide_fixed(f, *fixed, fx, fy)) {
       double g[kQ];  // read again: the fixed-point form keeps no copy
 #pragma unroll
       for (int l = 0; l < kQ; ++l) {
@@ -432,12 +433,12 @@ __device__ __forceinline__ void step_cell(const Member &M, int state, int x, int
 // without one the FP64 form is compiled in line.
 template <typename T, int NT, int MB, bool FIXED = false>
 __global__ void __launch_bounds__(NT, MB) k_step_scalar(const Member *__restrict__ members, int member, int state,
-                              double *rec) {
+                              double *rec, const FixedBgk *__restrict__ fixed) {
   const Member &M = members[member];
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   if (x >= M.nx || y >= M.ny) return;
-  step_cell<T, false, FIXED>(M, state, x, y, rec);
+  step_cell<T, false, FIXED>(M, state, x, y, rec, FIXED ? fixed + member : nullptr);
 }
 
 // ---------------------------------------------------------------------------
@@ -506,12 +507,13 @@ __global__ void __launch_bounds__(kPersistThreads)
 // partial wave per member.
 template <typename T, int NT, int MB, bool FIXED = false>
 __global__ void __launch_bounds__(NT, MB) k_step_scalar_multi(const Member *__restrict__ members, InitList list,
-                                    int state) {
-  const Member &M = members[list.m[blockIdx.z]];
+                                    int state, const FixedBgk *__restrict__ fixed) {
+  const int member = list.m[blockIdx.z];
+  const Member &M = members[member];
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   if (x >= M.nx || y >= M.ny) return;
-  step_cell<T, false, FIXED>(M, state, x, y);
+  step_cell<T, false, FIXED>(M, state, x, y, nullptr, FIXED ? fixed + member : nullptr);
 }
 
 static dim3 grid2d(int nx, int ny, dim3 b) {
@@ -582,8 +584,8 @@ cudaError_t launch_step_scalar_persistent(int precision, const Member *d_members
 }
 
 cudaError_t launch_step_scalar_batch(int precision, const Member *d_members, const int *members,
-                                     int n, int nx_max, int ny_max, int state, bool fixed,
-                                     cudaStream_t s) {
+                                     int n, int nx_max, int ny_max, int state,
+                                     const FixedBgk *fixed, cudaStream_t s) {
   const dim3 b = (long long)nx_max * ny_max < (1LL << 15) ? dim3(32, 2) : dim3(64, 4);
   for (int i0 = 0; i0 < n; i0 += InitList::kMax) {
     InitList list;
@@ -592,19 +594,19 @@ cudaError_t launch_step_scalar_batch(int precision, const Member *d_members, con
     dim3 g = grid2d(nx_max, ny_max, b);
     g.z = list.n;
     if (precision == 32)
-      k_step_scalar_multi<float, 256, 4><<<g, b, 0, s>>>(d_members, list, state);
+      k_step_scalar_multi<float, 256, 4><<<g, b, 0, s>>>(d_members, list, state, fixed);
     else if (b.x == 32)
       (fixed ? k_step_scalar_multi<double, 64, 1, true> : k_step_scalar_multi<double, 64, 1>)<<<g, b, 0, s>>>
-          (d_members, list, state);
+          (d_members, list, state, fixed);
     else
       (fixed ? k_step_scalar_multi<double, 256, 3, true> : k_step_scalar_multi<double, 256, 1>)<<<g, b, 0, s>>>
-          (d_members, list, state);
+          (d_members, list, state, fixed);
   }
   return cudaGetLastError();
 }
 
 cudaError_t launch_step_scalar(int precision, const Member *d_members, int member, int nx,
-                               int ny, int state, bool fixed, cudaStream_t s, double *rec) {
+                               int ny, int state, const FixedBgk *fixed, cudaStream_t s, double *rec) {
   // one thread per cell; grids below 2^17 cells get 64-thread CTAs, so that
   // their FP64 arithmetic (slow on this part) spreads evenly over the SMs
   // (256^2 FP64: 16.9 against 18.2 us per step with 256-thread CTAs in 1.7
@@ -612,13 +614,13 @@ cudaError_t launch_step_scalar(int precision, const Member *d_members, int membe
   const bool small = (long long)nx * ny < (1LL << 17);
   const dim3 b = small ? dim3(32, 2) : dim3(64, 4), g = grid2d(nx, ny, b);
   if (precision == 32)
-    k_step_scalar<float, 256, 4><<<g, b, 0, s>>>(d_members, member, state, rec);
+    k_step_scalar<float, 256, 4><<<g, b, 0, s>>>(d_members, member, state, rec, nullptr);
   else if (small)
     (fixed ? k_step_scalar<double, 64, 1, true> : k_step_scalar<double, 64, 1>)<<<g, b, 0, s>>>
-          (d_members, member, state, rec);
+          (d_members, member, state, rec, fixed);
   else
     (fixed ? k_step_scalar<double, 256, 3, true> : k_step_scalar<double, 256, 1>)<<<g, b, 0, s>>>
-          (d_members, member, state, rec);
+          (d_members, member, state, rec, fixed);
   return cudaGetLastError();
 }
 
