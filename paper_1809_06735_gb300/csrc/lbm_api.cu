@@ -1380,8 +1380,15 @@ int balance_members(lbm_handle *h, const int *members, int nm, const int *L, int
     J.max_boxes = maxb[i];
     J.qblocks = lbm::diag_query_blocks(hm.nx, hm.ny, maxb[i], origins != nullptr, batch_jobs, J.nL,
                                        h->diag_precision == 64);
-    J.qwhole = lbm::diag_whole_blocks(hm.nx * hm.ny, batch_jobs);
-    for (int q : where[i]) J.any_whole |= !origins && lbm::diag_whole_box(L[q], hm.nx, hm.ny, h->diag_precision == 64);
+    if (!origins) {
+      for (int q : where[i])
+        (lbm::diag_whole_box(L[q], hm.nx, hm.ny, h->diag_precision == 64) ? J.any_whole : J.planar) = 1;
+      J.qwhole = lbm::diag_whole_blocks(hm.nx * hm.ny, batch_jobs);
+      if (!J.planar) {  // only such sizes: k_query over records
+        J.qblocks = J.qwhole;
+        J.any_whole = 0;
+      }
+    }
     J.force_kind = hm.force_kind;
     if (hm.collision != 0) {  // local viscosity recorded with the snapshot at n
       const size_t N = (size_t)hm.nx * hm.ny;

@@ -96,8 +96,8 @@ __host__ __device__ inline size_t sat_stride(int nx, int ny) {
   return (size_t)(nx + 1) * (size_t)(ny + 1);
 }
 
-// For every periodic origin at once (no origin list) the tables are planar
-// instead: P_f(x, y) at f planar_stride + y planar_pitch + 3 + x, so that
+// For every periodic origin at once (no origin list, DiagJob::planar) the tables
+// are planar instead: P_f(x, y) at f planar_stride + y planar_pitch + 3 + x, so that
 // neighbouring origins read neighbouring words, and the four prefixes that a
 // lane of the table builder holds (x = 4 i + 1 on) start on a 32-byte boundary.
 __host__ __device__ inline size_t planar_pitch(int nx) { return ((size_t)nx + 7) / 4 * 4; }
@@ -1313,7 +1313,7 @@ __global__ void __launch_bounds__(NF * 32) k_sat_tile(const DiagJob *__restrict_
   const DiagJob &J = jobs[blockIdx.z];
   const int nx = J.nx, ny = J.ny, ns = (nx + kStrip - 1) / kStrip;
   const int ya = rb * rb_rows, yb = ya + rb_rows < ny ? ya + rb_rows : ny;
-  if (s >= ns || ya >= ny) return;  // whole CTA
+  if (s >= ns || ya >= ny || (J.planar != 0) != PLANAR) return;  // whole CTA
   const int x0 = s * kStrip, x = x0 + 4 * lane;
   const int nw = (nx - x0 < kStrip ? nx - x0 : kStrip) * NF;  // record words per row
   const size_t N = (size_t)nx * ny, rs = (size_t)nx + 1;
@@ -1449,7 +1449,7 @@ __device__ __forceinline__ MT delta_of(MT lhs, MT sum, MT mx) {
 }
 
 // One CTA per job, one thread per (size, field); constants at [size][kNT].
-__global__ void k_query_consts(const DiagJob *__restrict__ jobs, int nF, int planar) {
+__global__ void k_query_consts(const DiagJob *__restrict__ jobs, int nF) {
   const DiagJob &J = jobs[blockIdx.x];
   const int t = threadIdx.x;
   const int iL = t / kNT, k = t % kNT;
@@ -1457,7 +1457,7 @@ __global__ void k_query_consts(const DiagJob *__restrict__ jobs, int nF, int pla
   const int nx = J.nx, ny = J.ny;
   const size_t N = (size_t)nx * ny;
   const double area = (double)J.meta[8 * iL] * (double)J.meta[8 * iL];
-  const size_t last = planar ? (size_t)k * planar_stride(nx, ny) + ny * planar_pitch(nx) + 3 + nx
+  const size_t last = J.planar ? (size_t)k * planar_stride(nx, ny) + ny * planar_pitch(nx) + 3 + nx
                              : (sat_stride(nx, ny) - 1) * nF + k;
   const long long total = sat_base(J.base, N)[last];
   const double inv = J.part[inv_scale(k)];
@@ -1550,19 +1550,21 @@ __device__ void block_sum_store_pairs(MT (&v)[NQ], double *out0, double *out1) {
 // d_k, d_k^2 and of the error's (or Ma_V's) deviation and its square; with
 // EXT also a CTA histogram in shared memory, added to the global one with
 // integer atomics (order-free, so deterministic).
-// planar: every origin of the whole_grid_box sizes, from planar tables (other
-// sizes are k_query_all's).
-template <typename MT, bool PER_BOX, bool EXT>
+// PLANAR: the jobs with planar tables, every origin of their whole_grid_box
+// sizes (the other sizes are k_query_all's); else the jobs with record tables,
+// listed origins or every one (small FP64 grids, whose corners are then 48 bytes
+// in one place: read a word at a time from planar tables 64^2 took 10 us more).
+template <typename MT, bool PER_BOX, bool EXT, bool PLANAR>
 __global__ void __launch_bounds__(256, 3) k_query(const DiagJob *__restrict__ jobs, int nF,
                                                const int *__restrict__ origins,
-                                               double *per_box, DiagDist ext, int planar) {
+                                               double *per_box, DiagDist ext) {
   constexpr int NZ = EXT ? 2 : 1;
   const DiagJob &J = jobs[blockIdx.z / NZ];
   const bool mpart = EXT && blockIdx.z % NZ == 1;
   const int iL = blockIdx.y;
-  const int qb = planar ? J.qwhole : J.qblocks;
-  if (iL >= J.nL || (int)blockIdx.x >= qb) return;
-  if (planar && !whole_grid_box(J.meta[8 * iL], J.nx, J.ny, sizeof(MT) == 8)) return;
+  const int qb = PLANAR ? J.qwhole : J.qblocks;
+  if (iL >= J.nL || (int)blockIdx.x >= qb || (J.planar != 0) != PLANAR) return;
+  if (PLANAR && !whole_grid_box(J.meta[8 * iL], J.nx, J.ny, sizeof(MT) == 8)) return;
   const int grp = mpart ? 2 : (int)(threadIdx.x & 1), k0 = 6 * grp;
   const int slot = mpart ? (int)threadIdx.x : (int)(threadIdx.x >> 1);
   const int per_pass = mpart ? 256 : 128;
@@ -1600,26 +1602,39 @@ __global__ void __launch_bounds__(256, 3) k_query(const DiagJob *__restrict__ jo
   const int stride = qb * per_pass;
   int b = blockIdx.x * per_pass + slot;
   auto origin = [&](int i, int &x, int &y) {
-    if (planar) {
-      x = i % nx;
-      y = i / nx;
-    } else {
+    if (!PLANAR && ooff >= 0) {
       x = origins[2 * (ooff + i)];
       y = origins[2 * (ooff + i) + 1];
+    } else {
+      x = i % nx;
+      y = i / nx;
     }
   };
   int x0 = 0, y0 = 0;
   if (b < nb) origin(b, x0, y0);
+  // all periodic origins in row-major order: the next origin is this one
+  // advanced by the stride (no division per box)
+  const bool every = PLANAR || ooff < 0;
+  const int sdx = every ? stride % nx : 0, sdy = every ? stride / nx : 0;
   for (; b < nb; b += stride) {
     int xn = 0, yn = 0;  // the next box's origin, loaded ahead
-    if (b + stride < nb) origin(b + stride, xn, yn);
+    if (every) {
+      xn = x0 + sdx;
+      yn = y0 + sdy;
+      if (xn >= nx) {
+        xn -= nx;
+        ++yn;
+      }
+    } else if (b + stride < nb) {
+      origin(b + stride, xn, yn);
+    }
     const bool inside = x0 + L <= nx && y0 + L <= ny;
     MT lhs = 0, sum = 0, mx = 0;
     double *o = PER_BOX ? per_box + ((size_t)meta[8 * iL + 3] + b) * 15 : nullptr;
     // a non-wrapping box of a 12-field table: the six values of a corner are
     // 48 bytes at a 16-byte boundary, three vector loads per corner
     unsigned long long vs[6];
-    const bool vec = nF == 12 && nfield == 6 && !planar;
+    const bool vec = nF == 12 && nfield == 6 && !PLANAR;
     if (vec && !inside) {
       // a box across the periodic edge: the prefix sum extended periodically
       // is a signed sum of at most 3 x 3 table corners, columns
@@ -1671,7 +1686,7 @@ __global__ void __launch_bounds__(256, 3) k_query(const DiagJob *__restrict__ jo
       unsigned long long bs;
       if (vec) {
         bs = vs[j];
-      } else if (planar) {
+      } else if (PLANAR) {
         const long long *Sp = sat_base(J.base, N) + (size_t)(k0 + j) * planar_stride(nx, ny);
         bs = Pplane(Sp, nx, ny, x0 + L, y0 + L) - Pplane(Sp, nx, ny, x0, y0 + L) -
              Pplane(Sp, nx, ny, x0 + L, y0) + Pplane(Sp, nx, ny, x0, y0);
@@ -1929,7 +1944,7 @@ __global__ void __launch_bounds__(256, 2)
   constexpr int NG = EXT ? 3 : 2;
   const DiagJob &J = jobs[blockIdx.z / NG];
   const int grp = blockIdx.z % NG, iL = blockIdx.x, blk = blockIdx.y, qb = J.qblocks;
-  if (iL >= J.nL || blk >= qb || whole_grid_box(J.meta[8 * iL], J.nx, J.ny, sizeof(MT) == 8)) return;
+  if (iL >= J.nL || blk >= qb || !J.planar || whole_grid_box(J.meta[8 * iL], J.nx, J.ny, sizeof(MT) == 8)) return;
   __shared__ MT sedge[EXT ? kDiagMaxEdges : 1];
   __shared__ unsigned shist[EXT ? kDiagMaxEdges + 1 : 1];
   int ne = 0;
@@ -1969,13 +1984,13 @@ __global__ void __launch_bounds__(256, 2)
 // and with `mach` those of Ma_V.  Grid (sizes, jobs), 384 threads: 8 per
 // (group, slot) sum interleaved block partials in a fixed order.
 template <typename MT>
-__global__ void k_stats_final(const DiagJob *__restrict__ jobs, double *stats, double *mach,
-                              int planar) {
+__global__ void k_stats_final(const DiagJob *__restrict__ jobs, double *stats, double *mach) {
   const DiagJob &J = jobs[blockIdx.y];
   const int iL = blockIdx.x;
   if (iL >= J.nL) return;
-  const int nblocks =
-      planar && whole_grid_box(J.meta[8 * iL], J.nx, J.ny, sizeof(MT) == 8) ? J.qwhole : J.qblocks;
+  const int nblocks = J.planar && whole_grid_box(J.meta[8 * iL], J.nx, J.ny, sizeof(MT) == 8)
+                          ? J.qwhole
+                          : J.qblocks;
   const double *partials = J.part + kPartQuery;
   const QConst *consts = reinterpret_cast<const QConst *>(J.part + kPartConsts);
   const int q = threadIdx.x >> 3, j = threadIdx.x & 7;  // q = grp * 14 + slot
@@ -2056,9 +2071,8 @@ template <typename T, typename MT>
 cudaError_t balance_launches(const DiagJob *jobs_host, const DiagJob *jobs, int G, bool pairs,
                              const int *origins, double *stats, double *per_box,
                              const DiagDist *dist, cudaStream_t s) {
-  const bool planar = origins == nullptr;  // every periodic origin
   int nx = 1, ny = 1, nL = 1, qblocks = 1, qwhole = 1;
-  bool any_whole = false;
+  bool any_whole = false, any_planar = false, any_records = false;
   for (int j = 0; j < G; ++j) {
     nx = std::max(nx, jobs_host[j].nx);
     ny = std::max(ny, jobs_host[j].ny);
@@ -2066,6 +2080,7 @@ cudaError_t balance_launches(const DiagJob *jobs_host, const DiagJob *jobs, int 
     qblocks = std::max(qblocks, jobs_host[j].qblocks);
     qwhole = std::max(qwhole, jobs_host[j].qwhole);
     any_whole |= jobs_host[j].any_whole != 0;
+    (jobs_host[j].planar ? any_planar : any_records) = true;
   }
   const int nF = dist ? kNT : 12;  // |u|^2 gets a table only for Ma_V
   const dim3 cb(32, 8), cg((nx + 31) / 32, (ny + 7) / 8, G);
@@ -2118,19 +2133,21 @@ cudaError_t balance_launches(const DiagJob *jobs_host, const DiagJob *jobs, int 
       k_col_sums<T, 12><<<dim3(ns, nrb, G), 12 * 32, 0, s>>>(jobs, rb_rows);
   }
   const dim3 sg(ns, nrb, G);
-  if (planar) {
+  if (any_planar) {
     if (nF == kNT)
       k_sat_tile<T, kNT, true><<<sg, kNT * 32, 0, s>>>(jobs, rb_rows);
     else
       k_sat_tile<T, 12, true><<<sg, 12 * 32, 0, s>>>(jobs, rb_rows);
-  } else if (nF == kNT) {
-    k_sat_tile<T, kNT, false><<<sg, kNT * 32, 0, s>>>(jobs, rb_rows);
-  } else {
-    k_sat_tile<T, 12, false><<<sg, 12 * 32, 0, s>>>(jobs, rb_rows);
   }
-  k_query_consts<<<G, kDiagMaxL * kNT, 0, s>>>(jobs, nF, planar);
+  if (any_records) {
+    if (nF == kNT)
+      k_sat_tile<T, kNT, false><<<sg, kNT * 32, 0, s>>>(jobs, rb_rows);
+    else
+      k_sat_tile<T, 12, false><<<sg, 12 * 32, 0, s>>>(jobs, rb_rows);
+  }
+  k_query_consts<<<G, kDiagMaxL * kNT, 0, s>>>(jobs, nF);
   const DiagDist none{};
-  if (planar) {
+  if (any_planar) {
     const dim3 qg(nL, qblocks, (dist ? 3 : 2) * G);
     if (dist)
       k_query_all<MT, false, true><<<qg, 256, 0, s>>>(jobs, nullptr, *dist);
@@ -2139,17 +2156,26 @@ cudaError_t balance_launches(const DiagJob *jobs_host, const DiagJob *jobs, int 
     else
       k_query_all<MT, false, false><<<qg, 256, 0, s>>>(jobs, nullptr, none);
   }
-  if (!planar || any_whole) {
-    const dim3 qg(planar ? qwhole : qblocks, nL, (dist ? 2 : 1) * G);
+  const int nz = (dist ? 2 : 1) * G;
+  if (any_whole) {
+    const dim3 qg(qwhole, nL, nz);
     if (dist)
-      k_query<MT, false, true><<<qg, 256, 0, s>>>(jobs, nF, origins, nullptr, *dist, planar);
+      k_query<MT, false, true, true><<<qg, 256, 0, s>>>(jobs, nF, nullptr, nullptr, *dist);
     else if (per_box)
-      k_query<MT, true, false><<<qg, 256, 0, s>>>(jobs, nF, origins, per_box, none, planar);
+      k_query<MT, true, false, true><<<qg, 256, 0, s>>>(jobs, nF, nullptr, per_box, none);
     else
-      k_query<MT, false, false><<<qg, 256, 0, s>>>(jobs, nF, origins, nullptr, none, planar);
+      k_query<MT, false, false, true><<<qg, 256, 0, s>>>(jobs, nF, nullptr, nullptr, none);
   }
-  k_stats_final<MT><<<dim3(nL, G), 384, 0, s>>>(jobs, stats, dist ? dist->mach : nullptr,
-                                                  planar);
+  if (any_records) {
+    const dim3 qg(qblocks, nL, nz);
+    if (dist)
+      k_query<MT, false, true, false><<<qg, 256, 0, s>>>(jobs, nF, origins, nullptr, *dist);
+    else if (per_box)
+      k_query<MT, true, false, false><<<qg, 256, 0, s>>>(jobs, nF, origins, per_box, none);
+    else
+      k_query<MT, false, false, false><<<qg, 256, 0, s>>>(jobs, nF, origins, nullptr, none);
+  }
+  k_stats_final<MT><<<dim3(nL, G), 384, 0, s>>>(jobs, stats, dist ? dist->mach : nullptr);
   return cudaGetLastError();
 }
 

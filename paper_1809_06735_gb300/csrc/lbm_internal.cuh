@@ -363,8 +363,10 @@ struct DiagJob {
   const double *nu_cell_d;     // or FP64 storage), else both NULL
   int qblocks;                 // query CTAs per (size, balance):
                                // diag_query_blocks(...)
-  int qwhole, any_whole;       // every origin: the CTAs of the sizes of nearly the
-                               // whole grid, and whether there are any
+  int planar;                  // tables of one plane per field, every origin, else
+                               // records
+  int qwhole, any_whole;       // planar: the CTAs of the diag_whole_box sizes, and
+                               // whether there are any
 };
 // Query CTAs for a job: a fixed function of its own box count, so that the
 // statistics do not depend on which members share a batch.
