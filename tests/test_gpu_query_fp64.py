@@ -1,7 +1,9 @@
-"""The FP64 query over every periodic origin in batches in which members with
-planar tables (from 2^15 cells up) and members with record tables meet: the means
+"""The FP64 query over every periodic origin of grids from 2^15 cells up (planar
+tables, integer sums of deviations), which smaller FP64 grids do not take:
+every box against the same origins given as a list (record tables), the means
 and standard deviations against those of the boxes, the distributions against
-each member's own.
+the list's counts, and batches in which members with planar tables and members
+with record tables meet.
 
 Bars, from the arithmetic: a term's box is the same integer on both paths, so it
 differs by the rounding of mean + deviation (1e-15 of the largest box); its
@@ -18,6 +20,9 @@ import lbm_inputs as li
 
 pytestmark = pytest.mark.gpu
 
+GRIDS = [(257, 131), (131, 257), (400, 90), (1025, 33), (33, 1025), (182, 181), (184, 180)]
+
+
 @pytest.fixture(scope="module")
 def P():
     import paper_1809_06735_gb300 as P
@@ -32,6 +37,16 @@ def _lattice(P, grids, prec=64, terms=0):
         lat.init_fields(m, 1.0 + f[0], f[1], f[2])
     lat.step(4)
     return lat
+
+
+def _every(nx, ny):
+    y, x = np.mgrid[0:ny, 0:nx]
+    return np.stack([x.ravel(), y.ravel()], 1).astype(np.int32)
+
+
+def _sizes(nx, ny):
+    n = min(nx, ny)
+    return sorted({1, 2, n // 3, n // 2 + 1, n - 1, n})
 
 
 def _moments(b):
@@ -54,6 +69,38 @@ def _check_stats(stats, boxes, nL):
             ms = mean ** 2 + std ** 2
             assert np.all(np.abs(stats[i, :2, 0] - mean) <= 1e-13 * np.sqrt(ms)), i
             assert np.all(np.abs(stats[i, :2, 1] ** 2 - std ** 2) <= 1e-13 * ms), i
+
+
+@pytest.mark.parametrize("prec,terms", [(64, 0), (32, 64)])
+@pytest.mark.parametrize("nx,ny", GRIDS)
+def test_boxes_and_statistics(P, nx, ny, prec, terms):
+    lat = _lattice(P, [(nx, ny)], prec, terms)
+    Ls = _sizes(nx, ny)
+    sa, ba = lat.subvolume_balance(0, Ls, per_box=True)
+    _, bl = lat.subvolume_balance(0, Ls, origins=_every(nx, ny), per_box=True)
+    ba, bl = ba.cpu().numpy(), bl.cpu().numpy()
+    scale = np.max(np.abs(bl[:, 2:]), axis=0)
+    assert np.all(np.abs(ba[:, 2:] - bl[:, 2:]) <= 1e-15 * scale + 4e-16 * np.abs(bl[:, 2:]))
+    _check_stats(sa, ba, len(Ls))
+    s = lat.subvolume_balance(0, Ls)  # without the boxes' output
+    assert np.array_equal(s, sa, equal_nan=True)
+    lat.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(257, 131), (400, 90), (33, 1025)])
+def test_distributions(P, nx, ny):
+    lat = _lattice(P, [(nx, ny)])
+    Ls = _sizes(nx, ny)
+    de, me = np.linspace(0, 0.5, 33), np.linspace(0, 0.2, 17)
+    a = lat.subvolume_distributions([0], Ls, de, me)
+    b = lat.subvolume_distributions([0], Ls, de, me, origins=_every(nx, ny))
+    assert np.array_equal(a["delta_hist"], b["delta_hist"])
+    assert np.array_equal(a["mach_hist"], b["mach_hist"])
+    assert np.all(a["mach_hist"].sum(-1) == nx * ny)
+    np.testing.assert_allclose(a["mach"][..., 0], b["mach"][..., 0], rtol=1e-13)
+    _, boxes = lat.subvolume_balance(0, Ls, per_box=True)
+    _check_stats(a["stats"][0], boxes.cpu().numpy(), len(Ls))
+    lat.close()
 
 
 @pytest.mark.parametrize("dist", [False, True])
