@@ -30,6 +30,8 @@
 // 24 B), forced 8192^2 755 / 444 / 351 / 383, 15 forced members of 256^2 ..
 // 1024^2 79 / 52 / 45 / 50 (strips; whole rows 55 at T = 3: the barrier of 8
 // warps costs more than the halo lanes).
+#include <algorithm>
+
 #include "lbm_collide.cuh"
 
 namespace lbm {
@@ -302,6 +304,7 @@ static Split split_columns(int nx, int gmax) {
   return Split{1, ns, ((nx + ns - 1) / ns + 3) / 4 * 4};
 }
 static int block_rows(int ny, int rows) {
+  rows = std::min(rows, ny);  // any larger asks for whole columns
   const int nb = (ny + rows - 1) / rows;
   return (ny + nb - 1) / nb;
 }
