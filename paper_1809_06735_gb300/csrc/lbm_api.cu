@@ -853,10 +853,13 @@ int lbm_create(const lbm_config *cfg, void *workspace, size_t bytes, lbm_handle 
       B.om9h = (long long)(((unsigned __int128)B.om * 4 + 4) / 9);
       B.alpha = B.ok ? std::llrint(std::ldexp(c.alpha, 64)) : 0;
       B.forced = c.force_kind != 0 || c.alpha != 0.0;
-      // Small grids keep the FP64 form: the symmetric flows they are run with
-      // (Taylor-Green) amplify a change of the step's rounding until the
-      // balancing errors move by 1e-9 (64^2, 100 steps), more than results
-      // may.  The persistent kernel takes the same sizes.
+      // Grids below kPersistMaxCells keep the FP64 form, so that what such runs
+      // give stays as it was.  Not for accuracy: a Taylor-Green flow's balancing
+      // errors, which show the rounding of the state most, are nearer to those
+      // of extended precision in fixed point (100 steps of 192^2: 1e-9 against 6e-9
+      // to 8e-9, 256^2: 4e-9 against 1.3e-8 to 1.7e-8), but they are others, by up
+      // to 1e-9 at 64^2.  It costs such grids 1.4 times the step (64^2: 2.6
+      // against 5.3 us with graph replay).
       B.step = es == 8 && B.ok && (long long)c.nx * c.ny >= lbm::kPersistMaxCells;
     }
     h->hm.push_back(M);
