@@ -21,8 +21,12 @@
 #include <vector>
 
 #include "../../include/lbm3d.h"
+#include "lbm_num.cuh"
 
 namespace {
+
+using lbm::abs_max;
+using lbm::i64_to_f64;
 
 // Velocity sets: D3Q27 = rest, 6 axis, 12 edge, 8 corner velocities in the
 // order of include/lbm3d.h; D3Q19 is its first 19 entries.  Weights by
@@ -804,20 +808,13 @@ __global__ void __launch_bounds__(128) k3_scan_z(Diag3 J, long long *tab) {
   }
 }
 
-// max(m, |v|) for m >= 0, NaN ignored; FP64 by the bits, off the FP64 pipe.
-__device__ __forceinline__ float abs_max3(float m, float v) { return fmax(m, fabs(v)); }
-__device__ __forceinline__ double abs_max3(double m, double v) {
-  const long long b = __double_as_longlong(v) & 0x7fffffffffffffffll, a = __double_as_longlong(m);
-  return b > a && b <= 0x7ff0000000000000ll ? __longlong_as_double(b) : m;
-}
-
 template <int NRHS, typename MT>
 __device__ __forceinline__ MT delta3(const MT *v) {
   MT sum = MT(0), mx = MT(0);
 #pragma unroll
   for (int i = 1; i <= NRHS; ++i) {
     sum += v[i];
-    mx = abs_max3(mx, v[i]);
+    mx = abs_max(mx, v[i]);
   }
   const MT num = fabs(sum - v[0]);
   if (mx == MT(0)) return num == MT(0) ? MT(0) : MT(INFINITY);
@@ -831,14 +828,7 @@ template <typename MT>
 __device__ __forceinline__ MT i64_to(long long v);
 template <>
 __device__ __forceinline__ double i64_to<double>(long long v) {
-  // to nearest (ties away from zero) by integer instructions, off the FP64 pipe
-  const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
-  const int n = __clzll((long long)a);
-  const unsigned long long x = a << (n & 63), r = x + 0x400ull;
-  const unsigned carry = r < x;
-  const unsigned e = n == 64 ? 0u : (unsigned)(1023 + 63 - 1 - n) << 20;
-  const unsigned hi = (unsigned)(r >> 43) + e + (carry << 21);
-  return __hiloint2double((int)(hi | (v < 0 ? 0x80000000u : 0u)), (int)(unsigned)(r >> 11));
+  return i64_to_f64(v);
 }
 template <>
 __device__ __forceinline__ float i64_to<float>(long long v) {

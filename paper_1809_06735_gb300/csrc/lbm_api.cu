@@ -269,7 +269,6 @@ struct lbm_handle {
   lbm::LaunchCfg lc{8, 1, 0, 0, 8};
   MultiWarp *d_multi = nullptr;
   int multi_T = 1;      // steps per launch (1: the single-step kernel only)
-  int multi_rows = 0;   // rows of a block
   int multi_ctas = 0;
   bool multi_forced = false;  // some member has a force or drag
   int graph_k = 0;
@@ -339,7 +338,6 @@ int build_multi(lbm_handle *h, int T, int rows, int gmax) {
                      cudaMemcpyHostToDevice, h->stream));
   CK(cudaStreamSynchronize(h->stream));
   h->multi_T = T;
-  h->multi_rows = rows;
   h->multi_ctas = (int)(tab.size() / lbm::kMultiWarps);
   return LBM_OK;
 }

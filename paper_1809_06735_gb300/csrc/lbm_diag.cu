@@ -40,6 +40,7 @@
 #include <vector>
 
 #include "lbm_internal.cuh"
+#include "lbm_num.cuh"
 
 namespace lbm {
 
@@ -1433,14 +1434,6 @@ __device__ __forceinline__ unsigned long long Pplane(const long long *S, int nx,
   return v;
 }
 
-// max(m, |v|) for m >= 0; NaN in v is ignored, as fmax does.  FP64 by the bits
-// (non-negative doubles order like their bits), off the FP64 pipe.
-__device__ __forceinline__ float abs_max(float m, float v) { return fmax(m, fabs(v)); }
-__device__ __forceinline__ double abs_max(double m, double v) {
-  const long long b = __double_as_longlong(v) & 0x7fffffffffffffffll, a = __double_as_longlong(m);
-  return b > a && b <= 0x7ff0000000000000ll ? __longlong_as_double(b) : m;
-}
-
 template <typename MT>
 __device__ __forceinline__ MT delta_of(MT lhs, MT sum, MT mx) {
   const MT num = fabs(sum - lhs);
@@ -1800,19 +1793,6 @@ __host__ __device__ inline AllGrid all_grid(int nx, int ny, int nL, bool f64) {
   if (parts > kMaxQueryBlocks / g.nxb) parts = kMaxQueryBlocks / g.nxb;
   g.parts = parts < 1 ? 1 : parts;
   return g;
-}
-
-// 64-bit integer to double, to nearest (ties away from zero), by integer
-// instructions: the conversion instruction runs on the narrow FP64 pipe.
-__device__ __forceinline__ double i64_to_f64(long long v) {
-  const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
-  const int n = __clzll((long long)a);
-  unsigned long long x = a << (n & 63);
-  const unsigned long long r = x + 0x400ull;
-  const unsigned carry = r < x;  // all ones rounded up: the next power of two
-  const unsigned e = n == 64 ? 0u : (unsigned)(1023 + 63 - 1 - n) << 20;
-  const unsigned hi = (unsigned)(r >> 43) + e + (carry << 21);
-  return __hiloint2double((int)(hi | (v < 0 ? 0x80000000u : 0u)), (int)(unsigned)(r >> 11));
 }
 
 // The statistics of one column's boxes of NFLD fields from plane k0 on.

@@ -234,7 +234,7 @@ struct LaunchCfg {
 // rows, and its place w among the g warps of its group (consecutive warps of
 // one CTA).  member < 0: no work.
 struct MultiWarp {
-  int member, x0, xend, out0, out1, y0, rows, g, w, pad;
+  int member, x0, xend, out0, out1, y0, rows, g, w;
 };
 constexpr int kMultiWarps = 8;     // warps per CTA
 constexpr int kMultiMaxSteps = 4;  // steps per launch at most
@@ -368,8 +368,9 @@ struct DiagJob {
   int qwhole, any_whole;       // planar: the CTAs of the diag_whole_box sizes, and
                                // whether there are any
 };
-// Query CTAs for a job: a fixed function of its own box count, so that the
-// statistics do not depend on which members share a batch.
+// Query CTAs for a job.  Planar tables: a function of its grid and its number of
+// sizes.  Lists and record tables: of its boxes and of the number of jobs that the
+// scratch takes at once (so the last bits of a member's sums depend on that).
 int diag_query_blocks(int nx, int ny, int max_boxes, bool origin_list, int batch_jobs, int nL,
                       bool f64);
 int diag_whole_blocks(int boxes, int batch_jobs);
