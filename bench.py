@@ -100,9 +100,17 @@ def measured_peaks():
     return FALLBACK_HBM_GBS, "fallback"
 
 
+def sources_hash(names) -> str:
+    """Hash of the CUDA sources that a profiled figure is valid for."""
+    h = hashlib.sha256()
+    for name in names:
+        with open(os.path.join(ROOT, "paper_1809_06735_gb300", "csrc", name), "rb") as fh:
+            h.update(fh.read())
+    return h.hexdigest()[:16]
+
+
 def kernel_source_hash() -> str:
-    with open(os.path.join(ROOT, "paper_1809_06735_gb300", "csrc", "lbm_step.cu"), "rb") as fh:
-        return hashlib.sha256(fh.read()).hexdigest()[:16]
+    return sources_hash(("lbm_step.cu", "lbm_collide.cuh"))
 
 
 def profiled_traffic():
@@ -476,13 +484,7 @@ def collision_models_leg(P, stream, dev, peak):
                      "bound": "hbm"}
         if coll == 3:  # the entropic root keeps the issue slots busy: ALU-bound
             out[name].update({"bound": "alu", "hbm_frac": gbs / peak})
-            wi = issue_counts().get(out[name]["kernel"])
-            if wi is not None:
-                rate = wi * lu / secs
-                pk = issue_peak(dev.index or 0)
-                out[name].update({"warp_instr_per_lu": wi, "achieved": rate / 1e12,
-                                  "peak": pk / 1e12, "unit": "T warp instr/s",
-                                  "frac": rate / pk})
+            out[name].update(issue_roofline(out[name]["kernel"], lu / secs / 1e9, dev.index or 0))
         del lat
     return out
 
@@ -612,41 +614,17 @@ def alu_peaks(P, stream):
                    "CTAs per SM, CUDA events"}
 
 
-def fp64_instruction_counts():
-    """FP64 flops and FP64 instructions per lattice update of the FP64
-    kernels (dadd + dmul + 2 dfma, and dadd + dmul + dfma, ncu counters)
-    from the committed summary, valid only while the kernel sources are
-    unchanged."""
-    p = os.path.join(ROOT, "profiles", "fp64_flops_per_lu.json")
-    if not os.path.exists(p):
-        return {}
-    with open(p) as fh:
-        d = json.load(fh)
-    out = {}
-    for name, rec in d.get("kernels", {}).items():
-        src = os.path.join(ROOT, "paper_1809_06735_gb300", "csrc", rec["source"])
-        with open(src, "rb") as fh:
-            if hashlib.sha256(fh.read()).hexdigest()[:16] == rec.get("source_sha256_16"):
-                out[name] = (rec["fp64_flops_per_lu"], rec["fp64_instr_per_lu"])
-    return out
-
-
 def issue_counts():
     """Warp instructions per lattice update of the issue-bound kernels
     (sm__inst_executed.sum over the launch's cells, ncu) from the committed
-    summary, valid only while the kernel source is unchanged."""
-    p = os.path.join(ROOT, "profiles", "elbm_issue.json")
+    summary, valid only while the kernel's sources are unchanged."""
+    p = os.path.join(ROOT, "profiles", "issue_counts.json")
     if not os.path.exists(p):
         return {}
     with open(p) as fh:
         d = json.load(fh)
-    out = {}
-    for name, rec in d.get("kernels", {}).items():
-        src = os.path.join(ROOT, "paper_1809_06735_gb300", "csrc", rec["source"])
-        with open(src, "rb") as fh:
-            if hashlib.sha256(fh.read()).hexdigest()[:16] == rec.get("source_sha256_16"):
-                out[name] = rec["warp_instr_per_lu"]
-    return out
+    return {name: rec["warp_instr_per_lu"] for name, rec in d.get("kernels", {}).items()
+            if sources_hash(rec["sources"]) == rec.get("sources_sha256_16")}
 
 
 def issue_peak(dev_index=0):
@@ -662,25 +640,24 @@ def issue_peak(dev_index=0):
     return 4.0 * sms * mhz * 1e6
 
 
-def fp64_roofline(counts, glups, peaks):
-    """The FP64-pipe roofline of a kernel from its counted flops and
-    instructions per update: achieved flop rate against the measured FMA
-    rate, and the pipe's instruction rate against the FMA chains' (an add or
-    a multiply occupies the pipe like an FMA)."""
-    flops, instr = counts
-    tf = flops * glups / 1e3
-    return {"bound": "fp64", "fp64_flops_per_lu": flops, "fp64_instr_per_lu": instr,
-            "achieved": tf, "peak": peaks["fp64_tflops"], "unit": "TFLOP/s",
-            "frac": tf / peaks["fp64_tflops"],
-            "pipe_instr_frac": instr * glups * 1e9 / (peaks["fp64_tflops"] * 1e12 / 2)}
+def issue_roofline(kernel, glups, dev_index=0):
+    """The instruction-issue roofline of a kernel from its counted warp
+    instructions per update, or nothing where no valid count is on record."""
+    wi = issue_counts().get(kernel)
+    if wi is None:
+        return {}
+    rate, pk = wi * glups * 1e9, issue_peak(dev_index)
+    return {"bound": "alu", "warp_instr_per_lu": wi, "achieved": rate / 1e12, "peak": pk / 1e12,
+            "unit": "T warp instr/s", "frac": rate / pk}
 
 
-def fp64_plain_leg(P, stream, dev, peak_hbm, peaks, dev_fields=None):
+def fp64_plain_leg(P, stream, dev, peak_hbm):
     """The plain single-instance FP64 step (double buffer, general kernel)
     on one 4096^2 member (2 x 1.2 GB of populations: far beyond the L2, so
     the HBM figure means something), against both bounds: 144 algorithmic
-    bytes per update over the measured copy bandwidth, and the FP64 flops
-    per update (ncu counters) over the measured FP64 FMA rate."""
+    bytes per update over the measured copy bandwidth, and the warp
+    instructions per update (ncu counters) over the issue peak: the
+    collision runs in integer instructions."""
     import torch
     n = 4096
     lat = P.Lattice([P.Member(n, n, 0.52)], precision=64, graph_steps=10, stream=stream,
@@ -699,11 +676,11 @@ def fp64_plain_leg(P, stream, dev, peak_hbm, peaks, dev_fields=None):
     lat.close()
     glups = n * n / secs / 1e9
     gbs = BYTES_PER_LU_F64 * glups
-    counts = fp64_instruction_counts().get("k_step_scalar<double>")
     out = {"grid": [n, n], "glups": glups, "bytes_per_lu": BYTES_PER_LU_F64,
            "achieved_gbs": gbs, "hbm_frac": gbs / peak_hbm}
-    if counts is not None:
-        out["fp64_roofline"] = fp64_roofline(counts, glups, peaks)
+    roof = issue_roofline("k_step_scalar<double> (fixed point)", glups, dev.index or 0)
+    if roof:
+        out["issue_roofline"] = roof
     return out
 
 
@@ -798,7 +775,7 @@ def large_grid_leg(P, stream, dev, peak):
             "glups_with_diagnostic": n * n * D / (period_s + event_s) / 1e9}
 
 
-def adjoint_leg(P, stream, dev, peaks):
+def adjoint_leg(P, stream, dev):
     """The differentiation workload: 256^2, tau 0.55, Kolmogorov kf = 4
     (drag 1e-4), J = mean over n in [1000, 2000] of the L = 16 box average
     of the dissipation term, checkpoints every 100 steps; the forward pass
@@ -867,9 +844,9 @@ def adjoint_leg(P, stream, dev, peaks):
          "achieved_gbs": 216 * glups,
          "note": "256^2 FP64: 14 MB per step, L2-resident; one k_adjoint launch per step, "
                  "the gradient reduction (k_adjoint_final) once per 100-step sweep"}
-    counts = fp64_instruction_counts().get("k_adjoint")
-    if counts is not None:
-        k["fp64_roofline"] = fp64_roofline(counts, glups, peaks)
+    roof = issue_roofline("k_adjoint", glups, dev.index or 0)
+    if roof:
+        k["issue_roofline"] = roof
     out["adjoint_kernel"] = k
     return out
 
@@ -1073,7 +1050,8 @@ def case_adjoint(P, n=256, steps=6):
     acc = torch.zeros(2, dtype=torch.float64, device="cuda")
     lat.objective_steps(0, steps, 1e-3, (0, 0), 16, acc[0:1])  # forward objective levels
     f = lat.get_populations(0)
-    lam = torch.zeros_like(f)
+    # a dense adjoint, as after the steps that spread the objective's reach
+    lam = torch.randn(f.shape, generator=torch.Generator().manual_seed(0), dtype=f.dtype).to(f.device)
     out = torch.empty_like(f)
     for _ in range(steps):
         lat.adjoint_step(0, f, lam, out, 1e-3, (0, 0), 16, acc[0:1], acc[1:2])
@@ -1207,10 +1185,10 @@ def run_ours(args):
     fp64_glups = n * n / fp64_s / 1e9
     del lat64
     peaks_alu = alu_peaks(P, stream)
-    fp64_big = fp64_plain_leg(P, stream, dev, peak, peaks_alu)
+    fp64_big = fp64_plain_leg(P, stream, dev, peak)
     forced_sweep = forced_sweep_leg(P, stream, dev, peak)
     large_grid = large_grid_leg(P, stream, dev, peak)
-    adjoint = adjoint_leg(P, stream, dev, peaks_alu)
+    adjoint = adjoint_leg(P, stream, dev)
     paper_forcing = paper_forcing_leg(P, stream, dev, measured_peaks()[0])
     tau_trend = forced_tau_trend_leg(P, stream, dev)
     collisions = collision_models_leg(P, stream, dev, measured_peaks()[0])
