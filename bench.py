@@ -482,9 +482,9 @@ def collision_models_leg(P, stream, dev, peak):
         out[name] = {"glups": lu / secs / 1e9, "achieved_gbs": gbs, "frac": gbs / peak,
                      "kernel": step_kernel_name(lat) + (" (entropic)" if coll == 3 else " (extended)"),
                      "bound": "hbm"}
-        if coll == 3:  # the entropic root keeps the issue slots busy: ALU-bound
-            out[name].update({"bound": "alu", "hbm_frac": gbs / peak})
-            out[name].update(issue_roofline(out[name]["kernel"], lu / secs / 1e9, dev.index or 0))
+        roof = issue_roofline(out[name]["kernel"], lu / secs / 1e9, dev.index or 0)
+        if roof:
+            out[name]["issue_roofline"] = roof
         del lat
     return out
 
